@@ -60,6 +60,9 @@ STORAGE_TEXT = {
 
 STORAGE_NAMES = {0: "fp32", 1: "fp16", 2: "fp16_fit"}
 BYTES = {0: (BYTES_STEP, BYTES_KERNEL), 1: (BYTES_STEP_FP16, BYTES_KERNEL_FP16), 2: (BYTES_STEP_FIT, BYTES_KERNEL_FIT)}
+# inside a call of several steps advance_kernel goes from moment record to moment record: the 48-byte
+# moments and the phase entry read and written once, no populations
+BYTES_KERNEL["advance_kernel"] = 2 * (8 + BYTES_MOMENTS)
 # the fused step kernel (both passes in one launch) needs only the method's bytes
 for _s, (_b, _k) in BYTES.items():
     _k["step_kernel"] = _b
@@ -360,7 +363,7 @@ def measured_peaks():
 
 # The sources a kernel is compiled from, besides the shared headers: its translation unit, and
 # for the fused step kernel the host code that builds its item sequence.
-KERNEL_SOURCES = {"step_kernel": ("lbcm_step.cu", "lbcm_api.cu")}
+KERNEL_SOURCES = {"step_kernel": ("lbcm_step.cu", "lbcm_api.cu"), "advance_kernel": ("lbcm_advance.cu",)}
 
 
 def kernel_source_sha(kernel: str, src: str = None) -> str:

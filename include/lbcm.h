@@ -259,8 +259,11 @@ LB_API lb_status lb_load(lb_ctx *ctx, const void *buf, size_t nbytes);
 /* Index 0 is the boundary planes (one of two kernels, chosen by the plane size); 1 the step's
  * gather pass: moment_kernel with the paper's rates s3..s6 = 1 (phase field and collision
  * moments), phase_field_kernel otherwise; 2 the collision pass; 3 the fused step kernel, which
- * runs both passes in one launch (params.step_kernel = 1). */
-enum { LB_KERNEL_BOUNDARY = 0, LB_KERNEL_GATHER = 1, LB_KERNEL_COLLIDE = 2, LB_KERNEL_STEP = 3, LB_NKERNELS = 4,
+ * runs both passes in one launch (params.step_kernel = 1); 4 advance_kernel, which takes the
+ * place of a collision pass and the next gather pass inside an lb_step call of several steps
+ * (paper rates, FP32 and FP16 storage). */
+enum { LB_KERNEL_BOUNDARY = 0, LB_KERNEL_GATHER = 1, LB_KERNEL_COLLIDE = 2, LB_KERNEL_STEP = 3, LB_KERNEL_ADVANCE = 4,
+       LB_NKERNELS = 5,
        LB_KERNEL_PHASE_FIELD = LB_KERNEL_GATHER };
 LB_API lb_status lb_profile_enable(lb_ctx *ctx, int32_t capacity);
 LB_API lb_status lb_profile_read(lb_ctx *ctx, double *ms, int64_t *launches, int32_t n_kinds);

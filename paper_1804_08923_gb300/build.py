@@ -10,7 +10,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "liblbcm.so")
-SOURCES = ["lbcm_step.cu", "lbcm_adjoint.cu", "lbcm_fragments.cu", "lbcm_api.cu"]
+SOURCES = ["lbcm_step.cu", "lbcm_advance.cu", "lbcm_general.cu", "lbcm_adjoint.cu", "lbcm_fragments.cu", "lbcm_api.cu"]
+# the kernels that have to round alike (lbcm_collide.cuh) spell out their fused multiply-adds
+EXACT = ("lbcm_step.cu", "lbcm_advance.cu")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -47,6 +49,7 @@ def build(force: bool = False, verbose_ptxas: bool = False) -> str:
         obj = os.path.join(bdir, src.replace(".cu", ".o"))
         objs.append(obj)
         cmd = [nvcc(), "-c", os.path.join(CSRC, src), "-o", obj] + flags(verbose_ptxas)
+        cmd += ["-fmad=false"] if src in EXACT else []
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
     failed = []
     for cmd, p in procs:

@@ -90,6 +90,22 @@ __device__ __forceinline__ void cp_async8(unsigned smem, const void *gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// Coefficients of the inverse 1-D sweep: a value at c in {-1, 0, +1} from central moments
+// (m0, m1, m2) about u is G0[c] m0 + G1[c] m1 + G2[c] m2 with
+//   G0 = ((u^2 - u)/2, 1 - u^2, (u^2 + u)/2), G1 = (u - 1/2, -2u, u + 1/2), G2 = (1/2, -1, 1/2).
+struct InvAxis {
+    float g0[3], g1[3];
+    __device__ __forceinline__ explicit InvAxis(float u) {
+        const float u2 = u * u;
+        g0[0] = 0.5f * (u2 - u);
+        g0[1] = 1.0f - u2;
+        g0[2] = 0.5f * (u2 + u);
+        g1[0] = u - 0.5f;
+        g1[1] = -2.0f * u;
+        g1[2] = u + 0.5f;
+    }
+};
+
 // 1-D transpose of the inverse sweep: M_a = sum_c v_c G_a[c](u) for a = 0, 1, 2.
 __device__ __forceinline__ void sweep_inv_T(float &a0, float &a1, float &a2, const InvAxis &A) {
     const float v0 = a0, v1 = a1, v2 = a2;
@@ -256,8 +272,8 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     const float uF = ux * Fx + uy * Fy + uz * Fz;
     const float cs2 = oma * (9.0f / 19.0f);
     // Q: second central moment of f - f^e + F'/2 (Pi(f^e), Pi(F') in closed form)
-    float Qxx = mo.pxx - (rho * cs2 + rho * ux * ux + nu * (2.0f * ux * grx + ugr));
-    float Qyy = mo.pyy - (rho * cs2 + rho * uy * uy + nu * (2.0f * uy * gry + ugr));
+    float Qxx = (mo.pzz + mo.dxz) - (rho * cs2 + rho * ux * ux + nu * (2.0f * ux * grx + ugr));
+    float Qyy = (mo.pzz + mo.dyz) - (rho * cs2 + rho * uy * uy + nu * (2.0f * uy * gry + ugr));
     float Qzz = mo.pzz - (rho * cs2 + rho * uz * uz + nu * (2.0f * uz * grz + ugr));
     float Qxy = mo.pxy - (rho * ux * uy + nu * (ux * gry + uy * grx));
     float Qxz = mo.pxz - (rho * ux * uz + nu * (ux * grz + uz * grx));
@@ -573,7 +589,7 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g)
         adj_stencil_sums<W, false>(a, g, nb, z, lphi, lrho);
     float phv, S_;  // phi and rho_r/rho_r0 + rho_b/rho_b0 of this node
     if (g.mom) {
-        const float4 r0 = __ldg(g.mom + nb.n);  // (rho_r, rho_b, sf, jx)
+        const float4 r0 = __ldg(g.mom + nb.n);  // (rho_r, rho_b, phi, jx)
         phv = order_parameter(r0.x, r0.y, a.inv_rho_r0, a.inv_rho_b0);
         S_ = r0.x * a.inv_rho_r0 + r0.y * a.inv_rho_b0;
     } else {

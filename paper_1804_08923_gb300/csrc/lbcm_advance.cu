@@ -1,0 +1,312 @@
+// lbcm_advance.cu -- the steps between the first gather and the last collision of one lb_step call
+// with the paper's rates (arXiv:1804.08923, Section II, boundaries of Section IV.A).
+//
+// With s3 = s4 = s5 = s6 = 1 the collision depends on a node's 54 populations only through its 12
+// collision moments (lbcm_collide.cuh).  So inside one call the state between two steps is kept as
+// the moment record and the phase entry of the post-stream node (56 bytes with FP32 storage) and
+// advance_kernel takes one such state to the next: it rebuilds the populations that the collision
+// would have written (rounded as the storage rounds them), streams them through shared memory and
+// sums the next moments.  lb_step(n) is one gather pass, n - 1 advances and one collision pass,
+// with the same bits as n gather and n collision passes.
+//
+// A block owns a 32 x TY tile of columns and a run of planes and marches along z.  Per plane k:
+//   collide  each thread takes one node of the tile and its one-node halo in x and y, from the
+//            prefetched moments and a ring of phase planes in shared memory, and writes its 27
+//            population pairs to shared memory;
+//   gather   each thread of the tile reads the 27 pulls that come from plane k: c_z = -1 completes
+//            the node of plane k - 1, c_z = 0 is joined to plane k, c_z = +1 starts plane k + 1
+//            (z_class, join_classes, finish_moments; 20 registers hold the two open planes).
+// The halo is collided again by every block that needs it (1.2 times the nodes for TY = 14), which
+// costs arithmetic and no population traffic.
+#include <algorithm>
+#include <type_traits>
+
+#include "lbcm_collide.cuh"
+#include "lbcm_device.cuh"
+#include "lbcm_internal.h"
+#include "lbcm_node.cuh"
+
+namespace lbcm {
+
+template <int TY>
+struct AdvanceTile {
+    static constexpr int BX = 34, RX = 36, RY = TY + 4;    // row of collided nodes, ring of phase nodes
+    static constexpr int NB = BX * (TY + 2), NR = RX * RY;
+    static constexpr int NT = (NB + 31) / 32 * 32;
+    // bytes: populations [27][NB] float2, moments [3][NT] float4, ring [4][NR] float2, inlet velocities [NB] float4
+    static constexpr int kMom = (27 * NB * (int)sizeof(float2) + 15) / 16 * 16;
+    static constexpr int kRing = kMom + 3 * NT * (int)sizeof(float4);
+    static constexpr int kInflow = kRing + 4 * NR * (int)sizeof(float2);
+    static constexpr int kBytes = kInflow + NB * (int)sizeof(float4);
+    static_assert(kBytes <= 227 * 1024 && NR <= 2 * NT, "shared memory layout");
+};
+
+template <int B>
+__device__ __forceinline__ void cp_async(unsigned smem, const void *gmem) {
+    if constexpr (B == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+__device__ __forceinline__ int pmod(int a, int n) {
+    const int r = a % n;
+    return r < 0 ? r + n : r;
+}
+
+template <bool kForce, bool W, int TY, int MB>
+__global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepArgs a, AdvanceArgs v) {
+    using T = AdvanceTile<TY>;
+    constexpr int BX = T::BX, RX = T::RX, NB = T::NB, NT = T::NT;
+    extern __shared__ __align__(16) unsigned char smem[];
+    float4 *mb = reinterpret_cast<float4 *>(smem + T::kMom);
+    float2 *ring = reinterpret_cast<float2 *>(smem + T::kRing);
+    float4 *inflow = reinterpret_cast<float4 *>(smem + T::kInflow);
+
+    const int t = threadIdx.x;
+    const int tile = blockIdx.x % v.tiles, chunk = blockIdx.x / v.tiles;
+    const int x0 = (tile % v.tiles_x) * 32, y0 = (tile / v.tiles_x) * TY;
+    const int nx = a.nx, ny = a.ny, N = a.nz - 1, P = (int)a.plane;
+    const bool pz = a.bc_zlo == BC_PERIODIC, conv = a.bc_zhi == BC_CONVECTIVE;
+    const int z0 = (int)((long long)v.planes * chunk / v.chunks), z1 = (int)((long long)v.planes * (chunk + 1) / v.chunks);
+    const bool top = !pz && z1 == v.planes;  // the run that ends at z = N (conv: planes = N)
+    const int kb = pz ? z0 - 1 : max(z0 - 1, 0), ke = pz ? z1 : min(z1, N);
+
+    // the node this thread collides: tile position (bx, by) in the halo'd tile, wrapped where periodic;
+    // nothing lies beyond a side wall
+    const int bx = t % BX, by = t / BX;
+    int xs = x0 + bx - 1, ys = y0 + by - 1;
+    const bool wx = W && a.wall_x, wy = W && a.wall_y;
+    const bool collider = t < NB && xs <= nx && ys <= ny && !(wx && (xs < 0 || xs >= nx)) && !(wy && (ys < 0 || ys >= ny));
+    const bool inside = bx >= 1 && bx <= 32 && by >= 1 && by <= TY && xs < nx && ys < ny;
+    const int rpos = (by + 1) * RX + bx + 1;
+    xs = wrapi(xs, nx);
+    ys = wrapi(ys, ny);
+    const int cxy = collider ? ys * nx + xs : 0;
+    // the one or two ring positions this thread fills, clamped at side walls (mirror ghosts)
+    int fill[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int e = t + q * NT;
+        int X = x0 + e % RX - 2, Y = y0 + e / RX - 2;
+        X = wx ? min(max(X, 0), nx - 1) : pmod(X, nx);
+        Y = wy ? min(max(Y, 0), ny - 1) : pmod(Y, ny);
+        fill[q] = Y * nx + X;
+    }
+    // the node this thread gathers
+    const int gx_ = x0 + (t & 31), gy_ = y0 + (t >> 5);
+    const bool gatherer = t < 32 * TY && gx_ < nx && gy_ < ny;
+    const int gpos = ((t >> 5) + 1) * BX + (t & 31) + 1, gxy = gy_ * nx + gx_;
+
+    const unsigned s_ring = (unsigned)__cvta_generic_to_shared(ring), s_mb = (unsigned)__cvta_generic_to_shared(mb);
+    // planes beyond z walls mirror the wall plane
+    auto plane_of = [&](int k) { return pz ? pmod(k, a.nz) : min(max(k, 0), N); };
+    auto plane_after = [&](int z) { return z < N ? z + 1 : (pz ? 0 : N); };
+    auto fill_ring = [&](int k, int z) {  // slot of plane k from plane z
+        const float2 *src = v.phase + z * P;
+        const unsigned dst = s_ring + ((k & 3) * T::NR + t) * (int)sizeof(float2);
+        cp_async<sizeof(float2)>(dst, src + fill[0]);
+        if (t + NT < T::NR) cp_async<sizeof(float2)>(dst + NT * (int)sizeof(float2), src + fill[1]);
+    };
+    auto fetch_moments = [&](int z) {
+        const int n = z * P + cxy;
+        cp_async<16>(s_mb + t * 16, v.mom[0] + n);
+        cp_async<16>(s_mb + (NT + t) * 16, v.mom[1] + n);
+        cp_async<16>(s_mb + (2 * NT + t) * 16, v.mom[2] + n);
+    };
+    auto write_out = [&](int z, const Moments &m) {
+        const int n = z * P + gxy;
+        v.mom_out[0][n] = make_float4(m.rho_r, m.rho_b, m.phi, m.jx);
+        v.mom_out[1][n] = make_float4(m.jy, m.jz, m.dxz, m.dyz);
+        v.mom_out[2][n] = make_float4(m.pzz, m.pxy, m.pxz, m.pyz);
+        v.phase_out[n] = phase_entry(m);
+    };
+
+    fill_ring(kb - 1, plane_of(kb - 1));
+    fill_ring(kb, plane_of(kb));
+    int zr = plane_of(kb + 1);  // the last plane in the ring
+    fill_ring(kb + 1, zr);
+    int zm = plane_of(kb);      // the plane whose moments are here or on their way
+    fetch_moments(zm);
+    cp_async_commit();
+    cp_async_wait();
+    if (!pz && kb == 0 && a.bc_zlo == BC_INLET) {  // ghost plane z = -1 inside the inlet disc (own entries)
+        float2 *g = ring + 3 * T::NR;
+        for (int q = 0; q < 2; ++q)
+            if (t + q * NT < T::NR && a.disc[fill[q]]) g[t + q * NT] = make_float2(1.0f, a.rho_r0);
+    }
+    if (!pz && kb == 0 && a.bc_zlo == BC_INLET && collider) {  // velocity of the ghost columns inside the disc
+        float4 u = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (a.disc[cxy]) {
+            InletVel iv;
+            inlet_velocity(a.u_in, a.noise_amp, a.fourier, a.xc, a.yc, a.seed, a.step, xs, ys, nx, ny, iv);
+            u = make_float4(iv.ux, iv.uy, iv.uz, 1.0f);
+        }
+        inflow[t] = u;
+    }
+    __syncthreads();
+
+    auto collide = [&](int k) {
+        float2 *pop = reinterpret_cast<float2 *>(smem) + t;
+        const float4 *m = mb + t;
+        const Moments mo = unpack_moments(m[0], m[NT], m[2 * NT]);
+        const float2 *r[3] = {ring + ((k - 1) & 3) * T::NR + rpos, ring + (k & 3) * T::NR + rpos,
+                             ring + ((k + 1) & 3) * T::NR + rpos};
+        float2 gx, gy, gz;
+        gradients([&](int j) { return r[cz(j) + 1][cy(j) * RX + cx(j)]; }, gx, gy, gz);
+        if (a.grad4 && inside && k >= z0 && (k < z1 || top)) {
+            a.grad4[k * P + cxy] = make_float4(gx.x, gy.x, gz.x, gx.y);
+            a.grad2[k * P + cxy] = make_float2(gy.y, gz.y);
+        }
+        collide_node<kForce>(a, mo, gx, gy, gz, [&](int i, float2 f) {
+            pop[i * NB] = f;
+            // the record is in registers by now: its place takes the next plane's
+            if (i == 1 && k < ke) fetch_moments(plane_after(zm));
+            return f;
+        });
+    };
+
+    ZClass up{};      // class c_z = +1 of plane k + 1
+    HalfNode open{};  // classes +1 and 0 of plane k
+    const float2 *pop = reinterpret_cast<const float2 *>(smem);
+    // The pull of direction i comes from tile position gpos - c_i; wall: beyond a free-slip side wall it
+    // comes from the wall node itself, with that velocity component reversed (half-way specular
+    // reflection).  Blocks without wall nodes take the plain form.
+    const bool wxl = wx && gx_ == 0, wxh = wx && gx_ == nx - 1, wyl = wy && gy_ == 0, wyh = wy && gy_ == ny - 1;
+    const bool walled = (wx && (x0 == 0 || x0 + 32 >= nx)) || (wy && (y0 == 0 || y0 + TY >= ny));
+    auto gather = [&](int k, auto wall) {
+        constexpr bool kWall = decltype(wall)::value;
+        auto fx = [&](int i) { return kWall && (cx(i) > 0 ? wxl : (cx(i) < 0 ? wxh : false)); };
+        auto fy = [&](int i) { return kWall && (cy(i) > 0 ? wyl : (cy(i) < 0 ? wyh : false)); };
+        auto from = [&](int i) { return gpos - (fy(i) ? 0 : cy(i) * BX) - (fx(i) ? 0 : cx(i)); };
+        auto slot = [&](int i) { return fx(i) ? (fy(i) ? flip_xy(i) : flip_x(i)) : (fy(i) ? flip_y(i) : i); };
+        auto at = [&](int i) { return pop[slot(i) * NB + from(i)]; };
+        // reflected at a z wall: the slot whose direction has c_z reversed too
+        auto mirrored = [&](int i) {
+            const int m = mirror_z(i);
+            return pop[(fx(i) ? (fy(i) ? flip_xy(m) : flip_x(m)) : (fy(i) ? flip_y(m) : m)) * NB + from(i)];
+        };
+        if (!pz && k == 0)  // what enters plane 0 from z = -1: the inlet, or plane 0's own reflected
+            up = z_class<1>([&](int i) {
+                if (a.bc_zlo == BC_INLET) {
+                    const float4 u = inflow[from(i)];
+                    if (u.w != 0.0f)
+                        return make_float2(inlet_population(a, i, fx(i) ? -cx(i) : cx(i), fy(i) ? -cy(i) : cy(i), u.x, u.y, u.z), 0.0f);
+                }
+                return mirrored(i);
+            });
+        if (k > z0) write_out(k - 1, finish_moments(a, open, z_class<-1>(at)));
+        if (top && conv && k >= N - 2) {
+            // the outflow plane N needs the populations of plane N - 1 one by one: they are kept
+            // in this column's slots of the next history until the march is over
+            const size_t p = (size_t)P;
+#pragma unroll
+            for (int i = 0; i < 27; ++i)
+                if (cz(i) == N - 1 - k) {
+                    const float2 f = at(i);
+                    a.hist_out[i * p + gxy] = f.x;
+                    a.hist_out[(27 + i) * p + gxy] = f.y;
+                }
+        }
+        open = join_classes(up, z_class<0>(at), at(0));
+        up = z_class<1>(at);
+        if (top && !conv && k == N) write_out(N, finish_moments(a, open, z_class<-1>(mirrored)));
+    };
+    for (int k = kb; k <= ke; ++k) {
+        zr = plane_after(zr);
+        if (k < ke) fill_ring(k + 2, zr);
+        if (collider) collide(k);
+        zm = plane_after(zm);
+        cp_async_commit();
+        __syncthreads();
+        if (gatherer) {
+            if (W && walled)
+                gather(k, std::true_type{});
+            else
+                gather(k, std::false_type{});
+        }
+        cp_async_wait();
+        __syncthreads();
+    }
+    if (top && conv && gatherer) {  // f(N, t + 1) from f(N - 1, t + 1) and f(N, t)
+        const size_t p = (size_t)P;
+        float2 f[27];
+#pragma unroll
+        for (int i = 0; i < 27; ++i) f[i] = make_float2(a.hist_out[i * p + gxy], a.hist_out[(27 + i) * p + gxy]);
+        const float lam = outflow_lambda(a, moments_of(a, [&](int i) { return f[i]; }));
+        const float inv = 1.0f / (1.0f + lam);
+#pragma unroll
+        for (int i = 0; i < 27; ++i) {
+            if (i % 6 == 0) asm volatile("" ::: "memory");  // six directions' loads in flight, not all 27 in registers
+            if (a.fm_out) {
+                a.fm_out[i * p + gxy] = f[i].x;
+                a.fm_out[(27 + i) * p + gxy] = f[i].y;
+            }
+            f[i] = make_float2(outflow_blend(__ldg(a.hist_in + i * p + gxy), f[i].x, lam, inv),
+                               outflow_blend(__ldg(a.hist_in + (27 + i) * p + gxy), f[i].y, lam, inv));
+            a.hist_out[i * p + gxy] = f[i].x;
+            a.hist_out[(27 + i) * p + gxy] = f[i].y;
+        }
+        write_out(N, moments_of(a, [&](int i) { return f[i]; }));
+    }
+}
+
+// ------------------------------------------------------------------------ launchers
+template <bool kForce, bool W, int TY, int MB>
+static cudaError_t launch_tile(const StepArgs &a, AdvanceArgs v, int chunks, cudaStream_t s) {
+    using T = AdvanceTile<TY>;
+    auto *fn = advance_kernel<kForce, W, TY, MB>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kBytes);
+    if (e != cudaSuccess) return e;
+    v.tiles_x = (a.nx + 31) / 32;
+    v.tiles = v.tiles_x * ((a.ny + TY - 1) / TY);
+    v.planes = a.bc_zhi == BC_CONVECTIVE ? a.nz - 1 : a.nz;
+    v.chunks = std::min(chunks, v.planes);
+    for (int q = 1; q < 3; ++q) {
+        v.mom[q] = v.mom[0] + q * a.NN;
+        v.mom_out[q] = v.mom_out[0] + q * a.NN;
+    }
+    fn<<<(unsigned)v.tiles * v.chunks, T::NT, T::kBytes, s>>>(a, v);
+    return cudaGetLastError();
+}
+
+template <int TY, int MB>
+static cudaError_t launch_ty(const StepArgs &a, const AdvanceArgs &v, int chunks, cudaStream_t s) {
+    const bool force = a.gx != 0.0f || a.gy != 0.0f || a.gz != 0.0f;
+    if (a.wall_x || a.wall_y)
+        return force ? launch_tile<true, true, TY, MB>(a, v, chunks, s) : launch_tile<false, true, TY, MB>(a, v, chunks, s);
+    return force ? launch_tile<true, false, TY, MB>(a, v, chunks, s) : launch_tile<false, false, TY, MB>(a, v, chunks, s);
+}
+
+constexpr int kSMs = 152;
+
+// Which tile and how many runs of planes: the estimated time of the last wave's end, with the
+// measured time a plane takes a resident block (us, 256 x 256 x 512 periodic, FP32): 3.66 for the
+// 32 x 16 tile (one block of 20 warps on an SM), 3.28 for the 32 x 7 tile (two blocks of 10 warps;
+// 2.0 when a block has the SM to itself).  Both reach 19 G nodes/s on large lattices; the small tile
+// wastes less on planes that are no multiple of 16 rows and fills the chip with fewer columns.  A run
+// collides one plane more at each end, and about 8 us go into filling and draining it.
+AdvancePlan plan_advance(const StepArgs &a) {
+    const int planes = a.bc_zhi == BC_CONVECTIVE ? a.nz - 1 : a.nz;
+    AdvancePlan best{0, 1, 1e30f};
+    for (int ty : {16, 7}) {
+        const long long tiles = (long long)((a.nx + 31) / 32) * ((a.ny + ty - 1) / ty);
+        for (int chunks = 1; chunks <= planes && chunks <= 4 * kSMs; ++chunks) {
+            const long long blocks = tiles * chunks, slots = ty == 16 ? kSMs : 2 * kSMs;
+            const float plane_us = ty == 16 ? 3.66f : (blocks <= kSMs ? 2.0f : 3.28f);
+            const float us = (float)((blocks + slots - 1) / slots) * (float)((planes + chunks - 1) / chunks + 2) * plane_us + 8.0f;
+            if (us < best.us) best = AdvancePlan{ty, chunks, us};
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_advance(const StepArgs &a, const AdvancePlan &p, const AdvanceArgs &v, cudaStream_t s,
+                           long long *launches) {
+    *launches += 1;
+    return p.ty == 16 ? launch_ty<16, 1>(a, v, p.chunks, s) : launch_ty<7, 2>(a, v, p.chunks, s);
+}
+
+}  // namespace lbcm

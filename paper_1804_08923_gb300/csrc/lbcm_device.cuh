@@ -292,14 +292,13 @@ __device__ __forceinline__ float fit_entry_rho(float4 e) {
     return __half2float(__ushort_as_half((unsigned short)(__float_as_uint(e.w) >> 16)));
 }
 
+// from a phase entry
 template <int S>
-__device__ __forceinline__ Own own_of(const float4 *ph, int n) {
+__device__ __forceinline__ Own own_from(float4 v) {
     Own o{};
     if constexpr (S == STORE_FP16) {
-        const float4 v = __ldg(ph + n);
         o.A = make_float2(v.z, v.w);
     } else if constexpr (S == STORE_FP16_FIT) {
-        const float4 v = __ldg(ph + n);
         const unsigned int y = __float_as_uint(v.y), z = __float_as_uint(v.z), w = __float_as_uint(v.w);
         o.Ah = *reinterpret_cast<const __half2 *>(&y);
         o.v[0] = fp8x2_to_half2(z);
@@ -307,6 +306,13 @@ __device__ __forceinline__ Own own_of(const float4 *ph, int n) {
         o.v[2] = fp8x2_to_half2(w);
     }
     return o;
+}
+template <int S>
+__device__ __forceinline__ Own own_of(const float4 *ph, int n) {
+    if constexpr (S == STORE_FP32)
+        return Own{};
+    else
+        return own_from<S>(__ldg(ph + n));
 }
 
 // FP16_FIT prediction P^k for the slot of direction j (class q of i = class of j), in half-precision
@@ -401,6 +407,23 @@ __device__ __forceinline__ Own reader_shift(const StepArgs &a, int n) {
     return own_of<S>(a.ph_prev, n);
 }
 
+// Populations f of direction i >= 1 in half precision for a reader that decodes with dest: h is
+// what is stored, the result what that reader will decode.
+template <int S>
+__device__ __forceinline__ float2 encode_pop(const StepArgs &a, int i, float2 f, const Own &dest, __half2 &h) {
+    if constexpr (S == STORE_FP16) {
+        const float2 w = shift_w(a, i);
+        h = __floats2half2_rn(fmaf(-dest.A.x, w.x, f.x), fmaf(-dest.A.y, w.y, f.y));
+        const float2 hf = __half22float2(h);
+        return make_float2(fmaf(dest.A.x, w.x, hf.x), fmaf(dest.A.y, w.y, hf.y));
+    } else {
+        const float2 p = fit_pred(a, i, i, dest);
+        h = __floats2half2_rn((f.x - p.x) * a.dev_scale, (f.y - p.y) * a.dev_scale);
+        const float2 hf = __half22float2(h);
+        return make_float2(fmaf(hf.x, a.inv_dev_scale, p.x), fmaf(hf.y, a.inv_dev_scale, p.y));
+    }
+}
+
 // Store populations f of direction i at node n; dest = what the node n + c_i that will read
 // them decodes with (FP16).  Returns the values that node will decode, so the caller can
 // account for the storage rounding.
@@ -415,20 +438,10 @@ __device__ __forceinline__ float2 store_pop(const StepArgs &a, int i, int n, flo
             rest[n] = f;
             return f;
         }
-        __half2 *slot = reinterpret_cast<__half2 *>(rest + a.NN) + (size_t)(i - 1) * a.NN + n;
-        if constexpr (S == STORE_FP16) {
-            const float2 w = shift_w(a, i);
-            const __half2 h = __floats2half2_rn(fmaf(-dest.A.x, w.x, f.x), fmaf(-dest.A.y, w.y, f.y));
-            *slot = h;
-            const float2 hf = __half22float2(h);
-            return make_float2(fmaf(dest.A.x, w.x, hf.x), fmaf(dest.A.y, w.y, hf.y));
-        } else {
-            const float2 p = fit_pred(a, i, i, dest);
-            const __half2 h = __floats2half2_rn((f.x - p.x) * a.dev_scale, (f.y - p.y) * a.dev_scale);
-            *slot = h;
-            const float2 hf = __half22float2(h);
-            return make_float2(fmaf(hf.x, a.inv_dev_scale, p.x), fmaf(hf.y, a.inv_dev_scale, p.y));
-        }
+        __half2 h;
+        const float2 d = encode_pop<S>(a, i, f, dest, h);
+        reinterpret_cast<__half2 *>(rest + a.NN)[(size_t)(i - 1) * a.NN + n] = h;
+        return d;
     }
 }
 __device__ __forceinline__ Own no_shift() { return Own{}; }

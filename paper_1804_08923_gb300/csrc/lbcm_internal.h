@@ -15,6 +15,29 @@ enum { PASS_GATHER = 1, PASS_COLLIDE = 2, PASS_BOTH = 3 };
 cudaError_t launch_step(const StepArgs &a, int storage, cudaStream_t s, cudaEvent_t *ev, long long *launches,
                         int passes = PASS_BOTH);
 
+// One step from moment record to moment record (lbcm_advance.cu; paper rates, FP32 storage): mom and
+// phase are a gather pass's output (mom [3][NN] float4, phase [NN] float2), mom_out and phase_out receive those of the next step, whose index, history planes and
+// optional adjoint records (grad4, grad2: of the step that mom belongs to) are a's.
+struct AdvanceArgs {
+    const float4 *mom[3];  // [0] is given; the launcher sets the other two planes of the record
+    const float2 *phase;
+    float4 *mom_out[3];
+    float2 *phase_out;
+    int tiles_x, tiles, planes, chunks;  // set by the launcher: column tiles, planes marched, runs of planes
+};
+// Tile rows and runs of planes of an advance, and its estimated time (us).
+struct AdvancePlan {
+    int ty, chunks;
+    float us;
+};
+AdvancePlan plan_advance(const StepArgs &a);
+cudaError_t launch_advance(const StepArgs &a, const AdvancePlan &p, const AdvanceArgs &v, cudaStream_t s,
+                           long long *launches);
+
+// The two passes of a step with relaxation rates other than the paper's (lbcm_general.cu).
+void launch_general_gather(const StepArgs &a, int storage, cudaStream_t s);
+void launch_general_collide(const StepArgs &a, int storage, cudaStream_t s);
+
 // Control block of the fused step kernel (both passes of a step in one cooperative launch,
 // paper rates only): the item sequence and the per-plane completion counters.
 struct FusedCtl {
@@ -55,7 +78,7 @@ cudaError_t launch_fused_wait_probe(const FusedCtl &f, unsigned long long *ns, c
 //   acc_coll        FP64 per-block sums of dJ/d(sigma, nu_r, nu_b) [blocks][3]
 //   acc_inlet       FP64 per-block sums of dJ/d(u_in, a_1, b_1, ..., a_8, b_8) [blocks][17]
 //   mom             the forward step's collision moments per node, [3][NN] float4 as the moment
-//                   pass writes them: (rho_r, rho_b, sf, jx), (jy, jz, pxx, pyy), (pzz, pxy, pxz, pyz)
+//                   pass writes them: (rho_r, rho_b, phi, jx), (jy, jz, dxz, dyz), (pzz, pxy, pxz, pyz)
 //   grad4, grad2    its gradients per node (as StepArgs::grad4, grad2)
 //   fm              the forward step's f(N-1) of the outflow columns [54][nx ny]
 struct AdjArgs {
