@@ -32,7 +32,8 @@ template <int TY>
 struct AdvanceTile {
     static constexpr int BX = 34, RX = 36, RY = TY + 4;    // row of collided nodes, ring of phase nodes
     static constexpr int NB = BX * (TY + 2), NR = RX * RY;
-    static constexpr int NT = (NB + 31) / 32 * 32;
+    // warps: TY rows of the tile, the two halo rows, the halo columns with the corners
+    static constexpr int NT = 32 * (TY + 2) + (2 * (TY + 2) + 31) / 32 * 32;
     // bytes: populations [27][NB] float2, moments [3][NT] float4, ring [4][NR] float2, inlet velocities [NB] float4
     static constexpr int kMom = (27 * NB * (int)sizeof(float2) + 15) / 16 * 16;
     static constexpr int kRing = kMom + 3 * NT * (int)sizeof(float4);
@@ -74,14 +75,18 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
     const bool top = !pz && z1 == v.planes;  // the run that ends at z = N (conv: planes = N)
     const int kb = pz ? z0 - 1 : max(z0 - 1, 0), ke = pz ? z1 : min(z1, N);
 
-    // the node this thread collides: tile position (bx, by) in the halo'd tile, wrapped where periodic;
-    // nothing lies beyond a side wall
-    const int bx = t % BX, by = t / BX;
+    // the node this thread collides, at position (bx, by) of the tile with its halo, wrapped where
+    // periodic; nothing lies beyond a side wall
+    const int warp = t >> 5, lane = t & 31, e = t - 32 * (TY + 2);
+    const bool row = warp < TY, halo_y = !row && warp < TY + 2;
+    const int bx = e < 0 ? lane + 1 : (e & 1 ? BX - 1 : 0), by = row ? warp + 1 : (halo_y ? (warp == TY ? 0 : TY + 1) : e >> 1);
+    const float side = e < 0 ? (by == 0 ? 1.0f : -1.0f) : (bx == 0 ? 1.0f : -1.0f);  // halo: the component that enters
     int xs = x0 + bx - 1, ys = y0 + by - 1;
     const bool wx = W && a.wall_x, wy = W && a.wall_y;
-    const bool collider = t < NB && xs <= nx && ys <= ny && !(wx && (xs < 0 || xs >= nx)) && !(wy && (ys < 0 || ys >= ny));
-    const bool inside = bx >= 1 && bx <= 32 && by >= 1 && by <= TY && xs < nx && ys < ny;
-    const int rpos = (by + 1) * RX + bx + 1;
+    const bool collider = by < TY + 2 && xs <= nx && ys <= ny && !(wx && (xs < 0 || xs >= nx)) && !(wy && (ys < 0 || ys >= ny));
+    const bool inside = row && xs < nx && ys < ny;  // a node of the tile: this thread gathers it too
+    const int pos = by * BX + bx, rpos = (by + 1) * RX + bx + 1;
+    const int x = xs, y = ys;
     xs = wrapi(xs, nx);
     ys = wrapi(ys, ny);
     const int cxy = collider ? ys * nx + xs : 0;
@@ -95,11 +100,6 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
         Y = wy ? min(max(Y, 0), ny - 1) : pmod(Y, ny);
         fill[q] = Y * nx + X;
     }
-    // the node this thread gathers
-    const int gx_ = x0 + (t & 31), gy_ = y0 + (t >> 5);
-    const bool gatherer = t < 32 * TY && gx_ < nx && gy_ < ny;
-    const int gpos = ((t >> 5) + 1) * BX + (t & 31) + 1, gxy = gy_ * nx + gx_;
-
     const unsigned s_ring = (unsigned)__cvta_generic_to_shared(ring), s_mb = (unsigned)__cvta_generic_to_shared(mb);
     // planes beyond z walls mirror the wall plane
     auto plane_of = [&](int k) { return pz ? pmod(k, a.nz) : min(max(k, 0), N); };
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
         cp_async<16>(s_mb + (2 * NT + t) * 16, v.mom[2] + n);
     };
     auto write_out = [&](int z, const Moments &m) {
-        const int n = z * P + gxy;
+        const int n = z * P + cxy;
         v.mom_out[0][n] = make_float4(m.rho_r, m.rho_b, m.phi, m.jx);
         v.mom_out[1][n] = make_float4(m.jy, m.jz, m.dxz, m.dyz);
         v.mom_out[2][n] = make_float4(m.pzz, m.pxy, m.pxz, m.pyz);
@@ -144,12 +144,13 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
             inlet_velocity(a.u_in, a.noise_amp, a.fourier, a.xc, a.yc, a.seed, a.step, xs, ys, nx, ny, iv);
             u = make_float4(iv.ux, iv.uy, iv.uz, 1.0f);
         }
-        inflow[t] = u;
+        inflow[pos] = u;
     }
     __syncthreads();
 
-    auto collide = [&](int k) {
-        float2 *pop = reinterpret_cast<float2 *>(smem) + t;
+    // collides plane k; the rest population of a node of the tile stays with its thread
+    auto collide = [&](int k, float2 &rest) {
+        float2 *out = reinterpret_cast<float2 *>(smem) + pos;
         const float4 *m = mb + t;
         const Moments mo = unpack_moments(m[0], m[NT], m[2 * NT]);
         const float2 *r[3] = {ring + ((k - 1) & 3) * T::NR + rpos, ring + (k & 3) * T::NR + rpos,
@@ -160,27 +161,45 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
             a.grad4[k * P + cxy] = make_float4(gx.x, gy.x, gz.x, gx.y);
             a.grad2[k * P + cxy] = make_float2(gy.y, gz.y);
         }
-        collide_node<kForce>(a, mo, gx, gy, gz, [&](int i, float2 f) {
-            pop[i * NB] = f;
-            // the record is in registers by now: its place takes the next plane's
-            if (i == 1 && k < ke) fetch_moments(plane_after(zm));
-            return f;
-        });
+        // once the record is in registers its place takes the next plane's
+        auto fetch = [&](int i, int first) {
+            if (i == first && k < ke) fetch_moments(plane_after(zm));
+        };
+        if (row) {
+            collide_node<kForce>(a, mo, gx, gy, gz, [&](int i, float2 f) {
+                if (i == 0)
+                    rest = f;
+                else
+                    out[i * NB] = f;
+                fetch(i, 1);
+                return f;
+            });
+        } else if (halo_y) {
+            collide_halo_y<kForce>(a, mo, gx, gy, gz, side, [&](int i, float2 f) {
+                out[(side > 0.0f ? i : flip_y(i)) * NB] = f;
+                fetch(i, 3);
+            });
+        } else {
+            collide_halo_x<kForce>(a, mo, gx, gy, gz, side, [&](int i, float2 f) {
+                out[(side > 0.0f ? i : flip_x(i)) * NB] = f;
+                fetch(i, 1);
+            });
+        }
     };
 
     ZClass up{};      // class c_z = +1 of plane k + 1
     HalfNode open{};  // classes +1 and 0 of plane k
     const float2 *pop = reinterpret_cast<const float2 *>(smem);
-    // The pull of direction i comes from tile position gpos - c_i; wall: beyond a free-slip side wall it
+    // The pull of direction i comes from tile position pos - c_i; wall: beyond a free-slip side wall it
     // comes from the wall node itself, with that velocity component reversed (half-way specular
     // reflection).  Blocks without wall nodes take the plain form.
-    const bool wxl = wx && gx_ == 0, wxh = wx && gx_ == nx - 1, wyl = wy && gy_ == 0, wyh = wy && gy_ == ny - 1;
+    const bool wxl = wx && x == 0, wxh = wx && x == nx - 1, wyl = wy && y == 0, wyh = wy && y == ny - 1;
     const bool walled = (wx && (x0 == 0 || x0 + 32 >= nx)) || (wy && (y0 == 0 || y0 + TY >= ny));
-    auto gather = [&](int k, auto wall) {
+    auto gather = [&](int k, float2 rest, auto wall) {
         constexpr bool kWall = decltype(wall)::value;
         auto fx = [&](int i) { return kWall && (cx(i) > 0 ? wxl : (cx(i) < 0 ? wxh : false)); };
         auto fy = [&](int i) { return kWall && (cy(i) > 0 ? wyl : (cy(i) < 0 ? wyh : false)); };
-        auto from = [&](int i) { return gpos - (fy(i) ? 0 : cy(i) * BX) - (fx(i) ? 0 : cx(i)); };
+        auto from = [&](int i) { return pos - (fy(i) ? 0 : cy(i) * BX) - (fx(i) ? 0 : cx(i)); };
         auto slot = [&](int i) { return fx(i) ? (fy(i) ? flip_xy(i) : flip_x(i)) : (fy(i) ? flip_y(i) : i); };
         auto at = [&](int i) { return pop[slot(i) * NB + from(i)]; };
         // reflected at a z wall: the slot whose direction has c_z reversed too
@@ -205,49 +224,50 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
 #pragma unroll
             for (int i = 0; i < 27; ++i)
                 if (cz(i) == N - 1 - k) {
-                    const float2 f = at(i);
-                    a.hist_out[i * p + gxy] = f.x;
-                    a.hist_out[(27 + i) * p + gxy] = f.y;
+                    const float2 f = i == 0 ? rest : at(i);
+                    a.hist_out[i * p + cxy] = f.x;
+                    a.hist_out[(27 + i) * p + cxy] = f.y;
                 }
         }
-        open = join_classes(up, z_class<0>(at), at(0));
+        open = join_classes(up, z_class<0>(at), rest);
         up = z_class<1>(at);
         if (top && !conv && k == N) write_out(N, finish_moments(a, open, z_class<-1>(mirrored)));
     };
     for (int k = kb; k <= ke; ++k) {
         zr = plane_after(zr);
         if (k < ke) fill_ring(k + 2, zr);
-        if (collider) collide(k);
+        float2 rest;
+        if (collider) collide(k, rest);
         zm = plane_after(zm);
         cp_async_commit();
         __syncthreads();
-        if (gatherer) {
+        if (inside) {
             if (W && walled)
-                gather(k, std::true_type{});
+                gather(k, rest, std::true_type{});
             else
-                gather(k, std::false_type{});
+                gather(k, rest, std::false_type{});
         }
         cp_async_wait();
         __syncthreads();
     }
-    if (top && conv && gatherer) {  // f(N, t + 1) from f(N - 1, t + 1) and f(N, t)
+    if (top && conv && inside) {  // f(N, t + 1) from f(N - 1, t + 1) and f(N, t)
         const size_t p = (size_t)P;
         float2 f[27];
 #pragma unroll
-        for (int i = 0; i < 27; ++i) f[i] = make_float2(a.hist_out[i * p + gxy], a.hist_out[(27 + i) * p + gxy]);
+        for (int i = 0; i < 27; ++i) f[i] = make_float2(a.hist_out[i * p + cxy], a.hist_out[(27 + i) * p + cxy]);
         const float lam = outflow_lambda(a, moments_of(a, [&](int i) { return f[i]; }));
         const float inv = 1.0f / (1.0f + lam);
 #pragma unroll
         for (int i = 0; i < 27; ++i) {
             if (i % 6 == 0) asm volatile("" ::: "memory");  // six directions' loads in flight, not all 27 in registers
             if (a.fm_out) {
-                a.fm_out[i * p + gxy] = f[i].x;
-                a.fm_out[(27 + i) * p + gxy] = f[i].y;
+                a.fm_out[i * p + cxy] = f[i].x;
+                a.fm_out[(27 + i) * p + cxy] = f[i].y;
             }
-            f[i] = make_float2(outflow_blend(__ldg(a.hist_in + i * p + gxy), f[i].x, lam, inv),
-                               outflow_blend(__ldg(a.hist_in + (27 + i) * p + gxy), f[i].y, lam, inv));
-            a.hist_out[i * p + gxy] = f[i].x;
-            a.hist_out[(27 + i) * p + gxy] = f[i].y;
+            f[i] = make_float2(outflow_blend(__ldg(a.hist_in + i * p + cxy), f[i].x, lam, inv),
+                               outflow_blend(__ldg(a.hist_in + (27 + i) * p + cxy), f[i].y, lam, inv));
+            a.hist_out[i * p + cxy] = f[i].x;
+            a.hist_out[(27 + i) * p + cxy] = f[i].y;
         }
         write_out(N, moments_of(a, [&](int i) { return f[i]; }));
     }

@@ -59,140 +59,173 @@ struct Axis {
     __device__ __forceinline__ explicit Axis(float v) : u(v), u2(2.0f * v), uu(v * v) {}
 };
 
-// emit(i, f) stores the populations (red, blue) f of direction i and returns them as they will be
-// read back (with a half-precision storage, rounded); the mass of the moving ones is summed from
-// those, in the association of z_class / finish_moments (lbcm_node.cuh), so that the reader of an
-// unchanged set gets the node's colour densities back exactly.
+// The collision of one node, up to the evaluation of single directions.
 //
 // Every term but the recolouring's 1/|c_i| and the relaxed second moment is w_i times a polynomial
 // in c_i for i >= 1: varphi_i(alpha) = (27/19) w_i (1 - alpha), Phi_i = 9 w_i nu (c_i.u)(c_i.grad
 // rho), B_i = w_i.  So the even part of a pair of opposite directions is w_i (C0 + c_i^T Q c_i)
-// with one symmetric Q per node, and the odd part w_i (c_i.u)(b + d (c_i.u)^2) (+ the force).  The
+// with one symmetric Q per node, and the odd part w_i (c_i.u)(lb + ld (c_i.u)^2) (+ the force).  The
 // relaxed second moment K goes through the inverse central-moment transform about u by 1-D
 // sweeps (K has no moments of order 0 and 1: those of f - f^e + F'/2 vanish).
-template <bool kForce, class E>
-__device__ __forceinline__ void collide_node(const StepArgs &a, const Moments &mo, float2 gx, float2 gy, float2 gz,
-                                             E &&emit) {
-    const float gpx = gx.x, gpy = gy.x, gpz = gz.x, grx = gx.y, gry = gy.y, grz = gz.y;
-    // macroscopic quantities (Eqs. (13), (48), (23)) and mixture parameters
-    const float rho = mo.rho_r + mo.rho_b;
-    const float inv_rho = rcp_newton(rho);
-    float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
-    if (kForce) {
-        const float fo = rho - a.rho_b0;
-        Fx = fo * a.gx; Fy = fo * a.gy; Fz = fo * a.gz;
-    }
-    const float ux = (kForce ? fmaf(0.5f, Fx, mo.jx) : mo.jx) * inv_rho;
-    const float uy = (kForce ? fmaf(0.5f, Fy, mo.jy) : mo.jy) * inv_rho;
-    const float uz = (kForce ? fmaf(0.5f, Fz, mo.jz) : mo.jz) * inv_rho;
-    const float hp = fmaf(0.5f, mo.phi, 0.5f), hm = fmaf(-0.5f, mo.phi, 0.5f);
-    const float oma = a.alpha_mix ? fmaf(mo.rho_r, a.oma_r, mo.rho_b * a.oma_b) * inv_rho : fmaf(hp, a.oma_r, hm * a.oma_b);
-    const float nu = rcp_newton(fmaf(hp, a.inv_nu_r, hm * a.inv_nu_b));
-    const float s2nu = rcp_newton(fmaf(3.0f, nu, 0.5f));  // 1/tau
-    const float usq = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
-    const float g2 = fmaf(gpx, gpx, fmaf(gpy, gpy, gpz * gpz));
-    const float inv_gm = rsqrt_newton(fmaxf(g2 + a.eps2, 1.1754944e-38f));  // 1/|grad phi|_eps, a normal number
-    const float pert = (2.25f * a.sigma) * s2nu * inv_gm;  // A / |grad phi|, A = 9 sigma / (4 tau)
+//
+// Reversing the sign of one component of every vector and tensor reverses that component of c_i in the
+// result and nothing else, bit for bit: products and sums only change sign.  The halo versions below
+// rest on it.
+template <bool kForce>
+struct Collision {
+    float rho_r, rho_b, rho, ux, uy, uz, Fx, Fy, Fz, gpx, gpy, gpz;
+    float C0, qxx, qyy, qzz, qxy, qxz, qyz, lb, ld, frac_r, frac_b, sg1, sg2, sg3;
+    float V00[3], V10[3], V01[3], V20[3], V02[3], V11[3];  // [c_z + 1], moments (p, q) in (x, y), half values
 
-    // S = rho u u + nu (u g + g u), the anisotropic second moment of f^e; Fh = (u F + F u) / 2
-    const float rux = rho * ux, ruy = rho * uy, ruz = rho * uz;
-    float Sxx = fmaf(rux, ux, nu * (2.0f * ux * grx)), Syy = fmaf(ruy, uy, nu * (2.0f * uy * gry)),
-          Szz = fmaf(ruz, uz, nu * (2.0f * uz * grz));
-    float Sxy = fmaf(rux, uy, nu * fmaf(ux, gry, uy * grx)), Sxz = fmaf(rux, uz, nu * fmaf(ux, grz, uz * grx)),
-          Syz = fmaf(ruy, uz, nu * fmaf(uy, grz, uz * gry));
-    // second central moments of Delta = f - f^e + F'/2, without the isotropic part of f^e
-    float uF = 0.0f;
-    float Txx = Sxx, Tyy = Syy, Tzz = Szz, Txy = Sxy, Txz = Sxz, Tyz = Syz;  // what Delta takes off Pi(f)
-    if (kForce) {
-        uF = fmaf(ux, Fx, fmaf(uy, Fy, uz * Fz));
-        const float hxx = ux * Fx, hyy = uy * Fy, hzz = uz * Fz;
-        const float hxy = 0.5f * fmaf(ux, Fy, uy * Fx), hxz = 0.5f * fmaf(ux, Fz, uz * Fx), hyz = 0.5f * fmaf(uy, Fz, uz * Fy);
-        Txx -= hxx; Tyy -= hyy; Tzz -= hzz; Txy -= hxy; Txz -= hxz; Tyz -= hyz;
-        Sxx += hxx; Syy += hyy; Szz += hzz; Sxy += hxy; Sxz += hxz; Syz += hyz;
-    }
-    // K: shear part with 1 - 1/tau, trace with 1 - s2b (0 with the paper's s2b = 1); halved
-    const float o2 = 1.0f - s2nu, h2 = 0.5f * o2, t3 = (0.5f / 3.0f) * o2;
-    const float k110 = h2 * (mo.pxy - Txy), k101 = h2 * (mo.pxz - Txz), k011 = h2 * (mo.pyz - Tyz);
-    const float e1 = t3 * (mo.dxz - (Txx - Tzz)), e2 = t3 * (mo.dyz - (Tyy - Tzz));
-    float k200 = fmaf(2.0f, e1, -e2), k020 = fmaf(2.0f, e2, -e1), k002 = -(e1 + e2);
-    if (a.s2b != 1.0f) {
-        const float ugr = fmaf(ux, grx, fmaf(uy, gry, uz * grz));
-        const float iso = fmaf(rho * oma, 9.0f / 19.0f, nu * ugr);
-        const float tr = (fmaf(3.0f, mo.pzz, mo.dxz + mo.dyz) - ((Txx + Tyy) + Tzz)) - 3.0f * iso;
-        const float t = (0.5f / 3.0f) * (1.0f - a.s2b) * tr;
-        k200 += t; k020 += t; k002 += t;
-    }
+    // ax, ay, az: gravity
+    __device__ __forceinline__ Collision(const StepArgs &a, const Moments &mo, float2 gx, float2 gy, float2 gz, float ax,
+                                         float ay, float az) {
+        gpx = gx.x; gpy = gy.x; gpz = gz.x;
+        const float grx = gx.y, gry = gy.y, grz = gz.y;
+        rho_r = mo.rho_r;
+        rho_b = mo.rho_b;
+        // macroscopic quantities (Eqs. (13), (48), (23)) and mixture parameters
+        rho = mo.rho_r + mo.rho_b;
+        const float inv_rho = rcp_newton(rho);
+        Fx = Fy = Fz = 0.0f;
+        if (kForce) {
+            const float fo = rho - a.rho_b0;
+            Fx = fo * ax; Fy = fo * ay; Fz = fo * az;
+        }
+        ux = (kForce ? fmaf(0.5f, Fx, mo.jx) : mo.jx) * inv_rho;
+        uy = (kForce ? fmaf(0.5f, Fy, mo.jy) : mo.jy) * inv_rho;
+        uz = (kForce ? fmaf(0.5f, Fz, mo.jz) : mo.jz) * inv_rho;
+        const float hp = fmaf(0.5f, mo.phi, 0.5f), hm = fmaf(-0.5f, mo.phi, 0.5f);
+        const float oma = a.alpha_mix ? fmaf(mo.rho_r, a.oma_r, mo.rho_b * a.oma_b) * inv_rho : fmaf(hp, a.oma_r, hm * a.oma_b);
+        const float nu = rcp_newton(fmaf(hp, a.inv_nu_r, hm * a.inv_nu_b));
+        const float s2nu = rcp_newton(fmaf(3.0f, nu, 0.5f));  // 1/tau
+        const float usq = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
+        const float g2 = fmaf(gpx, gpx, fmaf(gpy, gpy, gpz * gpz));
+        const float inv_gm = rsqrt_newton(fmaxf(g2 + a.eps2, 1.1754944e-38f));  // 1/|grad phi|_eps, a normal number
+        const float pert = (2.25f * a.sigma) * s2nu * inv_gm;  // A / |grad phi|, A = 9 sigma / (4 tau)
 
-    // even part of the pairs: C0 + c^T Q c
-    const float C0 = fmaf(rho * oma, 27.0f / 19.0f, fmaf(-1.5f * rho, usq, fmaf(-pert, g2, -1.5f * uF)));
-    const float px = pert * gpx, py = pert * gpy;
-    const float qxx = fmaf(4.5f, Sxx, px * gpx), qyy = fmaf(4.5f, Syy, py * gpy), qzz = fmaf(4.5f, Szz, pert * gpz * gpz);
-    const float qxy = fmaf(9.0f, Sxy, 2.0f * px * gpy), qxz = fmaf(9.0f, Sxz, 2.0f * px * gpz),
-                qyz = fmaf(9.0f, Syz, 2.0f * py * gpz);
-    const float cx0 = C0 + qxx, cy0 = C0 + qyy, cz0 = C0 + qzz;
-    const float exy = cx0 + qyy, exz = cx0 + qzz, eyz = cy0 + qzz, exyz = exy + qzz;
-    // odd part: (c.u) (lb + ld (c.u)^2) + 3/2 c.F
-    const float lb = rho * fmaf(-4.5f, usq, 3.0f), ld = 4.5f * rho;
-    // recolouring: +- seg_i, seg_i = w_i/|c_i| seg0 (c_i.grad phi); seg0 = beta rho_r rho_b (27/19)(1 - alpha) / (rho |grad phi|)
-    const float frac_r = mo.rho_r * inv_rho, frac_b = mo.rho_b * inv_rho;
-    const float seg0 = a.beta * mo.rho_r * frac_b * inv_gm * (oma * (27.0f / 19.0f));
-    const float sg1 = (2.0f / 27.0f) * seg0, sg2 = (float)(0.70710678118654752 / 54.0) * seg0,
-                sg3 = (float)(0.57735026918962576 / 216.0) * seg0;
+        // S = rho u u + nu (u g + g u), the anisotropic second moment of f^e; Fh = (u F + F u) / 2
+        const float rux = rho * ux, ruy = rho * uy, ruz = rho * uz;
+        float Sxx = fmaf(rux, ux, nu * (2.0f * ux * grx)), Syy = fmaf(ruy, uy, nu * (2.0f * uy * gry)),
+              Szz = fmaf(ruz, uz, nu * (2.0f * uz * grz));
+        float Sxy = fmaf(rux, uy, nu * fmaf(ux, gry, uy * grx)), Sxz = fmaf(rux, uz, nu * fmaf(ux, grz, uz * grx)),
+              Syz = fmaf(ruy, uz, nu * fmaf(uy, grz, uz * gry));
+        // second central moments of Delta = f - f^e + F'/2, without the isotropic part of f^e
+        float uF = 0.0f;
+        float Txx = Sxx, Tyy = Syy, Tzz = Szz, Txy = Sxy, Txz = Sxz, Tyz = Syz;  // what Delta takes off Pi(f)
+        if (kForce) {
+            uF = fmaf(ux, Fx, fmaf(uy, Fy, uz * Fz));
+            const float hxx = ux * Fx, hyy = uy * Fy, hzz = uz * Fz;
+            const float hxy = 0.5f * fmaf(ux, Fy, uy * Fx), hxz = 0.5f * fmaf(ux, Fz, uz * Fx), hyz = 0.5f * fmaf(uy, Fz, uz * Fy);
+            Txx -= hxx; Tyy -= hyy; Tzz -= hzz; Txy -= hxy; Txz -= hxz; Tyz -= hyz;
+            Sxx += hxx; Syy += hyy; Szz += hzz; Sxy += hxy; Sxz += hxz; Syz += hyz;
+        }
+        // K: shear part with 1 - 1/tau, trace with 1 - s2b (0 with the paper's s2b = 1); halved
+        const float o2 = 1.0f - s2nu, h2 = 0.5f * o2, t3 = (0.5f / 3.0f) * o2;
+        const float k110 = h2 * (mo.pxy - Txy), k101 = h2 * (mo.pxz - Txz), k011 = h2 * (mo.pyz - Tyz);
+        const float e1 = t3 * (mo.dxz - (Txx - Tzz)), e2 = t3 * (mo.dyz - (Tyy - Tzz));
+        float k200 = fmaf(2.0f, e1, -e2), k020 = fmaf(2.0f, e2, -e1), k002 = -(e1 + e2);
+        if (a.s2b != 1.0f) {
+            const float ugr = fmaf(ux, grx, fmaf(uy, gry, uz * grz));
+            const float iso = fmaf(rho * oma, 9.0f / 19.0f, nu * ugr);
+            const float tr = (fmaf(3.0f, mo.pzz, mo.dxz + mo.dyz) - ((Txx + Tyy) + Tzz)) - 3.0f * iso;
+            const float t = (0.5f / 3.0f) * (1.0f - a.s2b) * tr;
+            k200 += t; k020 += t; k002 += t;
+        }
 
-    // inverse transform, z then y: half values of the lines (cy, cz) of K's moments of order 0, 1
-    // and 2 in x
-    const Axis X(ux), Y(uy), Z(uz);
-    float W0[3][3], W1[3][3], W2[3][3];
-    {
-        float V00[3], V10[3], V01[3], V20[3], V02[3], V11[3];  // [c_z + 1], moments (p, q) in (x, y)
-        // a line with halves m0 alone (order 0), m1 alone (order 1) or m2 alone (order 2)
-        auto line0 = [](const Axis &A, float m0, float (&v)[3]) {
-            const float t = A.uu * m0, o = A.u * m0;
+        // even part of the pairs: C0 + c^T Q c (off-diagonal entries doubled)
+        C0 = fmaf(rho * oma, 27.0f / 19.0f, fmaf(-1.5f * rho, usq, fmaf(-pert, g2, -1.5f * uF)));
+        const float px = pert * gpx, py = pert * gpy;
+        qxx = fmaf(4.5f, Sxx, px * gpx); qyy = fmaf(4.5f, Syy, py * gpy); qzz = fmaf(4.5f, Szz, pert * gpz * gpz);
+        qxy = fmaf(9.0f, Sxy, 2.0f * px * gpy); qxz = fmaf(9.0f, Sxz, 2.0f * px * gpz); qyz = fmaf(9.0f, Syz, 2.0f * py * gpz);
+        // odd part: (c.u) (lb + ld (c.u)^2) + 3/2 c.F
+        lb = rho * fmaf(-4.5f, usq, 3.0f);
+        ld = 4.5f * rho;
+        // recolouring: +- seg_i, seg_i = w_i/|c_i| seg0 (c_i.grad phi), seg0 = beta rho_r rho_b (27/19)
+        // (1 - alpha) / (rho |grad phi|)
+        frac_r = mo.rho_r * inv_rho;
+        frac_b = mo.rho_b * inv_rho;
+        const float seg0 = a.beta * mo.rho_r * frac_b * inv_gm * (oma * (27.0f / 19.0f));
+        sg1 = (2.0f / 27.0f) * seg0;
+        sg2 = (float)(0.70710678118654752 / 54.0) * seg0;
+        sg3 = (float)(0.57735026918962576 / 216.0) * seg0;
+        // inverse transform, z sweep; a line that has one moment only, of order 0, 1 or 2
+        const Axis Z(uz);
+        auto line0 = [&](float m0, float (&v)[3]) {
+            const float t = Z.uu * m0, o = Z.u * m0;
             v[0] = 0.5f * (t - o); v[1] = m0 - t; v[2] = 0.5f * (t + o);
         };
-        auto line1 = [](const Axis &A, float m1, float (&v)[3]) {
-            const float t = A.u2 * m1;
+        auto line1 = [&](float m1, float (&v)[3]) {
+            const float t = Z.u2 * m1;
             v[0] = 0.5f * (t - m1); v[1] = -t; v[2] = 0.5f * (t + m1);
         };
         V00[0] = 0.5f * k002; V00[1] = -k002; V00[2] = 0.5f * k002;
-        line1(Z, k101, V10);
-        line1(Z, k011, V01);
-        line0(Z, k200, V20);
-        line0(Z, k020, V02);
-        line0(Z, k110, V11);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            {
-                const float t = fmaf(Y.uu, V00[c], fmaf(Y.u2, V01[c], V02[c])), o = fmaf(Y.u, V00[c], V01[c]);
-                W0[0][c] = 0.5f * (t - o); W0[1][c] = V00[c] - t; W0[2][c] = 0.5f * (t + o);
-            }
-            {
-                const float t = fmaf(Y.uu, V10[c], Y.u2 * V11[c]), o = fmaf(Y.u, V10[c], V11[c]);
-                W1[0][c] = 0.5f * (t - o); W1[1][c] = V10[c] - t; W1[2][c] = 0.5f * (t + o);
-            }
-            {
-                const float t = Y.uu * V20[c], o = Y.u * V20[c];
-                W2[0][c] = 0.5f * (t - o); W2[1][c] = V20[c] - t; W2[2][c] = 0.5f * (t + o);
-            }
+        line1(k101, V10);
+        line1(k011, V01);
+        line0(k200, V20);
+        line0(k020, V02);
+        line0(k110, V11);
+    }
+
+    // y sweep of the plane c = c_z + 1: half the moments of order 0, 1, 2 in x of the line c_y = b - 1
+    __device__ __forceinline__ void yline(const Axis &Y, int c, float (&W0)[3], float (&W1)[3], float (&W2)[3]) const {
+        {
+            const float t = fmaf(Y.uu, V00[c], fmaf(Y.u2, V01[c], V02[c])), o = fmaf(Y.u, V00[c], V01[c]);
+            W0[0] = 0.5f * (t - o); W0[1] = V00[c] - t; W0[2] = 0.5f * (t + o);
+        }
+        {
+            const float t = fmaf(Y.uu, V10[c], Y.u2 * V11[c]), o = fmaf(Y.u, V10[c], V11[c]);
+            W1[0] = 0.5f * (t - o); W1[1] = V10[c] - t; W1[2] = 0.5f * (t + o);
+        }
+        {
+            const float t = Y.uu * V20[c], o = Y.u * V20[c];
+            W2[0] = 0.5f * (t - o); W2[1] = V20[c] - t; W2[2] = 0.5f * (t + o);
         }
     }
-    // the line (cy, cz) = (b - 1, c - 1) in x: values of K at c_x = -1, 0, +1 (full, from the halves)
-    auto xline = [&](int b, int c, float &vm, float &v0, float &vp) {
-        const float t = fmaf(X.uu, W0[b][c], fmaf(X.u2, W1[b][c], W2[b][c])), o = fmaf(X.u, W0[b][c], W1[b][c]);
+    // x sweep of a line: the values of K at c_x = -1, 0, +1
+    static __device__ __forceinline__ void xline(const Axis &X, float w0, float w1, float w2, float &vm, float &v0, float &vp) {
+        const float t = fmaf(X.uu, w0, fmaf(X.u2, w1, w2)), o = fmaf(X.u, w0, w1);
         vm = t - o;
         vp = t + o;
-        v0 = 2.0f * (W0[b][c] - t);
-    };
-    // a pair of opposite directions: the odd terms change sign
+        v0 = 2.0f * (w0 - t);
+    }
+    __device__ __forceinline__ float odd(float cu, float cF) const {
+        const float p = fmaf(ld, cu * cu, lb);
+        return kForce ? fmaf(p, cu, 1.5f * cF) : p * cu;
+    }
+    // the first (kSecond = false) or second direction of an opposite pair, of the class of i
+    template <bool kSecond>
+    __device__ __forceinline__ float2 one(int i, float ev, float cu, float cF, float cgp, float sg, float r) const {
+        const float od = odd(cu, cF), seg = sg * cgp;
+        const float s = fmaf(wgt(i), kSecond ? ev - od : ev + od, r);
+        return kSecond ? make_float2(fmaf(frac_r, s, -seg), fmaf(frac_b, s, seg))
+                       : make_float2(fmaf(frac_r, s, seg), fmaf(frac_b, s, -seg));
+    }
+};
+
+// emit(i, f) stores the populations (red, blue) f of direction i and returns them as they will be
+// read back (with a half-precision storage, rounded); the mass of the moving ones is summed from
+// those, in the association of z_class / finish_moments (lbcm_node.cuh), so that the reader of an
+// unchanged set gets the node's colour densities back exactly.
+template <bool kForce, class E>
+__device__ __forceinline__ void collide_node(const StepArgs &a, const Moments &mo, float2 gx, float2 gy, float2 gz,
+                                             E &&emit) {
+    const Collision<kForce> q(a, mo, gx, gy, gz, a.gx, a.gy, a.gz);
+    const Axis X(q.ux), Y(q.uy);
+    float W0[3][3], W1[3][3], W2[3][3];  // [c_z + 1][c_y + 1]
+#pragma unroll
+    for (int c = 0; c < 3; ++c) q.yline(Y, c, W0[c], W1[c], W2[c]);
+    auto xline = [&](int b, int c, float &vm, float &v0, float &vp) { q.xline(X, W0[c][b], W1[c][b], W2[c][b], vm, v0, vp); };
     auto pair = [&](int i, int j, float ev, float cu, float cF, float cgp, float sg, float ri, float rj, float2 &fi,
                     float2 &fj) {
-        const float t = cu * cu;
-        const float od = kForce ? fmaf(fmaf(ld, t, lb), cu, 1.5f * cF) : fmaf(ld, t, lb) * cu;
-        const float si = fmaf(wgt(i), ev + od, ri), sj = fmaf(wgt(i), ev - od, rj);
-        const float seg = sg * cgp;
-        fi = emit(i, make_float2(fmaf(frac_r, si, seg), fmaf(frac_b, si, -seg)));
-        fj = emit(j, make_float2(fmaf(frac_r, sj, -seg), fmaf(frac_b, sj, seg)));
+        fi = emit(i, q.template one<false>(i, ev, cu, cF, cgp, sg, ri));
+        fj = emit(j, q.template one<true>(i, ev, cu, cF, cgp, sg, rj));
     };
+    const float cx0 = q.C0 + q.qxx, cy0 = q.C0 + q.qyy, cz0 = q.C0 + q.qzz;
+    const float exy = cx0 + q.qyy, exz = cx0 + q.qzz, eyz = cy0 + q.qzz, exyz = exy + q.qzz;
+    const float ux = q.ux, uy = q.uy, uz = q.uz, Fx = q.Fx, Fy = q.Fy, Fz = q.Fz, gpx = q.gpx, gpy = q.gpy, gpz = q.gpz;
+    const float qxy = q.qxy, qxz = q.qxz, qyz = q.qyz, sg1 = q.sg1, sg2 = q.sg2, sg3 = q.sg3;
+
     auto add = [](float2 &acc, float2 v) { acc = __fadd2_rn(acc, v); };
     float2 s0, sp, sm;  // masses of the moving populations by c_z = 0, +1, -1, each a running sum (z_class)
     float m_, z_, p_, n_, y_, q_;
@@ -241,7 +274,64 @@ __device__ __forceinline__ void collide_node(const StepArgs &a, const Moments &m
     // (sum_i f_i^k* = rho_k), so the rest population is that mass minus the moving ones as
     // they will be read back; this equals Eqs. (33), (34) for i = 0 and keeps the FP32 rounding
     // of the lattice constants and any storage rounding from drifting the colour masses.
-    emit(0, make_float2(mo.rho_r - s.x, mo.rho_b - s.y));
+    emit(0, make_float2(q.rho_r - s.x, q.rho_b - s.y));
+}
+
+// The populations of a halo node that enter the tile beside it, put(i, f) for each of the nine: those
+// with c_y = +1 (halo_y) or c_x = +1 (halo_x) of the node mirrored in that axis when s = -1, that is,
+// the node's own ones with c_y (c_x) = s, direction i mirrored.
+template <bool kForce, class E>
+__device__ __forceinline__ void collide_halo_y(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s, E &&put) {
+    mo.jy *= s; mo.pxy *= s; mo.pyz *= s;
+    const Collision<kForce> q(a, mo, gx, make_float2(s * gy.x, s * gy.y), gz, a.gx, s * a.gy, a.gz);
+    const Axis X(q.ux), Y(q.uy);
+    float W0[3], W1[3], W2[3];
+    float m_, z_, p_;
+    const float cy0 = q.C0 + q.qyy, exy = (q.C0 + q.qxx) + q.qyy, eyz = cy0 + q.qzz, exyz = exy + q.qzz;
+    const float uxy = q.ux + q.uy, vxy = q.ux - q.uy, gxy = q.gpx + q.gpy, hxy = q.gpx - q.gpy, Fxy = q.Fx + q.Fy, Hxy = q.Fx - q.Fy;
+    const float qp = q.qxy + q.qxz, qm = q.qxy - q.qxz;
+    q.yline(Y, 1, W0, W1, W2);
+    q.xline(X, W0[2], W1[2], W2[2], m_, z_, p_);
+    put(3, q.template one<false>(3, cy0, q.uy, q.Fy, q.gpy, q.sg1, z_));
+    put(7, q.template one<false>(7, exy + q.qxy, uxy, Fxy, gxy, q.sg2, p_));
+    put(10, q.template one<true>(9, exy - q.qxy, vxy, Hxy, hxy, q.sg2, m_));
+    q.yline(Y, 2, W0, W1, W2);
+    q.xline(X, W0[2], W1[2], W2[2], m_, z_, p_);
+    put(11, q.template one<false>(11, eyz + q.qyz, q.uy + q.uz, q.Fy + q.Fz, q.gpy + q.gpz, q.sg2, z_));
+    put(19, q.template one<false>(19, exyz + (qp + q.qyz), uxy + q.uz, Fxy + q.Fz, gxy + q.gpz, q.sg3, p_));
+    put(25, q.template one<false>(25, exyz + (q.qyz - qp), q.uz - vxy, q.Fz - Hxy, q.gpz - hxy, q.sg3, m_));
+    q.yline(Y, 0, W0, W1, W2);
+    q.xline(X, W0[2], W1[2], W2[2], m_, z_, p_);
+    put(13, q.template one<false>(13, eyz - q.qyz, q.uy - q.uz, q.Fy - q.Fz, q.gpy - q.gpz, q.sg2, z_));
+    put(21, q.template one<false>(21, exyz + (qm - q.qyz), uxy - q.uz, Fxy - q.Fz, gxy - q.gpz, q.sg3, p_));
+    put(24, q.template one<true>(23, exyz - (qm + q.qyz), vxy + q.uz, Hxy + q.Fz, hxy + q.gpz, q.sg3, m_));
+}
+template <bool kForce, class E>
+__device__ __forceinline__ void collide_halo_x(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s, E &&put) {
+    mo.jx *= s; mo.pxy *= s; mo.pxz *= s;
+    const Collision<kForce> q(a, mo, make_float2(s * gx.x, s * gx.y), gy, gz, s * a.gx, a.gy, a.gz);
+    const Axis X(q.ux), Y(q.uy);
+    float W0[3], W1[3], W2[3];
+    auto xplus = [&](int b) {
+        float m_, z_, p_;
+        q.xline(X, W0[b], W1[b], W2[b], m_, z_, p_);
+        return p_;
+    };
+    const float cx0 = q.C0 + q.qxx, exy = cx0 + q.qyy, exz = cx0 + q.qzz, exyz = exy + q.qzz;
+    const float uxy = q.ux + q.uy, vxy = q.ux - q.uy, gxy = q.gpx + q.gpy, hxy = q.gpx - q.gpy, Fxy = q.Fx + q.Fy, Hxy = q.Fx - q.Fy;
+    const float qp = q.qxy + q.qxz, qm = q.qxy - q.qxz;
+    q.yline(Y, 1, W0, W1, W2);
+    put(1, q.template one<false>(1, cx0, q.ux, q.Fx, q.gpx, q.sg1, xplus(1)));
+    put(7, q.template one<false>(7, exy + q.qxy, uxy, Fxy, gxy, q.sg2, xplus(2)));
+    put(9, q.template one<false>(9, exy - q.qxy, vxy, Hxy, hxy, q.sg2, xplus(0)));
+    q.yline(Y, 2, W0, W1, W2);
+    put(15, q.template one<false>(15, exz + q.qxz, q.ux + q.uz, q.Fx + q.Fz, q.gpx + q.gpz, q.sg2, xplus(1)));
+    put(19, q.template one<false>(19, exyz + (qp + q.qyz), uxy + q.uz, Fxy + q.Fz, gxy + q.gpz, q.sg3, xplus(2)));
+    put(23, q.template one<false>(23, exyz - (qm + q.qyz), vxy + q.uz, Hxy + q.Fz, hxy + q.gpz, q.sg3, xplus(0)));
+    q.yline(Y, 0, W0, W1, W2);
+    put(17, q.template one<false>(17, exz - q.qxz, q.ux - q.uz, q.Fx - q.Fz, q.gpx - q.gpz, q.sg2, xplus(1)));
+    put(21, q.template one<false>(21, exyz + (qm - q.qyz), uxy - q.uz, Fxy - q.Fz, gxy - q.gpz, q.sg3, xplus(2)));
+    put(26, q.template one<true>(25, exyz + (q.qyz - qp), q.uz - vxy, q.Fz - Hxy, q.gpz - hxy, q.sg3, xplus(0)));
 }
 
 }  // namespace lbcm
