@@ -10,14 +10,21 @@
 // with the same bits as n gather and n collision passes.
 //
 // A block owns a 32 x TY tile of columns and a run of planes and marches along z.  Per plane k:
-//   collide  each thread takes one node of the tile and its one-node halo in x and y, from the
-//            prefetched moments and a ring of phase planes in shared memory, and writes its 27
-//            population pairs to shared memory;
+//   collide  a warp takes a row of the tile, its halo rows or its halo columns (of which only the nine
+//            populations that enter the tile are built), from prefetched moments and the gradients,
+//            and writes the populations to shared memory;
+//   gradient of plane k + 1, from a ring of four phase planes in shared memory, while other warps are
+//            still colliding;
 //   gather   each thread of the tile reads the 27 pulls that come from plane k: c_z = -1 completes
 //            the node of plane k - 1, c_z = 0 is joined to plane k, c_z = +1 starts plane k + 1
-//            (z_class, join_classes, finish_moments; 20 registers hold the two open planes).
-// The halo is collided again by every block that needs it (1.2 times the nodes for TY = 14), which
-// costs arithmetic and no population traffic.
+//            (z_class, join_classes, finish_moments; 22 registers hold the two open planes).
+// What bounds it: instruction issue and the shared-memory pipe, in turn rather than together (issue
+// slots 61%, FMA pipe 49%, shared memory 49% of the time; DRAM 103 bytes a node, a quarter of its
+// bandwidth), because the warps of a block go through the same phase at the same time.  Tried on
+// 256 x 256 x 512, G nodes/s: 32 x 16 tile, 20 warps, a barrier after each phase 19.2; halo warps of
+// their own 20.2; gradient moved between arriving at and waiting on the first barrier, the scalar
+// part of the collision before the second 22.4; both barriers split in two halves 21.5.  Two
+// population buffers and one barrier (32 x 11, 14 warps) 16.3 when the first form had 17.2.
 #include <algorithm>
 #include <type_traits>
 
@@ -38,7 +45,8 @@ struct AdvanceTile {
     static constexpr int kMom = (27 * NB * (int)sizeof(float2) + 15) / 16 * 16;
     static constexpr int kRing = kMom + 3 * NT * (int)sizeof(float4);
     static constexpr int kInflow = kRing + 4 * NR * (int)sizeof(float2);
-    static constexpr int kBytes = kInflow + NB * (int)sizeof(float4);
+    static constexpr int kBar = kInflow + NB * (int)sizeof(float4);
+    static constexpr int kBytes = kBar + 16;
     static_assert(kBytes <= 227 * 1024 && NR <= 2 * NT, "shared memory layout");
 };
 
@@ -51,6 +59,34 @@ __device__ __forceinline__ void cp_async(unsigned smem, const void *gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Barrier of the block's warps in two halves: a warp arrives when it has written what it shares, goes
+// on with work of its own and waits when it needs the others'.  The wait is bounded; a wait that runs
+// out (none does while every warp arrives once a phase) sets *err and goes on.
+__device__ __forceinline__ void warps_init(unsigned bar, int warps) {
+    asm volatile("mbarrier.init.shared.b64 [%0], %1;\n" ::"r"(bar), "r"(warps) : "memory");
+}
+__device__ __forceinline__ void warps_arrive(unsigned bar) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void warps_wait(unsigned bar, int phase, int *err) {
+    for (int n = 0; n < (1 << 22); ++n) {
+        unsigned done;
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                     : "=r"(done)
+                     : "r"(bar), "r"(phase & 1)
+                     : "memory");
+        if (done) return;
+    }
+    *err = 1;
+}
+
+// Barrier of the whole block that the warps may reach at different places of the code.
+template <int NT>
+__device__ __forceinline__ void block_sync() {
+    asm volatile("barrier.sync 1, %0;\n" ::"n"(NT) : "memory");
+}
 
 __device__ __forceinline__ int pmod(int a, int n) {
     const int r = a % n;
@@ -126,11 +162,14 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
 
     fill_ring(kb - 1, plane_of(kb - 1));
     fill_ring(kb, plane_of(kb));
-    int zr = plane_of(kb + 1);  // the last plane in the ring
-    fill_ring(kb + 1, zr);
+    fill_ring(kb + 1, plane_of(kb + 1));
+    int zr = plane_after(plane_of(kb + 1));  // the last plane in the ring
+    fill_ring(kb + 2, zr);
     int zm = plane_of(kb);      // the plane whose moments are here or on their way
     fetch_moments(zm);
     cp_async_commit();
+    const unsigned bar_full = (unsigned)__cvta_generic_to_shared(smem + T::kBar);
+    if (t == 0) warps_init(bar_full, NT / 32);
     cp_async_wait();
     if (!pz && kb == 0 && a.bc_zlo == BC_INLET) {  // ghost plane z = -1 inside the inlet disc (own entries)
         float2 *g = ring + 3 * T::NR;
@@ -148,43 +187,42 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
     }
     __syncthreads();
 
-    // collides plane k; the rest population of a node of the tile stays with its thread
-    auto collide = [&](int k, float2 &rest) {
-        float2 *out = reinterpret_cast<float2 *>(smem) + pos;
-        const float4 *m = mb + t;
-        const Moments mo = unpack_moments(m[0], m[NT], m[2 * NT]);
+    // gradients of plane k's node from ring planes k - 1, k, k + 1
+    float2 gx, gy, gz;
+    auto gradient = [&](int k) {
         const float2 *r[3] = {ring + ((k - 1) & 3) * T::NR + rpos, ring + (k & 3) * T::NR + rpos,
                              ring + ((k + 1) & 3) * T::NR + rpos};
-        float2 gx, gy, gz;
         gradients([&](int j) { return r[cz(j) + 1][cy(j) * RX + cx(j)]; }, gx, gy, gz);
         if (a.grad4 && inside && k >= z0 && (k < z1 || top)) {
             a.grad4[k * P + cxy] = make_float4(gx.x, gy.x, gz.x, gx.y);
             a.grad2[k * P + cxy] = make_float2(gy.y, gz.y);
         }
-        // once the record is in registers its place takes the next plane's
-        auto fetch = [&](int i, int first) {
-            if (i == first && k < ke) fetch_moments(plane_after(zm));
+    };
+    // collides plane k; the rest population of a node of the tile stays with its thread
+    auto collide = [&](int k, float2 &rest) {
+        float2 *out = reinterpret_cast<float2 *>(smem) + pos;
+        const float4 *m = mb + t;
+        const Moments mo = unpack_moments(m[0], m[NT], m[2 * NT]);
+        // the record is in registers: its place takes the next plane's; the populations' place is free
+        // once every warp has gathered plane k - 1
+        auto ready = [&] {
+            if (k < ke) fetch_moments(plane_after(zm));
+            if (k > kb) block_sync<NT>();
         };
-        if (row) {
+        if (row)
             collide_node<kForce>(a, mo, gx, gy, gz, [&](int i, float2 f) {
                 if (i == 0)
                     rest = f;
                 else
                     out[i * NB] = f;
-                fetch(i, 1);
                 return f;
-            });
-        } else if (halo_y) {
-            collide_halo_y<kForce>(a, mo, gx, gy, gz, side, [&](int i, float2 f) {
-                out[(side > 0.0f ? i : flip_y(i)) * NB] = f;
-                fetch(i, 3);
-            });
-        } else {
-            collide_halo_x<kForce>(a, mo, gx, gy, gz, side, [&](int i, float2 f) {
-                out[(side > 0.0f ? i : flip_x(i)) * NB] = f;
-                fetch(i, 1);
-            });
-        }
+            }, ready);
+        else if (halo_y)
+            collide_halo_y<kForce>(a, mo, gx, gy, gz, side,
+                                   [&](int i, float2 f) { out[(side > 0.0f ? i : flip_y(i)) * NB] = f; }, ready);
+        else
+            collide_halo_x<kForce>(a, mo, gx, gy, gz, side,
+                                   [&](int i, float2 f) { out[(side > 0.0f ? i : flip_x(i)) * NB] = f; }, ready);
     };
 
     ZClass up{};      // class c_z = +1 of plane k + 1
@@ -233,14 +271,21 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
         up = z_class<1>(at);
         if (top && !conv && k == N) write_out(N, finish_moments(a, open, z_class<-1>(mirrored)));
     };
+    if (collider) gradient(kb);
+    __syncthreads();  // the first refill of the ring takes the place of plane kb - 1
     for (int k = kb; k <= ke; ++k) {
-        zr = plane_after(zr);
-        if (k < ke) fill_ring(k + 2, zr);
         float2 rest;
-        if (collider) collide(k, rest);
+        if (collider)
+            collide(k, rest);
+        else if (k > kb)  // no warp runs ahead of the ring's readers
+            block_sync<NT>();
+        warps_arrive(bar_full);
         zm = plane_after(zm);
+        zr = plane_after(zr);
+        if (k + 2 <= ke) fill_ring(k + 3, zr);  // over plane k - 1, whose last reader was gradient(k)
         cp_async_commit();
-        __syncthreads();
+        if (collider && k < ke) gradient(k + 1);
+        warps_wait(bar_full, k - kb, v.err);
         if (inside) {
             if (W && walled)
                 gather(k, rest, std::true_type{});
@@ -248,7 +293,6 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
                 gather(k, rest, std::false_type{});
         }
         cp_async_wait();
-        __syncthreads();
     }
     if (top && conv && inside) {  // f(N, t + 1) from f(N - 1, t + 1) and f(N, t)
         const size_t p = (size_t)P;
@@ -303,11 +347,11 @@ static cudaError_t launch_ty(const StepArgs &a, const AdvanceArgs &v, int chunks
 constexpr int kSMs = 152;
 
 // Which tile and how many runs of planes: the estimated time of the last wave's end, with the
-// measured time a plane takes a resident block (us, 256 x 256 x 512 periodic, FP32): 3.66 for the
-// 32 x 16 tile (one block of 20 warps on an SM), 3.28 for the 32 x 7 tile (two blocks of 10 warps;
-// 2.0 when a block has the SM to itself).  Both reach 19 G nodes/s on large lattices; the small tile
-// wastes less on planes that are no multiple of 16 rows and fills the chip with fewer columns.  A run
-// collides one plane more at each end, and about 8 us go into filling and draining it.
+// measured time a plane takes a resident block (us, 256 x 256 x 512 periodic, FP32): 3.15 for the
+// 32 x 16 tile (one block of 20 warps on an SM), 3.1 for the 32 x 7 tile (two blocks of 10 warps;
+// 1.9 when a block has the SM to itself).  They reach 22 and 20 G nodes/s on large lattices; the small
+// tile wastes less on planes that are no multiple of 16 rows and fills the chip with fewer columns.  A
+// run collides one plane more at each end, and about 12 us go into filling and draining it.
 AdvancePlan plan_advance(const StepArgs &a) {
     const int planes = a.bc_zhi == BC_CONVECTIVE ? a.nz - 1 : a.nz;
     AdvancePlan best{0, 1, 1e30f};
@@ -315,8 +359,8 @@ AdvancePlan plan_advance(const StepArgs &a) {
         const long long tiles = (long long)((a.nx + 31) / 32) * ((a.ny + ty - 1) / ty);
         for (int chunks = 1; chunks <= planes && chunks <= 4 * kSMs; ++chunks) {
             const long long blocks = tiles * chunks, slots = ty == 16 ? kSMs : 2 * kSMs;
-            const float plane_us = ty == 16 ? 3.66f : (blocks <= kSMs ? 2.0f : 3.28f);
-            const float us = (float)((blocks + slots - 1) / slots) * (float)((planes + chunks - 1) / chunks + 2) * plane_us + 8.0f;
+            const float plane_us = ty == 16 ? 3.15f : (blocks <= kSMs ? 1.9f : 3.1f);
+            const float us = (float)((blocks + slots - 1) / slots) * (float)((planes + chunks - 1) / chunks + 2) * plane_us + 12.0f;
             if (us < best.us) best = AdvancePlan{ty, chunks, us};
         }
     }

@@ -558,7 +558,7 @@ lb_status run_mass(lb_ctx *c, double out[2], int z0 = 0, int z1 = -1) {
     LB_CUDA(cudaStreamSynchronize(c->stream));
     if (err) {
         cudaMemsetAsync(c->ferr, 0, sizeof(int), c->stream);
-        return fail(LB_ETIMEOUT, "a wait of the fused step kernel ran out: the state is not to be trusted");
+        return fail(LB_ETIMEOUT, "a wait inside a step kernel ran out: the state is not to be trusted");
     }
     return LB_OK;
 }
@@ -984,6 +984,7 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
         v.mom_out[0] = mom[out];
         v.phase = phase[in];
         v.phase_out = phase[out];
+        v.err = c->ferr;
         ev = profile_record(c, s == n - 1 ? PROF_ADVANCE_COLLIDE : PROF_ADVANCE);
         if (ev) cudaEventRecord(ev[0], c->stream);
         e = launch_advance(a, plan, v, c->stream, &c->launches);

@@ -207,10 +207,12 @@ struct Collision {
 // read back (with a half-precision storage, rounded); the mass of the moving ones is summed from
 // those, in the association of z_class / finish_moments (lbcm_node.cuh), so that the reader of an
 // unchanged set gets the node's colour densities back exactly.
-template <bool kForce, class E>
+// ready() is called once, when the moments have been used and nothing has been emitted yet.
+template <bool kForce, class E, class R>
 __device__ __forceinline__ void collide_node(const StepArgs &a, const Moments &mo, float2 gx, float2 gy, float2 gz,
-                                             E &&emit) {
+                                             E &&emit, R &&ready) {
     const Collision<kForce> q(a, mo, gx, gy, gz, a.gx, a.gy, a.gz);
+    ready();
     const Axis X(q.ux), Y(q.uy);
     float W0[3][3], W1[3][3], W2[3][3];  // [c_z + 1][c_y + 1]
 #pragma unroll
@@ -280,10 +282,12 @@ __device__ __forceinline__ void collide_node(const StepArgs &a, const Moments &m
 // The populations of a halo node that enter the tile beside it, put(i, f) for each of the nine: those
 // with c_y = +1 (halo_y) or c_x = +1 (halo_x) of the node mirrored in that axis when s = -1, that is,
 // the node's own ones with c_y (c_x) = s, direction i mirrored.
-template <bool kForce, class E>
-__device__ __forceinline__ void collide_halo_y(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s, E &&put) {
+template <bool kForce, class E, class R>
+__device__ __forceinline__ void collide_halo_y(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s,
+                                               E &&put, R &&ready) {
     mo.jy *= s; mo.pxy *= s; mo.pyz *= s;
     const Collision<kForce> q(a, mo, gx, make_float2(s * gy.x, s * gy.y), gz, a.gx, s * a.gy, a.gz);
+    ready();
     const Axis X(q.ux), Y(q.uy);
     float W0[3], W1[3], W2[3];
     float m_, z_, p_;
@@ -306,10 +310,12 @@ __device__ __forceinline__ void collide_halo_y(const StepArgs &a, Moments mo, fl
     put(21, q.template one<false>(21, exyz + (qm - q.qyz), uxy - q.uz, Fxy - q.Fz, gxy - q.gpz, q.sg3, p_));
     put(24, q.template one<true>(23, exyz - (qm + q.qyz), vxy + q.uz, Hxy + q.Fz, hxy + q.gpz, q.sg3, m_));
 }
-template <bool kForce, class E>
-__device__ __forceinline__ void collide_halo_x(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s, E &&put) {
+template <bool kForce, class E, class R>
+__device__ __forceinline__ void collide_halo_x(const StepArgs &a, Moments mo, float2 gx, float2 gy, float2 gz, float s,
+                                               E &&put, R &&ready) {
     mo.jx *= s; mo.pxy *= s; mo.pxz *= s;
     const Collision<kForce> q(a, mo, make_float2(s * gx.x, s * gx.y), gy, gz, s * a.gx, a.gy, a.gz);
+    ready();
     const Axis X(q.ux), Y(q.uy);
     float W0[3], W1[3], W2[3];
     auto xplus = [&](int b) {

@@ -23,6 +23,7 @@ struct AdvanceArgs {
     const float2 *phase;
     float4 *mom_out[3];
     float2 *phase_out;
+    int *err;              // set if a wait inside the kernel ran out
     int tiles_x, tiles, planes, chunks;  // set by the launcher: column tiles, planes marched, runs of planes
 };
 // Tile rows and runs of planes of an advance, and its estimated time (us).

@@ -297,7 +297,7 @@ __device__ __forceinline__ void collide_at(const StepArgs &a, int x, int y, int 
     }
     collide_node<kForce>(a, mo, gx, gy, gz, [&](int i, float2 f) {
         return store_pop<S>(a, i, nb.n, f, S == STORE_FP32 || i == 0 ? no_shift() : dest_shift<S>(a, nb, i));
-    });
+    }, [] {});
 }
 
 template <bool kForce, int S, bool kRec>
