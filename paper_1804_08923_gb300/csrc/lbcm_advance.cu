@@ -95,6 +95,7 @@ __device__ __forceinline__ int pmod(int a, int n) {
 
 template <bool kForce, bool W, int TY, int MB>
 __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepArgs a, AdvanceArgs v) {
+    chain_begin();
     using T = AdvanceTile<TY>;
     constexpr int BX = T::BX, RX = T::RX, NB = T::NB, NT = T::NT;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -332,8 +333,7 @@ static cudaError_t launch_tile(const StepArgs &a, AdvanceArgs v, int chunks, cud
         v.mom[q] = v.mom[0] + q * a.NN;
         v.mom_out[q] = v.mom_out[0] + q * a.NN;
     }
-    fn<<<(unsigned)v.tiles * v.chunks, T::NT, T::kBytes, s>>>(a, v);
-    return cudaGetLastError();
+    return launch_chained(fn, dim3((unsigned)v.tiles * v.chunks), dim3(T::NT), T::kBytes, s, a, v);
 }
 
 template <int TY, int MB>

@@ -948,15 +948,15 @@ static cudaEvent_t *profile_record(lb_ctx *c, ProfKind kind) {
 // Whether several steps of one call go from moment record to moment record (lbcm_advance.cu) instead
 // of through the populations: the paper's rates, FP32 storage and the default step kernel, where an
 // advance is estimated faster than the two passes it replaces.  Those run at 12.7 G nodes/s on large
-// lattices and take 7.5 us on the smallest (two dependent launches; 32^3: 10.3 us in all, against
-// 14 us for an advance, whose blocks collide three planes for each that they own), 4 us more where
+// lattices and take 6 us on the smallest (two dependent launches; 32^3: 8.5 us in all, against
+// 14 us for an advance, whose blocks collide three planes for each that they own), 3 us more where
 // boundary planes are computed first.
 static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
     const lb_params &p = c->p;
     if (p.step_kernel != 0 || p.storage != LB_STORE_FP32 || p.s3 != 1.0 || p.s4 != 1.0 || p.s5 != 1.0 || p.s6 != 1.0) return false;
     *plan = plan_advance(a);
     const bool planes = c->g.bc_zlo != LB_BC_PERIODIC || c->g.bc_zhi != LB_BC_PERIODIC;
-    return plan->us < 7.5f + (planes ? 4.0f : 0.0f) + 7.87e-5f * (float)c->nn;
+    return plan->us < 6.0f + (planes ? 3.0f : 0.0f) + 7.87e-5f * (float)c->nn;
 }
 
 // n >= 2 steps: one gather pass, n - 1 advances, one collision pass.  Moment records and phase entries

@@ -476,6 +476,14 @@ __device__ __forceinline__ float2 fit_even(const StepArgs &a, float rr, float rb
     return make_float2(rr * oma, rb * oma);
 }
 
+// First statement of every kernel of a step: lets the next kernel of the stream be scheduled while
+// this one runs (launch_chained, lbcm_internal.h), and waits until the kernel before it has completed
+// and its writes are visible.  Nothing is read or written before.
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
 // 32-bit offsets of the node and of its three neighbouring columns, rows and planes:

@@ -4,6 +4,25 @@
 #include "lbcm_device.cuh"
 
 namespace lbcm {
+// Launches a kernel that begins with chain_begin(): its blocks may be scheduled as the kernel before
+// it in the stream drains, and wait there for its completion.  What it saves is the gap between two
+// dependent kernels: 32^3 droplet 10.3 -> 8.5 us a step (two launches), 45 x 37 x 53 box 14.4 -> 10.5,
+// 96 x 96 x 384 jet 182 -> 179 (one advance).
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, fn, args...);
+}
+
 // One time step (boundary planes, gather pass, collision) on stream s, for population storage
 // STORE_FP32, STORE_FP16 or STORE_FP16_FIT.  passes selects PASS_GATHER (boundary planes and the
 // gather pass: phase field and collision moments), PASS_COLLIDE (the collision, which writes

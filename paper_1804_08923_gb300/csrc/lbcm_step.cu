@@ -46,6 +46,7 @@ namespace lbcm {
 // kColumnKernelPlane columns.
 template <int S>
 __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const long long col = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (col >= a.plane) return;  // whole warps leave together
@@ -121,6 +122,7 @@ __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
 constexpr long long kColumnKernelPlane = 24576;
 template <int S>
 __global__ void __launch_bounds__(128) boundary_column_kernel(StepArgs a) {
+    chain_begin();
     const long long col = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (col >= a.plane) return;
     const int x = (int)(col % a.nx), y = (int)(col / a.nx);
@@ -206,9 +208,9 @@ __global__ void __launch_bounds__(128) boundary_column_kernel(StepArgs a) {
 template <int S>
 static void launch_boundary(const StepArgs &a, cudaStream_t s) {
     if (a.plane >= kColumnKernelPlane)
-        boundary_column_kernel<S><<<(unsigned)((a.plane + 127) / 128), 128, 0, s>>>(a);
+        launch_chained(boundary_column_kernel<S>, dim3((unsigned)((a.plane + 127) / 128)), dim3(128), 0, s, a);
     else
-        boundary_plane_kernel<S><<<(unsigned)((a.plane + 3) / 4), 128, 0, s>>>(a);
+        launch_chained(boundary_plane_kernel<S>, dim3((unsigned)((a.plane + 3) / 4)), dim3(128), 0, s, a);
 }
 
 // ------------------------------------------- moment pass (K_A with the paper's rates)
@@ -249,10 +251,12 @@ __device__ __forceinline__ void moment_node(const StepArgs &a) {
 
 template <int S, bool W>
 __global__ void __launch_bounds__(128) moment_kernel(StepArgs a) {
+    chain_begin();
     moment_node<S, W>(a);
 }
 template <int S>
 __global__ void __launch_bounds__(128, S == STORE_FP16_FIT ? 5 : 1) moment_wall_kernel(StepArgs a) {
+    chain_begin();
     moment_node<S, true>(a);
 }
 
@@ -302,6 +306,7 @@ __device__ __forceinline__ void collide_at(const StepArgs &a, int x, int y, int 
 
 template <bool kForce, int S, bool kRec>
 __global__ void __launch_bounds__(128, (S == STORE_FP32 ? 6 : (S == STORE_FP16 ? 5 : 4))) collide_kernel(StepArgs a) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z + a.z_base;
@@ -437,9 +442,9 @@ static void launch_step_sw(const StepArgs &a, cudaStream_t s, cudaEvent_t *ev, l
         // paper's rates let the collision work from them)
         if (paper_rates) {
             if constexpr (W && S != STORE_FP32)
-                moment_wall_kernel<S><<<grd, blk, 0, s>>>(a);
+                launch_chained(moment_wall_kernel<S>, grd, blk, 0, s, a);
             else
-                moment_kernel<S, W><<<grd, blk, 0, s>>>(a);
+                launch_chained(moment_kernel<S, W>, grd, blk, 0, s, a);
         } else {
             launch_general_gather(a, S, s);
         }
@@ -453,13 +458,13 @@ static void launch_step_sw(const StepArgs &a, cudaStream_t s, cudaEvent_t *ev, l
     if (!paper_rates)
         launch_general_collide(a, S, s);
     else if (rec && force)
-        collide_kernel<true, S, S == STORE_FP32><<<grd, blk, 0, s>>>(a);
+        launch_chained(collide_kernel<true, S, S == STORE_FP32>, grd, blk, 0, s, a);
     else if (rec)
-        collide_kernel<false, S, S == STORE_FP32><<<grd, blk, 0, s>>>(a);
+        launch_chained(collide_kernel<false, S, S == STORE_FP32>, grd, blk, 0, s, a);
     else if (force)
-        collide_kernel<true, S, false><<<grd, blk, 0, s>>>(a);
+        launch_chained(collide_kernel<true, S, false>, grd, blk, 0, s, a);
     else
-        collide_kernel<false, S, false><<<grd, blk, 0, s>>>(a);
+        launch_chained(collide_kernel<false, S, false>, grd, blk, 0, s, a);
     if (ev) cudaEventRecord(ev[3], s);
     *launches += 1;
 }
