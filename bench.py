@@ -317,7 +317,7 @@ def run_reference(args, cfg):
 
 
 def adjoint_leg(lb, torch, name="jet64", T=500, objective="area", args=(1e-3,), checkpoint=0):
-    """Cost of lb_adjoint (T steps forward with ceil(sqrt T) checkpoints, objective, reverse
+    """Cost of lb_adjoint (T steps forward, every step recorded or with ceil(sqrt T) checkpoints, objective, reverse
     sweep) against lb_step(T) from the same state, both timed with CUDA events."""
     cfg = workloads.CONFIGS[name]
     nx, ny, nz = cfg["grid"]

@@ -524,6 +524,7 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
 #endif
 template <bool kForce, bool W>
 __global__ void __launch_bounds__(128, LBCM_ADJ_MIN_BLOCKS) adj_collide_kernel(StepArgs a, AdjArgs g) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -577,6 +578,7 @@ __device__ __forceinline__ void adj_stencil_sums(const StepArgs &a, const AdjArg
 
 template <bool W>
 __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -610,6 +612,7 @@ __device__ __forceinline__ float warp_sum(float v) {
 }
 
 __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g) {
+    chain_begin();
     const int lane = threadIdx.x & 31;
     const long long col = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     float part[17];
@@ -860,20 +863,20 @@ cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_
     }
     const dim3 gr = node_grid(a), bl = node_block();
     if (force && walls)
-        adj_collide_kernel<true, true><<<gr, bl, kAdjSmem, s>>>(a, g);
+        launch_chained(adj_collide_kernel<true, true>, gr, bl, kAdjSmem, s, a, g);
     else if (force)
-        adj_collide_kernel<true, false><<<gr, bl, kAdjSmem, s>>>(a, g);
+        launch_chained(adj_collide_kernel<true, false>, gr, bl, kAdjSmem, s, a, g);
     else if (walls)
-        adj_collide_kernel<false, true><<<gr, bl, kAdjSmem, s>>>(a, g);
+        launch_chained(adj_collide_kernel<false, true>, gr, bl, kAdjSmem, s, a, g);
     else
-        adj_collide_kernel<false, false><<<gr, bl, kAdjSmem, s>>>(a, g);
+        launch_chained(adj_collide_kernel<false, false>, gr, bl, kAdjSmem, s, a, g);
     if (walls)
-        adj_stencil_kernel<true><<<gr, bl, 0, s>>>(a, g);
+        launch_chained(adj_stencil_kernel<true>, gr, bl, 0, s, a, g);
     else
-        adj_stencil_kernel<false><<<gr, bl, 0, s>>>(a, g);
+        launch_chained(adj_stencil_kernel<false>, gr, bl, 0, s, a, g);
     *launches += 2;
     if (a.bc_zlo == BC_INLET || a.bc_zhi == BC_CONVECTIVE) {
-        adj_boundary_kernel<<<col_grid(a), col_block(), 0, s>>>(a, g);
+        launch_chained(adj_boundary_kernel, col_grid(a), col_block(), 0, s, a, g);
         *launches += 1;
     }
     return cudaGetLastError();

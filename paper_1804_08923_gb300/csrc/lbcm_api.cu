@@ -160,7 +160,8 @@ struct lb_ctx {
     struct {
         void *base = nullptr;
         size_t bytes = 0;
-        float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lp[2] = {}, *lr[2] = {}, *lgb = nullptr, *objph = nullptr;
+        float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lp[2] = {}, *lr[2] = {}, *lgb = nullptr, *objph = nullptr,
+               *phase2 = nullptr;
         float *ckpt_hist = nullptr, *seg_fm[2] = {}, *seg_hist[2] = {}, *lc = nullptr, *li = nullptr, *lh[2] = {};
         float4 *lga = nullptr, *seg_mom[2] = {}, *seg_g4[2] = {};
         float2 *seg_g2[2] = {};
@@ -815,11 +816,8 @@ static lb_status prepare_fused(lb_ctx *c, const StepArgs &a) {
     return LB_OK;
 }
 
-// The end of a step: the state now at t+1, and the periodic mass check.
-static lb_status finish_step(lb_ctx *c) {
-    c->cur ^= 1;
-    if (c->g.bc_zhi == LB_BC_CONVECTIVE) c->hcur ^= 1;
-    c->step += 1;
+// The periodic mass check of the state at c->step.
+static lb_status check_step(lb_ctx *c) {
     if (c->p.check_every > 0 && c->step % c->p.check_every == 0) {
         double m[2];
         lb_status st = run_mass(c, m);
@@ -828,6 +826,14 @@ static lb_status finish_step(lb_ctx *c) {
             return fail(LB_EUNSTABLE, "non-finite colour mass at step " + std::to_string(c->step));
     }
     return LB_OK;
+}
+
+// The end of a step: the state now at t+1, and the periodic mass check.
+static lb_status finish_step(lb_ctx *c) {
+    c->cur ^= 1;
+    if (c->g.bc_zhi == LB_BC_CONVECTIVE) c->hcur ^= 1;
+    c->step += 1;
+    return check_step(c);
 }
 
 lb_status lb_step_gather(lb_ctx *c) {
@@ -997,10 +1003,23 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
     a.pout = c->pop[dst];
     e = launch_step(a, c->p.storage, c->stream, ev, &c->launches, PASS_COLLIDE);
     if (e != cudaSuccess) return cuda_fail(e, "launch_step (collide)");
-    c->cur = dst ^ 1;  // finish_step flips these for the last step
-    if (conv) c->hcur ^= (int)((n - 1) & 1);
-    c->step += n - 1;
-    return finish_step(c);
+    c->cur = dst;
+    if (conv) c->hcur ^= (int)(n & 1);
+    c->step += n;
+    return LB_OK;
+}
+
+// n steps by advances (plan not NULL, n >= 2) or one by one in two passes, without mass checks.
+static lb_status steps_unchecked(lb_ctx *c, const AdvancePlan *plan, int64_t n) {
+    if (plan && n >= 2) return advance_steps(c, *plan, n);
+    for (int64_t s = 0; s < n; ++s) {
+        cudaError_t e = launch_step(make_args(c), c->p.storage, c->stream, nullptr, &c->launches);
+        if (e != cudaSuccess) return cuda_fail(e, "launch_step");
+        c->cur ^= 1;
+        if (c->g.bc_zhi == LB_BC_CONVECTIVE) c->hcur ^= 1;
+        c->step += 1;
+    }
+    return LB_OK;
 }
 
 lb_status lb_step(lb_ctx *c, int64_t n) {
@@ -1015,6 +1034,7 @@ lb_status lb_step(lb_ctx *c, int64_t n) {
             const int64_t m = c->p.check_every > 0 ? std::min<int64_t>(n - s, c->p.check_every - c->step % c->p.check_every) : n - s;
             if (m >= 2) {
                 lb_status st = advance_steps(c, plan, m);
+                if (st == LB_OK) st = check_step(c);
                 if (st != LB_OK) return st;
                 s += m;
                 continue;
@@ -1290,46 +1310,72 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         return fail(LB_EINVAL, "unknown objective");
     }
     if (obj_args[2] < 0) return fail(LB_EINVAL, "checkpoint interval obj_args[2] must be >= 0");
-    long long k = obj_args[2] >= 1 ? (long long)obj_args[2] : (long long)std::ceil(std::sqrt((double)T));
-    k = std::max(1ll, std::min<long long>(k, T));
-    const long long nseg = (T + k - 1) / k;
 
     // workspace: checkpoints every k steps; two sets of per-step records (one segment is
     // recomputed into one set while the reverse sweep steps back through the other); the
-    // adjoint state
+    // adjoint state.  Per recorded step: the collision inputs (the moment pass's 48 B and the 24 B
+    // of gradients a node), f(N-1) and hist(n+1) of the outflow plane; the recomputed populations
+    // themselves only in two alternating buffers.  With a single segment (k = T) the forward pass
+    // records every step, and checkpoints, the second set and those buffers drop out.
     const size_t NN = (size_t)c->nn, P = (size_t)c->plane;
     const size_t pb = 27 * NN * sizeof(float2), hb = 54 * P * sizeof(float), nb2 = NN * sizeof(float2);
     StepArgs a0 = make_args(c);
     const long long nblk_coll = adj_collide_blocks(a0), nblk_inlet = adj_boundary_blocks(a0);
-    // per recorded step: the collision inputs (the moment pass's 48 B and the 24 B of gradients
-    // a node), f(N-1) and hist(n+1) of the outflow plane; the recomputed populations
-    // themselves only in two alternating buffers
-    const size_t rmom = k * 3 * NN * sizeof(float4), rg4 = k * NN * sizeof(float4), rg2 = k * nb2, rfm = k * hb,
-                 rhist = (k + 1) * hb;
-    const size_t parts[] = {nseg * pb, nseg * hb, 2 * pb, rmom, rg4, rg2, rfm, rhist, rmom, rg4, rg2, rfm, rhist,
-                            pb, pb, nb2, nb2, NN * sizeof(float4), nb2, hb, 9 * P * sizeof(float), hb, hb,
-                            nblk_coll * 3 * sizeof(double), nblk_inlet * 17 * sizeof(double),
-                            nblk_coll * sizeof(double), 32 * sizeof(double), nb2};
-    constexpr int kParts = (int)(sizeof(parts) / sizeof(parts[0]));
-    size_t need = 0;
-    for (size_t v : parts) need += align_up(v);
-    if (need > c->adj.bytes) {
+    constexpr int kParts = 29;
+    auto layout = [&](long long k, size_t (&parts)[kParts]) {
+        const long long nseg = (T + k - 1) / k;
+        const size_t one = nseg > 1 ? 1 : 0, ku = (size_t)k;
+        const size_t rec[5] = {ku * 3 * NN * sizeof(float4), ku * NN * sizeof(float4), ku * nb2, ku * hb, (ku + 1) * hb};
+        const size_t v[kParts] = {one * nseg * pb, one * nseg * hb, one * 2 * pb,
+                                  rec[0], rec[1], rec[2], rec[3], rec[4],
+                                  one * rec[0], one * rec[1], one * rec[2], one * rec[3], one * rec[4],
+                                  pb, pb, nb2, nb2, NN * sizeof(float4), nb2, hb, 9 * P * sizeof(float), hb, hb,
+                                  nblk_coll * 3 * sizeof(double), nblk_inlet * 17 * sizeof(double),
+                                  nblk_coll * sizeof(double), 32 * sizeof(double), nb2, nb2};
+        size_t need = 0;
+        for (int q = 0; q < kParts; ++q) need += align_up(parts[q] = v[q]);
+        return need;
+    };
+    size_t parts[kParts];
+    auto allocate = [&](size_t need) {
+        if (need <= c->adj.bytes) return true;
         if (c->adj.base) cudaFree(c->adj.base);
         c->adj.base = nullptr;
         c->adj.bytes = 0;
         c->adj.valid = false;
         if (cudaMalloc(&c->adj.base, need) != cudaSuccess) {
             cudaGetLastError();
-            return fail(LB_ENOMEM, "cannot allocate the adjoint workspace (" + std::to_string(need >> 20) + " MiB)");
+            c->adj.base = nullptr;
+            return false;
         }
         c->adj.bytes = need;
+        return true;
+    };
+    // k = 0: every step recorded where that takes no more than an eighth of the free device memory
+    // (what a previous call left allocated counts as free), else ceil(sqrt(T)).  The recompute that this
+    // saves costs as much as the forward pass; run beside the reverse sweep it hid nothing (64x64x256
+    // jet, 50 steps: 20.2 ms with it).
+    long long k = obj_args[2] >= 1 ? std::min<long long>((long long)obj_args[2], T) : 0;
+    bool have = false;
+    if (k == 0) {
+        size_t free_b = 0, total_b = 0;
+        LB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        const size_t all = layout(T, parts);
+        have = all <= (free_b + c->adj.bytes) / 8 && allocate(all);
+        k = have ? T : std::max(1ll, std::min<long long>((long long)std::ceil(std::sqrt((double)T)), T));
+    }
+    const long long nseg = (T + k - 1) / k;
+    if (!have) {
+        const size_t need = layout(k, parts);
+        if (!allocate(need)) return fail(LB_ENOMEM, "cannot allocate the adjoint workspace (" + std::to_string(need >> 20) + " MiB)");
     }
     {
         char *p = (char *)c->adj.base;
-        size_t j = 0;
-        auto take = [&](void *&dst) { dst = p; p += align_up(parts[j++]); };
         void *v[kParts];
-        for (int q = 0; q < kParts; ++q) take(v[q]);
+        for (int q = 0; q < kParts; ++q) {
+            v[q] = p;
+            p += align_up(parts[q]);
+        }
         auto &w = c->adj;
         w.ckpt_pop = (float2 *)v[0]; w.ckpt_hist = (float *)v[1]; w.seg_pop = (float2 *)v[2];
         for (int r = 0; r < 2; ++r) {
@@ -1341,7 +1387,7 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         w.lr[1] = (float2 *)v[16]; w.lga = (float4 *)v[17]; w.lgb = (float2 *)v[18]; w.lc = (float *)v[19];
         w.li = (float *)v[20]; w.lh[0] = (float *)v[21]; w.lh[1] = (float *)v[22]; w.acc_coll = (double *)v[23];
         w.acc_inlet = (double *)v[24]; w.acc_obj = (double *)v[25]; w.out = (double *)v[26];
-        w.objph = (float2 *)v[27];
+        w.objph = (float2 *)v[27]; w.phase2 = (float2 *)v[28];
         w.nblk_coll = nblk_coll;
         w.nblk_inlet = nblk_inlet;
     }
@@ -1375,6 +1421,47 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         a.grad2 = w.seg_g2[r] + t * NN;
         a.fm_out = conv ? w.seg_fm[r] + t * 54 * P : nullptr;
     };
+    // len recorded steps (record set r, indices from step) from the populations a.pin to a.pout; `a`
+    // carries everything else of the first step
+    AdvancePlan plan;
+    const bool advance = use_advance(c, a0, &plan);
+    auto recorded_steps = [&](StepArgs a, cudaStream_t s, long long len, int64_t step, int r, void *const (&pops)[2]) -> lb_status {
+        float2 *phase[2] = {c->phase, w.phase2};
+        for (long long t = 0; t < len; ++t) {
+            a.step = step + t;
+            record(a, t, r);
+            cudaError_t e;
+            if (!advance || len < 2) {  // pops[t & 1] -> pops[(t + 1) & 1]
+                a.pin = pops[t & 1];
+                a.pout = pops[(t + 1) & 1];
+                e = launch_step(a, LB_STORE_FP32, s, nullptr, &c->launches);
+            } else if (t == 0) {
+                a.pin = pops[0];
+                a.phase = phase[0];
+                e = launch_step(a, LB_STORE_FP32, s, nullptr, &c->launches, PASS_GATHER);
+            } else {  // the gradients an advance takes are those of the step before
+                StepArgs b = a;
+                b.grad4 -= NN;
+                b.grad2 -= NN;
+                AdvanceArgs v{};
+                v.mom[0] = a.mom - 3 * NN;
+                v.mom_out[0] = a.mom;
+                v.phase = phase[(t - 1) & 1];
+                v.phase_out = phase[t & 1];
+                v.err = c->ferr;
+                e = launch_advance(b, plan, v, s, &c->launches);
+            }
+            if (e != cudaSuccess) return cuda_fail(e, "recorded step");
+        }
+        if (advance && len >= 2) {
+            a.phase = phase[(len - 1) & 1];
+            a.pout = pops[len & 1];
+            cudaError_t e = launch_step(a, LB_STORE_FP32, s, nullptr, &c->launches, PASS_COLLIDE);
+            if (e != cudaSuccess) return cuda_fail(e, "recorded step (collide)");
+        }
+        return LB_OK;
+    };
+
     // forward pass with a checkpoint at the start of every segment; the last segment records
     // as it goes, so the reverse sweep needs no recompute for it
     const int64_t step0 = c->step;
@@ -1386,19 +1473,18 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
             LB_CUDA(cudaMemcpyAsync(w.ckpt_pop + sg * 27 * NN, c->pop[c->cur], pb, cudaMemcpyDeviceToDevice, st));
             if (conv)
                 LB_CUDA(cudaMemcpyAsync(w.ckpt_hist + sg * 54 * P, c->hist[c->hcur], hb, cudaMemcpyDeviceToDevice, st));
+            lb_status rs = steps_unchecked(c, advance ? &plan : nullptr, len);
+            if (rs != LB_OK) return rs;
+        } else {
+            LB_CUDA(cudaMemcpyAsync(w.seg_hist[r], c->hist[c->hcur], hb, cudaMemcpyDeviceToDevice, st));
+            void *const pops[2] = {c->pop[c->cur], c->pop[c->cur ^ 1]};
+            lb_status rs = recorded_steps(make_args(c), st, len, c->step, r, pops);
+            if (rs != LB_OK) return rs;
+            c->cur ^= (int)(len & 1);
+            c->step += len;
+            if (conv)
+                LB_CUDA(cudaMemcpyAsync(c->hist[c->hcur], w.seg_hist[r] + len * 54 * P, hb, cudaMemcpyDeviceToDevice, st));
         }
-        if (last) LB_CUDA(cudaMemcpyAsync(w.seg_hist[r], c->hist[c->hcur], hb, cudaMemcpyDeviceToDevice, st));
-        for (long long t = 0; t < len; ++t) {
-            StepArgs a = make_args(c);
-            if (last) record(a, t, r);
-            cudaError_t e = launch_step(a, LB_STORE_FP32, st, nullptr, &c->launches);
-            if (e != cudaSuccess) return cuda_fail(e, "launch_step");
-            c->cur ^= 1;
-            if (conv && !last) c->hcur ^= 1;
-            c->step += 1;
-        }
-        if (last && conv)
-            LB_CUDA(cudaMemcpyAsync(c->hist[c->hcur], w.seg_hist[r] + len * 54 * P, hb, cudaMemcpyDeviceToDevice, st));
     }
 
     // objective of S(T) and its adjoint
@@ -1423,8 +1509,6 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     // kernels read none of them).
     auto seg_args = [&](long long t, int64_t step, int r) {
         StepArgs a = make_args(c);
-        a.pin = w.seg_pop + (t & 1) * 27 * NN;
-        a.pout = w.seg_pop + ((t + 1) & 1) * 27 * NN;
         record(a, t, r);
         a.step = step;
         return a;
@@ -1437,10 +1521,9 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         LB_CUDA(cudaMemcpyAsync(w.seg_pop, w.ckpt_pop + sg * 27 * NN, pb, cudaMemcpyDeviceToDevice, s2));
         if (conv)
             LB_CUDA(cudaMemcpyAsync(w.seg_hist[r], w.ckpt_hist + sg * 54 * P, hb, cudaMemcpyDeviceToDevice, s2));
-        for (long long t = 0; t < len; ++t) {
-            cudaError_t e = launch_step(seg_args(t, step0 + n0 + t, r), LB_STORE_FP32, s2, nullptr, &c->launches);
-            if (e != cudaSuccess) return cuda_fail(e, "launch_step (recompute)");
-        }
+        void *const pops[2] = {w.seg_pop, w.seg_pop + 27 * NN};
+        lb_status rs = recorded_steps(make_args(c), s2, len, step0 + n0, r, pops);
+        if (rs != LB_OK) return rs;
         LB_CUDA(cudaEventRecord(w.ev_rec[r], s2));
         return LB_OK;
     };
@@ -1478,8 +1561,14 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         if (e != cudaSuccess) return cuda_fail(e, "launch_adjoint_reduce");
     }
     double host[32];
+    int ran_out = 0;
     LB_CUDA(cudaMemcpyAsync(host, w.out, sizeof(host), cudaMemcpyDeviceToHost, st));
+    LB_CUDA(cudaMemcpyAsync(&ran_out, c->ferr, sizeof(int), cudaMemcpyDeviceToHost, st));
     LB_CUDA(cudaStreamSynchronize(st));
+    if (ran_out) {
+        cudaMemsetAsync(c->ferr, 0, sizeof(int), st);
+        return fail(LB_ETIMEOUT, "a wait inside a step kernel ran out: the state is not to be trusted");
+    }
     grad_out[0] = host[24];
     for (int j = 1; j < LB_ADJ_NOUT; ++j) grad_out[j] = host[j];
     w.cl = cl;
