@@ -25,6 +25,7 @@ __all__ = ["Lattice", "LBError", "library", "make_grid", "make_params", "BC_PERI
 # order of the gradient entries lb_adjoint returns after J
 GRAD_NAMES = ("u_in", "sigma", "nu_r", "nu_b") + tuple(f"{ab}{m}" for m in range(1, 9) for ab in "ab")
 OBJECTIVES = {"area": 0, "penetration": 1}
+_FieldPointers = C.c_void_p * len(FIELD_NAMES)
 
 
 def _torch():
@@ -168,21 +169,25 @@ class Lattice:
         """Dict of macroscopic fields (float32, shape (nz, ny, nx)) as CUDA tensors
         (device=True) or numpy arrays (device=False); `out` may supply the arrays."""
         torch = _torch()
-        mask, outs, keep = 0, (C.POINTER(C.c_float) * len(FIELD_NAMES))(), {}
-        for j, nm in enumerate(FIELD_NAMES):
-            if nm not in names:
-                continue
-            mask |= 1 << j
-            if device:
-                t = out[nm] if out else torch.empty(self.shape, dtype=torch.float32, device=self.device)
-                assert t.is_cuda and t.dtype == torch.float32 and t.is_contiguous() and t.numel() == self.nodes
-                outs[j] = C.cast(C.c_void_p(t.data_ptr()), C.POINTER(C.c_float))
-            else:
-                t = out[nm] if out else np.empty(self.shape, dtype=np.float32)
+        sel = [j for j, nm in enumerate(FIELD_NAMES) if nm in names]
+        if not device:
+            ts = [out[FIELD_NAMES[j]] if out else np.empty(self.shape, dtype=np.float32) for j in sel]
+            for t in ts:
                 assert t.dtype == np.float32 and t.flags.c_contiguous and t.size == self.nodes
-                outs[j] = t.ctypes.data_as(C.POINTER(C.c_float))
-            keep[nm] = t
-        _abi.check(self.lib.lb_fields(self._ctx, C.c_uint32(mask), outs, 1 if device else 0))
+        elif out:
+            ts = [out[FIELD_NAMES[j]] for j in sel]
+            for t in ts:
+                assert t.is_cuda and t.dtype == torch.float32 and t.is_contiguous() and t.numel() == self.nodes
+        elif self.nodes <= 65536:  # one allocation: seven cost more host time than the kernel runs
+            ts = torch.empty((len(sel),) + self.shape, dtype=torch.float32, device=self.device).unbind(0)
+        else:
+            ts = [torch.empty(self.shape, dtype=torch.float32, device=self.device) for _ in sel]
+        mask, outs, keep = 0, _FieldPointers(), {}
+        for j, t in zip(sel, ts):
+            mask |= 1 << j
+            outs[j] = t.data_ptr() if device else t.ctypes.data
+            keep[FIELD_NAMES[j]] = t
+        _abi.check(self.lib.lb_fields(self._ctx, mask, outs, 1 if device else 0))
         return keep
 
     def populations(self, device=True):

@@ -80,7 +80,7 @@ def library(path: str = LIB_PATH):
         L.lb_step.argtypes = [vp, C.c_int64]
         L.lb_step_count.argtypes = [vp]
         L.lb_step_count.restype = C.c_int64
-        L.lb_fields.argtypes = [vp, C.c_uint32, C.POINTER(fp), C.c_int32]
+        L.lb_fields.argtypes = [vp, C.c_uint32, vp, C.c_int32]  # an array of field pointers
         L.lb_populations.argtypes = [vp, fp, C.c_int32]
         L.lb_history.argtypes = [vp, fp, C.c_int32]
         L.lb_mass.argtypes = [vp, dp]

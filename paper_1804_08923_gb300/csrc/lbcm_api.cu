@@ -283,14 +283,23 @@ struct FieldOut {
 
 template <int S>
 __global__ void fields_kernel(StepArgs sa, FieldOut fo, float gx, float gy, float gz) {
+    chain_begin();
     const long long NN = sa.NN;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < NN; n += (long long)gridDim.x * blockDim.x) {
-        const Nbr nb = node_nbr(sa, n);
         MassAcc mr, mb;
         float jx = 0.0f, jy = 0.0f, jz = 0.0f;
+        float2 f[27];
+        if constexpr (S == STORE_FP32) {  // all loads in flight before the first sum
+#pragma unroll
+            for (int i = 0; i < 27; ++i) f[i] = load_pop<S>(sa, i, (int)n, no_shift());
+        } else {
+            const Nbr nb = node_nbr(sa, n);
+#pragma unroll
+            for (int i = 0; i < 27; ++i) f[i] = stored_pop<S>(sa, nb, i);
+        }
 #pragma unroll
         for (int i = 0; i < 27; ++i) {
-            const float2 v = stored_pop<S>(sa, nb, i);
+            const float2 v = f[i];
             mr.add(i, v.x);
             mb.add(i, v.y);
             if (cx(i) != 0) jx += cx(i) * (v.x + v.y);
@@ -1082,11 +1091,11 @@ lb_status lb_fields(lb_ctx *c, uint32_t mask, float *const *outs, int32_t on_dev
     FieldOut fo;
     for (int j = 0; j < LB_NFIELDS; ++j) fo.o[j] = dst[j];
     if (c->p.storage == LB_STORE_FP16)
-        fields_kernel<STORE_FP16><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(fields_kernel<STORE_FP16>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     else if (c->p.storage == LB_STORE_FP16_FIT)
-        fields_kernel<STORE_FP16_FIT><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(fields_kernel<STORE_FP16_FIT>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     else
-        fields_kernel<STORE_FP32><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(fields_kernel<STORE_FP32>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     c->launches += 1;
     LB_CUDA(cudaGetLastError());
     if (!on_device) {
