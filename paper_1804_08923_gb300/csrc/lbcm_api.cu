@@ -324,16 +324,26 @@ __global__ void fields_kernel(StepArgs sa, FieldOut fo, float gx, float gy, floa
     }
 }
 
-// Decoded populations of colour k in the canonical layout out[i][n] (27 x NN floats).
+// Decoded populations in the canonical layout out[k][i][n], of both colours in one pass (colour < 0;
+// 432 bytes a node with FP32 storage) or of one, to out[i][n] (a pass reads both: host output staged
+// in half the space).
 template <int S>
-__global__ void canonical_kernel(StepArgs sa, int k, float *__restrict__ out) {
+__global__ void __launch_bounds__(256) canonical_kernel(StepArgs sa, int colour, float *__restrict__ out) {
+    chain_begin();
     const long long NN = sa.NN;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < NN; n += (long long)gridDim.x * blockDim.x) {
-        const Nbr nb = node_nbr(sa, n);
+        auto put = [&](int i, float2 v) {
+            if (colour <= 0) out[(long long)i * NN + n] = v.x;
+            if (colour < 0) out[(long long)(27 + i) * NN + n] = v.y;
+            if (colour == 1) out[(long long)i * NN + n] = v.y;
+        };
+        if constexpr (S == STORE_FP32) {
 #pragma unroll
-        for (int i = 0; i < 27; ++i) {
-            const float2 v = stored_pop<S>(sa, nb, i);
-            out[(long long)i * NN + n] = k == 0 ? v.x : v.y;
+            for (int i = 0; i < 27; ++i) put(i, load_pop<S>(sa, i, (int)n, no_shift()));
+        } else {
+            const Nbr nb = node_nbr(sa, n);
+#pragma unroll
+            for (int i = 0; i < 27; ++i) put(i, stored_pop<S>(sa, nb, i));
         }
     }
 }
@@ -1109,23 +1119,24 @@ lb_status lb_fields(lb_ctx *c, uint32_t mask, float *const *outs, int32_t on_dev
 lb_status lb_populations(lb_ctx *c, float *out, int32_t on_device) {
     if (!c || !out) return fail(LB_EINVAL, "ctx and out must not be NULL");
     if (!c->initialized) return fail(LB_ESTATE, "lb_populations before lb_init/lb_load");
-    // decode one colour at a time (27 x nodes floats); host output is staged in the idle
-    // population buffer, which holds at least one colour in either storage
+    // host output is staged in the idle population buffer, which holds both colours with FP32
+    // storage and one (27 x nodes floats) with the half-precision ones
     const StepArgs sa = state_args(c);
-    float *stage = (float *)c->pop[c->cur ^ 1];
     const size_t cbytes = (size_t)27 * c->nn * sizeof(float);
-    for (int k = 0; k < 2; ++k) {
-        float *dst = on_device ? out + (size_t)k * 27 * c->nn : stage;
+    const bool both = on_device || c->p.storage == LB_STORE_FP32;
+    for (int k = both ? -1 : 0; k < (both ? 0 : 2); ++k) {
+        float *dst = on_device ? out : (float *)c->pop[c->cur ^ 1];
         if (c->p.storage == LB_STORE_FP16)
-            canonical_kernel<STORE_FP16><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, k, dst);
+            launch_chained(canonical_kernel<STORE_FP16>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, k, dst);
         else if (c->p.storage == LB_STORE_FP16_FIT)
-            canonical_kernel<STORE_FP16_FIT><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, k, dst);
+            launch_chained(canonical_kernel<STORE_FP16_FIT>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, k, dst);
         else
-            canonical_kernel<STORE_FP32><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(sa, k, dst);
+            launch_chained(canonical_kernel<STORE_FP32>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, k, dst);
         c->launches += 1;
         LB_CUDA(cudaGetLastError());
         if (!on_device)
-            LB_CUDA(cudaMemcpyAsync(out + (size_t)k * 27 * c->nn, stage, cbytes, cudaMemcpyDeviceToHost, c->stream));
+            LB_CUDA(cudaMemcpyAsync(both ? out : out + (size_t)k * 27 * c->nn, dst, both ? 2 * cbytes : cbytes,
+                                    cudaMemcpyDeviceToHost, c->stream));
     }
     if (!on_device) LB_CUDA(cudaStreamSynchronize(c->stream));
     return LB_OK;
