@@ -334,7 +334,7 @@ LB_API lb_status lb_adjoint_state(lb_ctx *ctx, float *out, int32_t on_device);
  * roots / volumes / diameters (host, each may be NULL): the first min(n_fragments, cap) kept
  * fragments in increasing order of their smallest linear node index (z, y, x row-major), which
  * names them.
- * Device scratch of ~9 B per node is allocated for the call.  LB_EINVAL for connectivity other
+ * The idle population buffer is its scratch.  LB_EINVAL for connectivity other
  * than 6 or 26. */
 typedef struct {
     int64_t n_fragments;          /* kept fragments */

@@ -274,15 +274,16 @@ class Lattice:
         equivalent diameters (6V/pi)^(1/3), the excluded column volume and the mass-median
         diameter, all computed by the library."""
         st = _abi.FragmentStats()
-        _abi.check(self.lib.lb_fragments(self._ctx, int(connectivity), int(bool(exclude_inlet)), None, None, None, 0,
-                                         C.byref(st)))
-        n = int(st.n_fragments)
-        roots, vols, diam = np.zeros(n, np.int64), np.zeros(n, np.int64), np.zeros(n, np.float64)
-        if n:
+        n, cap = 4096, -1
+        while n > cap:  # again with the exact number if there are more than the first guess
+            cap = n
+            roots, vols, diam = np.empty(cap, np.int64), np.empty(cap, np.int64), np.empty(cap, np.float64)
             _abi.check(self.lib.lb_fragments(self._ctx, int(connectivity), int(bool(exclude_inlet)),
                                              roots.ctypes.data_as(C.POINTER(C.c_int64)),
                                              vols.ctypes.data_as(C.POINTER(C.c_int64)),
-                                             diam.ctypes.data_as(C.POINTER(C.c_double)), n, C.byref(st)))
+                                             diam.ctypes.data_as(C.POINTER(C.c_double)), cap, C.byref(st)))
+            n = int(st.n_fragments)
+        roots, vols, diam = roots[:n].copy(), vols[:n].copy(), diam[:n].copy()
         return {"roots": roots, "volumes": vols, "diameters": diam,
                 "mass_median_diameter": float(st.mass_median_diameter), "column_volume": int(st.column_volume),
                 "total_volume": int(st.total_volume)}

@@ -1604,23 +1604,29 @@ lb_status lb_fragments(lb_ctx *c, int32_t connectivity, int32_t exclude_inlet, i
     if (cap < 0) return fail(LB_EINVAL, "cap must be >= 0");
     const size_t NN = (size_t)c->nn;
     const long long nblk = ((long long)NN + 1023) / 1024;
-    // scratch: label, count (int32), touch (u8), block counts, block offsets, error flag
-    const size_t parts[] = {NN * 4, NN * 4, NN, (size_t)nblk * 4, (size_t)(nblk + 1) * 8, 16};
+    // scratch: label, count (int32), touch (u8), block counts, block offsets, error flag, then the list
+    // of roots (17 bytes each), in the idle population buffer (at least 112 bytes a node); allocated
+    // only for lattices so small that the parts' alignment exceeds it
+    const size_t parts[] = {NN * 4, NN * 4, NN, (size_t)nblk * 4, (size_t)(nblk + 1) * 8, 16, NN * 17 + 64};
     size_t need = 0;
     for (size_t v : parts) need += align_up(v);
-    char *base = nullptr;
-    if (cudaMalloc(&base, need) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(LB_ENOMEM, "cannot allocate fragment scratch");
+    struct Free { char *p = nullptr; ~Free() { if (p) cudaFree(p); } } guard;
+    char *base = (char *)c->pop[c->cur ^ 1];
+    if (need > c->sizes[c->cur ^ 1]) {
+        if (cudaMalloc(&guard.p, need) != cudaSuccess) {
+            cudaGetLastError();
+            guard.p = nullptr;
+            return fail(LB_ENOMEM, "cannot allocate fragment scratch");
+        }
+        base = guard.p;
     }
-    struct Free { char *p; ~Free() { cudaFree(p); } } guard{base};
     char *q = base;
     int *label = (int *)q; q += align_up(parts[0]);
     int *count = (int *)q; q += align_up(parts[1]);
     uint8_t *touch = (uint8_t *)q; q += align_up(parts[2]);
     int *bc = (int *)q; q += align_up(parts[3]);
     long long *boff = (long long *)q; q += align_up(parts[4]);
-    int *err = (int *)q;
+    int *err = (int *)q; q += align_up(parts[5]);
     cudaStream_t st = c->stream;
     LB_CUDA(cudaMemsetAsync(count, 0, NN * 4, st));
     LB_CUDA(cudaMemsetAsync(touch, 0, NN, st));
@@ -1638,13 +1644,7 @@ lb_status lb_fragments(lb_ctx *c, int32_t connectivity, int32_t exclude_inlet, i
     std::vector<long long> hroot((size_t)nroots), hvol((size_t)nroots);
     std::vector<uint8_t> htouch((size_t)nroots);
     if (nroots > 0) {
-        char *ob = nullptr;
-        if (cudaMalloc(&ob, (size_t)nroots * 17 + 64) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(LB_ENOMEM, "cannot allocate the fragment list");
-        }
-        Free og{ob};
-        long long *o_root = (long long *)ob, *o_vol = o_root + nroots;
+        long long *o_root = (long long *)q, *o_vol = o_root + nroots;
         uint8_t *o_touch = (uint8_t *)(o_vol + nroots);
         e = launch_fragments_write(sa, connectivity, label, count, touch, boff, o_root, o_vol, o_touch, st,
                                    &c->launches);
