@@ -23,6 +23,7 @@
 #include "lbcm_device.cuh"
 #include "lbcm_internal.h"
 #include "lbcm_node.cuh"
+#include "lbcm_pairs.cuh"
 
 #include <algorithm>
 
@@ -89,22 +90,6 @@ __device__ __forceinline__ void cp_async8(unsigned smem, const void *gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// Coefficients of the inverse 1-D sweep: a value at c in {-1, 0, +1} from central moments
-// (m0, m1, m2) about u is G0[c] m0 + G1[c] m1 + G2[c] m2 with
-//   G0 = ((u^2 - u)/2, 1 - u^2, (u^2 + u)/2), G1 = (u - 1/2, -2u, u + 1/2), G2 = (1/2, -1, 1/2).
-struct InvAxis {
-    float g0[3], g1[3];
-    __device__ __forceinline__ explicit InvAxis(float u) {
-        const float u2 = u * u;
-        g0[0] = 0.5f * (u2 - u);
-        g0[1] = 1.0f - u2;
-        g0[2] = 0.5f * (u2 + u);
-        g1[0] = u - 0.5f;
-        g1[1] = -2.0f * u;
-        g1[2] = u + 0.5f;
-    }
-};
 
 // 1-D transpose of the inverse sweep: M_a = sum_c v_c G_a[c](u) for a = 0, 1, 2.
 __device__ __forceinline__ void sweep_inv_T(float &a0, float &a1, float &a2, const InvAxis &A) {

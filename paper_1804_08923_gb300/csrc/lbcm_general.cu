@@ -14,6 +14,7 @@
 #include "lbcm_device.cuh"
 #include "lbcm_internal.h"
 #include "lbcm_node.cuh"
+#include "lbcm_pairs.cuh"
 
 namespace lbcm {
 
@@ -55,50 +56,6 @@ __global__ void __launch_bounds__(128) phase_field_kernel(StepArgs a) {
 template <int S>
 __global__ void __launch_bounds__(128, S == STORE_FP16_FIT ? 5 : 1) phase_field_wall_kernel(StepArgs a) {
     phase_field_node<S, true>(a);
-}
-
-// Isotropic gradients of phi and rho (end of Section II): grad chi = 3 sum_j w_j chi(x + c_j)
-// c_j, summed over the 13 pairs of opposite directions (j, j+1) as 3 w_j c_j (chi(x + c_j) -
-// chi(x - c_j)), so that a uniform field gives exactly zero and nearby values subtract
-// exactly.  Ghosts: z = -1 is phi = 1, rho = rho_r0 inside the inlet disc and the mirror of
-// z = 0 elsewhere; z = N + 1 mirrors z = N.  kEdge = false: the caller knows that z > 0.
-template <int S, bool kEdge = true>
-__device__ __forceinline__ void stencil_gradients(const StepArgs &a, const Nbr &nb, int z, float &gpx, float &gpy,
-                                                  float &gpz, float &grx, float &gry, float &grz) {
-    const bool inlet_lo = kEdge && z == 0 && a.bc_zlo == BC_INLET;
-    float ph[27], rh[27];
-#pragma unroll
-    for (int j = 1; j < 27; ++j) {
-        // ghost planes were clamped onto z = 0 / z = N (mirror)
-        if constexpr (S == STORE_FP32) {
-            const float2 v = __ldg(a.phase + nb.nbr(j));
-            ph[j] = v.x;
-            rh[j] = v.y;
-        } else if constexpr (S == STORE_FP16) {
-            const float4 v = __ldg(a.ph_cur + nb.nbr(j));
-            ph[j] = v.x;
-            rh[j] = v.y;
-        } else {
-            const float4 v = __ldg(a.ph_cur + nb.nbr(j));
-            ph[j] = v.x;
-            rh[j] = fit_entry_rho(v);
-        }
-        if (cz(j) == -1 && inlet_lo) {
-            if (a.disc[nb.yo[1 - cy(j)] + nb.xo[1 - cx(j)]]) {  // z = -1 inside the inlet disc
-                ph[j] = 1.0f;
-                rh[j] = a.rho_r0;
-            }
-        }
-    }
-    gpx = gpy = gpz = grx = gry = grz = 0.0f;
-#pragma unroll
-    for (int j = 1; j < 27; j += 2) {  // c_{j+1} = -c_j
-        const float w3 = 3.0f * wgt(j);
-        const float dp = ph[j] - ph[j + 1], dr = rh[j] - rh[j + 1];
-        if (cx(j) != 0) { gpx = fmaf(w3 * cx(j), dp, gpx); grx = fmaf(w3 * cx(j), dr, grx); }
-        if (cy(j) != 0) { gpy = fmaf(w3 * cy(j), dp, gpy); gry = fmaf(w3 * cy(j), dr, gry); }
-        if (cz(j) != 0) { gpz = fmaf(w3 * cz(j), dp, gpz); grz = fmaf(w3 * cz(j), dr, grz); }
-    }
 }
 
 // 1-D shifted moment sweep: values at c = -1, 0, +1 -> central moments of order 0, 1, 2

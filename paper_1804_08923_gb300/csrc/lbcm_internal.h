@@ -54,6 +54,13 @@ AdvancePlan plan_advance(const StepArgs &a);
 cudaError_t launch_advance(const StepArgs &a, const AdvancePlan &p, const AdvanceArgs &v, cudaStream_t s,
                            long long *launches);
 
+// The same with half-precision storage (lbcm_half.cu): a step, its boundary planes alone, and the fused
+// kernel (or, occ not NULL, its blocks per SM).
+struct FusedCtl;
+void launch_half_step(const StepArgs &a, int storage, cudaStream_t s, cudaEvent_t *ev, long long *launches, int passes);
+void launch_half_boundary(const StepArgs &a, int storage, cudaStream_t s);
+cudaError_t half_fused(const StepArgs &a, int storage, const FusedCtl &f, int grid, cudaStream_t s, int *occ);
+
 // The two passes of a step with relaxation rates other than the paper's (lbcm_general.cu).
 void launch_general_gather(const StepArgs &a, int storage, cudaStream_t s);
 void launch_general_collide(const StepArgs &a, int storage, cudaStream_t s);

@@ -226,12 +226,8 @@ __device__ __forceinline__ float inlet_population_at(const StepArgs &a, int i, i
     return inlet_population(a, i, cxs, cys, iv.ux, iv.uy, iv.uz);
 }
 
-// The phase entry of a node as its storage keeps it: FP32 (phi, rho); FP16 (phi, rho, rho_r,
-// rho_b), which the next populations are encoded against.
+// The phase entry of a node (FP32 storage).
 __device__ __forceinline__ float2 phase_entry(const Moments &m) { return make_float2(m.phi, m.rho_r + m.rho_b); }
-__device__ __forceinline__ float4 phase_entry_fp16(const Moments &m) {
-    return make_float4(m.phi, m.rho_r + m.rho_b, m.rho_r, m.rho_b);
-}
 
 // The collision moments of a node as the moment pass stores them: three float4 planes of NN
 // entries, (rho_r, rho_b, phi, jx), (jy, jz, dxz, dyz), (pzz, pxy, pxz, pyz).
