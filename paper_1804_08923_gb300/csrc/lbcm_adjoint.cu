@@ -6,19 +6,22 @@
 //   densities and isotropic gradients                   rho_k = sum_i f_i^k, grad phi, grad rho
 //   per-node collision, perturbation, recolouring        S(n+1) = C(f, grad phi, grad rho)
 // and its transpose, given lambda = dJ/dS(n+1), runs in three launches:
-//   adj_collide_kernel   per node: recomputes the node's forward quantities from S(n) and the
-//                        saved phase field, applies (dC/df)^T, (dC/dgrad)^T and accumulates
-//                        dJ/d(sigma, nu_r, nu_b); pushes lambda_f to the slots of S(n) its pulls
-//                        read (the transposed streaming), writes lambda of the two gradients.
+//   adj_collide_kernel   per node: applies (dC/df)^T, (dC/dgrad)^T to lambda of S(n+1) from the
+//                        forward step's recorded moments and gradients, and accumulates dJ/d(sigma,
+//                        nu_r, nu_b); writes lambda of the two gradients and the node's record (below).
 //   adj_stencil_kernel   per node: transposes the gradient stencil (with the ghost rules) into
-//                        lambda_rho_k, the adjoint of the node's colour densities.  It is added
-//                        to every population the node pulled, i.e. "deferred" to the reader in
-//                        the next reverse step instead of another full pass.
+//                        lambda_rho_k, the adjoint of the node's colour densities, and adds it to
+//                        the record.
 //   adj_boundary_kernel  per (x, y) column: inlet-disc gradients w.r.t. u_in and the 16 profile
 //                        coefficients, and the transpose of the convective outflow
 //                        f(N) = [hist + lambda f(N-1)] / (1 + lambda), lambda = clamp(u_z(N-1)).
-// The adjoint state between steps is (Lp, Lr, Lh): lambda_S(n)(x, k, i) = Lp(x, k, i) +
-// Lr^k(reader of slot (x, i)), and Lh = dJ/dhist(n).  Parameter gradients are summed per
+// A node's collision depends on its 54 pulled populations through its colour densities, momentum and
+// second moment, so their adjoint has the form
+//   lambda_f_i^k(y) = l_j . c_i + c_i Lambda c_i + l_k,
+// and the adjoint state between two reverse steps is those 11 numbers a node (AdjRec, 48 bytes) where
+// the populations' adjoint would be 54: lambda of slot (x, i) of S(n) is lambda_f of the node y that
+// pulls it, evaluated when it is needed.  On a convective lattice the outflow adds lx, 54 numbers
+// a column, to the pulls of plane N - 1, and Lh = dJ/dhist(n).  Parameter gradients are summed per
 // block in FP64 into one accumulator slot per block (deterministic, no atomics).
 #include "lbcm_device.cuh"
 #include "lbcm_internal.h"
@@ -62,34 +65,47 @@ __device__ __forceinline__ long long block_id() {
     return blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
 }
 
-// Whether a pull of step n+1 reads slot (node at height z, direction i): the inlet disc and the
-// convective plane read nothing.
-__device__ __forceinline__ bool slot_read(const StepArgs &a, int i, int z, bool own_in_disc) {
-    if (a.bc_zlo == BC_PERIODIC) return true;
-    const int zr = z + cz(i);
-    if (a.bc_zhi == BC_CONVECTIVE && zr >= a.nz - 1) return false;
-    return !(zr < 0 && own_in_disc);
+// lambda_f of the pull of direction i by node n, with the signs of c as given: the record's polynomial.
+// i selects which components are there at compile time; sx, sy, sz are their signs.
+__device__ __forceinline__ float2 adj_pull(const AdjRec &r, int i, int n, float sx, float sy, float sz) {
+    const float4 v0 = __ldg(r.p[0] + n);  // (l_r, l_b, l_jx, l_jy)
+    if (i == 0) return make_float2(v0.x, v0.y);
+    const float4 v1 = __ldg(r.p[1] + n);  // (l_jz, L_xx, L_yy, L_zz)
+    float t = 0.0f, q = 0.0f;
+    if (cx(i) != 0) { t = sx * v0.z; q = v1.y; }
+    if (cy(i) != 0) { t = fmaf(sy, v0.w, t); q += v1.z; }
+    if (cz(i) != 0) { t = fmaf(sz, v1.x, t); q += v1.w; }
+    if (csq(i) > 1) {
+        const float4 v2 = __ldg(r.p[2] + n);  // (L_xy, L_xz, L_yz, -), off-diagonal entries doubled
+        if (cx(i) != 0 && cy(i) != 0) q = fmaf(sx * sy, v2.x, q);
+        if (cx(i) != 0 && cz(i) != 0) q = fmaf(sx * sz, v2.y, q);
+        if (cy(i) != 0 && cz(i) != 0) q = fmaf(sy * sz, v2.z, q);
+    }
+    t += q;
+    return make_float2(v0.x + t, v0.y + t);
 }
 
-// lambda_S(n+1) of slot (node nb.n, direction i): the pushed part plus the deferred density
-// adjoint of the node that reads the slot in step n+1, if a pull reads it.
-__device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int i, int z,
-                                           bool own_in_disc) {
-    float2 v = __ldg(g.lp_in + (size_t)i * a.NN + nb.n);
-    if (slot_read(a, i, z, own_in_disc)) {
-        const float2 r = __ldg(g.lr_in + nb.nbr(i));
-        v.x += r.x;
-        v.y += r.y;
+// lambda of slot (node nb.n at height z, direction i) of S(n+1): lambda_f of the node that pulls it, in
+// the direction of its pull (beyond a wall that is the node of the wall layer, with the component
+// reversed).  The inlet disc and the convective plane pull nothing; the pulls of plane N - 1 have the
+// outflow's part too.  kEdge = false: the caller knows that 0 < z < N - 2.  On the first reverse step
+// (g.lr_obj) S(T)'s own lambda, the objective's density adjoint, is the same for every direction.
+template <bool W, bool kEdge>
+__device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int i, int z, bool own_in_disc) {
+    const float sx = W && nb.gx(i) ? -(float)cx(i) : (float)cx(i), sy = W && nb.gy(i) ? -(float)cy(i) : (float)cy(i);
+    if (!kEdge || a.bc_zlo == BC_PERIODIC) return adj_pull(g.rec_in, i, nb.nbr(i), sx, sy, (float)cz(i));
+    const int zr = z + cz(i), N = a.nz - 1;
+    if ((zr < 0 && own_in_disc) || (a.bc_zhi == BC_CONVECTIVE && zr >= N)) return make_float2(0.0f, 0.0f);
+    const float sz = zr < 0 || zr > N ? -(float)cz(i) : (float)cz(i);
+    float2 v = adj_pull(g.rec_in, i, nb.nbr(i), sx, sy, sz);
+    if (a.bc_zhi == BC_CONVECTIVE && zr == N - 1) {
+        const size_t P = (size_t)a.plane;
+        const float *x = g.lx + dir_of((int)sx, (int)sy, cz(i)) * P + (nb.nbr(i) - (N - 1) * (int)P);
+        v.x += x[0];
+        v.y += x[27 * P];
     }
     return v;
 }
-
-// 8-byte asynchronous global -> shared copy (no register holds the value in flight).
-__device__ __forceinline__ void cp_async8(unsigned smem, const void *gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // 1-D transpose of the inverse sweep: M_a = sum_c v_c G_a[c](u) for a = 0, 1, 2.
 __device__ __forceinline__ void sweep_inv_T(float &a0, float &a1, float &a2, const InvAxis &A) {
@@ -140,77 +156,6 @@ __device__ __forceinline__ void m3uu(const RawMom &M, float ux, float uy, float 
     oz = M.m201 * xx + M.m021 * yy + M.m001 * zz + M.m111 * xy + M.m102 * xz + M.m012 * yz;
 }
 
-// Starts the copies of lambda_S(n+1) of node nb.n into shared memory: the pushed part of each
-// slot, and the deferred density adjoint of the node that reads the slot in step n+1 where a
-// pull reads it (else zero).  kEdge = false: the caller knows that 0 < z < N - 1, where every
-// slot is read.
-template <bool kEdge>
-__device__ __forceinline__ void adj_fetch(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int z, float2 *L_s,
-                                          float2 *R_s) {
-    const bool own_in_disc = kEdge && a.bc_zlo == BC_INLET && z == 0 && a.disc[nb.pxy];
-    const unsigned sL = (unsigned)__cvta_generic_to_shared(L_s), sR = (unsigned)__cvta_generic_to_shared(R_s);
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        cp_async8(sL + cell(i) * 128 * 8, g.lp_in + (size_t)i * a.NN + nb.n);
-        if (!kEdge || slot_read(a, i, z, own_in_disc))
-            cp_async8(sR + cell(i) * 128 * 8, g.lr_in + nb.nbr(i));
-        else
-            R_s[cell(i) * 128] = make_float2(0.0f, 0.0f);
-    }
-    cp_async_commit();
-}
-
-// The adjoints of the 54 gathered populations of a node, from the adjoints of its momentum,
-// raw second moment and colour densities.
-struct AdjPush {
-    float ljx, ljy, ljz, lQxx, lQyy, lQzz, lQxy, lQxz, lQyz, lrr, lrb;
-};
-
-// Pushes lambda_f_i of node nb.n to the slot its pull read: the transposed streaming, with the
-// mirror, the inlet disc and the convective outflow on the boundary planes.  kEdge = false:
-// the caller knows that 0 < z < N, and the boundary-plane tests of every direction drop out.
-template <bool W, bool kEdge>
-__device__ __forceinline__ void adj_push(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int z, const AdjPush &q) {
-    const int N = a.nz - 1;
-    const bool pz = a.bc_zlo == BC_PERIODIC;
-    const bool conv_top = kEdge && !pz && z == N && a.bc_zhi == BC_CONVECTIVE;
-    const bool bot = kEdge && !pz && z == 0;
-    const bool slip_top = kEdge && !pz && z == N && a.bc_zhi == BC_FREESLIP;
-    const size_t P = (size_t)a.plane;
-#define PULLED(i) (W ? nb.pulled(i) : (i))
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        const float c0 = (float)cx(i), c1 = (float)cy(i), c2 = (float)cz(i);
-        float lf = c0 * q.ljx + c1 * q.ljy + c2 * q.ljz;
-        lf += c0 * c0 * q.lQxx + c1 * c1 * q.lQyy + c2 * c2 * q.lQzz + c0 * c1 * q.lQxy + c0 * c2 * q.lQxz +
-              c1 * c2 * q.lQyz;
-        const float2 o = make_float2(lf + q.lrr, lf + q.lrb);
-        if (conv_top) {
-            // f(N) comes from the outflow rule: its adjoint goes to the boundary kernel; the
-            // slots the plain pulls would have read are read by nobody
-            g.lc[(size_t)i * P + nb.pxy] = o.x;
-            g.lc[(size_t)(27 + i) * P + nb.pxy] = o.y;
-            if (cz(i) >= 0) g.lp_out[(size_t)PULLED(i) * a.NN + nb.src(i)] = make_float2(0.0f, 0.0f);
-            if (cz(i) == 1) g.lp_out[(size_t)i * a.NN + nb.n] = make_float2(0.0f, 0.0f);
-        } else if (bot && cz(i) == 1) {
-            const int xs = nb.xo[cx(i) + 1], ys = nb.yo[cy(i) + 1];  // source column (offsets, reflected)
-            const size_t slot = (size_t)mirror_z(PULLED(i)) * a.NN + ys + xs;
-            if (a.bc_zlo == BC_INLET && a.disc[ys + xs]) {
-                g.li[(size_t)zrank(i) * P + nb.pxy] = o.x;
-                g.lp_out[slot] = make_float2(0.0f, 0.0f);
-            } else {
-                g.lp_out[slot] = o;
-            }
-        } else if (slip_top && cz(i) == -1) {
-            const int xs = nb.xo[cx(i) + 1], ys = nb.yo[cy(i) + 1];
-            g.lp_out[(size_t)mirror_z(PULLED(i)) * a.NN + (size_t)N * P + ys + xs] = o;
-        } else {
-            g.lp_out[(size_t)PULLED(i) * a.NN + nb.src(i)] = o;
-        }
-    }
-#undef PULLED
-}
-
 // ---------------------------------------------------------------- reverse collision
 // Every per-direction sum of the reverse pass is linear in a_i = (rho_r lS^r_i + rho_b lS^b_i)/rho
 // or b_i = lS^r_i - lS^b_i with coefficients that are polynomials in c_i times shell constants
@@ -219,17 +164,9 @@ __device__ __forceinline__ void adj_push(const StepArgs &a, const AdjArgs &g, co
 // third order.  Only the recolouring's 1/|c_i| is not separable and is summed directly.
 template <bool kForce, bool W>
 __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArgs &g, int x, int y, int z,
-                                                 float (&part)[3], float2 *L_s, float2 *R_s) {
+                                                 float (&part)[3], float2 *L_s) {
     const Nbr nb(a, x, y, z);
     const int N = a.nz - 1;
-
-    // lambda of S(n+1) for the 27 directions: the pushed and the deferred parts are copied
-    // asynchronously into this thread's two columns of shared memory (tensor layout), and the
-    // node's recorded forward quantities are loaded and used while they are in flight
-    if (z == 0 || z >= N - 1)
-        adj_fetch<true>(a, g, nb, z, L_s, R_s);
-    else
-        adj_fetch<false>(a, g, nb, z, L_s, R_s);
 
     // ---- the forward step's collision inputs of this node (recorded in the recompute)
     const size_t NN = (size_t)a.NN;
@@ -279,13 +216,19 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     const float pert = Acoef * inv_gm;
     const float R = a.beta * rr * rb * inv_rho;
 
-    // ---- a_i and b_i, in place, from lambda S = pushed + deferred
-    cp_async_wait_all();
+    // ---- a_i and b_i into this thread's column of shared memory (tensor layout): 54 registers less
+    auto put = [&](int i, float2 l) { L_s[cell(i) * 128] = make_float2((rr * l.x + rb * l.y) * inv_rho, l.x - l.y); };
+    if (g.lr_obj) {
+        const float2 l = __ldg(g.lr_obj + nb.n);
 #pragma unroll
-    for (int c = 0; c < 27; ++c) {
-        const float2 P_ = L_s[c * 128], D_ = R_s[c * 128];
-        const float lx = P_.x + D_.x, ly = P_.y + D_.y;
-        L_s[c * 128] = make_float2((rr * lx + rb * ly) * inv_rho, lx - ly);
+        for (int i = 0; i < 27; ++i) put(i, l);
+    } else if (z == 0 || z >= N - 2) {
+        const bool own_in_disc = a.bc_zlo == BC_INLET && z == 0 && a.disc[nb.pxy];
+#pragma unroll
+        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, true>(a, g, nb, i, z, own_in_disc));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, false>(a, g, nb, i, z, false));
     }
     const float a0 = L_s[13 * 128].x, b0 = L_s[13 * 128].y;  // rest direction: cell 13
     const float w0 = 8.0f / 27.0f, k27 = 27.0f / 19.0f;
@@ -493,15 +436,12 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     lrr += lrho;
     lrb += lrho;
 
-    // ---- outputs: lambda_f_i^k = lambda_j . c_i + c_i Lambda_P c_i + lambda_rho_k, pushed to the
-    // slot the pull read (with side walls, W: the reflected direction, selected at run time)
+    // ---- outputs: the record of lambda_f_i^k = lambda_j . c_i + c_i Lambda_P c_i + lambda_rho_k
     g.lga[nb.n] = make_float4(lgpx, lgpy, lgpz, lgrx);
     g.lgb[nb.n] = make_float2(lgry, lgrz);
-    const AdjPush o{ljx, ljy, ljz, lQxx, lQyy, lQzz, lQxy, lQxz, lQyz, lrr, lrb};
-    if (z == 0 || z == N)
-        adj_push<W, true>(a, g, nb, z, o);
-    else
-        adj_push<W, false>(a, g, nb, z, o);
+    g.rec_out.p[0][nb.n] = make_float4(lrr, lrb, ljx, ljy);
+    g.rec_out.p[1][nb.n] = make_float4(ljz, lQxx, lQyy, lQzz);
+    g.rec_out.p[2][nb.n] = make_float4(lQxy, lQxz, lQyz, 0.0f);
 }
 
 #ifndef LBCM_ADJ_MIN_BLOCKS
@@ -513,10 +453,10 @@ __global__ void __launch_bounds__(128, LBCM_ADJ_MIN_BLOCKS) adj_collide_kernel(S
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
-    extern __shared__ float2 adj_dsm[];  // [2][27][128]: pushed and deferred lambda S(n+1)
+    __shared__ float2 adj_sm[27 * 128];  // a_i, b_i
     const int t = threadIdx.y * 32 + threadIdx.x;
     float part[3] = {0.0f, 0.0f, 0.0f};
-    if (x < a.nx && y < a.ny) adj_collide_node<kForce, W>(a, g, x, y, z, part, adj_dsm + t, adj_dsm + 27 * 128 + t);
+    if (x < a.nx && y < a.ny) adj_collide_node<kForce, W>(a, g, x, y, z, part, adj_sm + t);
     block_accumulate<3>(part, g.acc_coll, block_id());
 }
 
@@ -585,7 +525,14 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g)
         S_ = ph.y / (a.rho_r0 * 0.5f * (1.0f + ph.x) + a.rho_b0 * 0.5f * (1.0f - ph.x));
     }
     const float t = lphi / S_;
-    g.lr_out[nb.n] = make_float2(fmaf(t * (1.0f - phv), a.inv_rho_r0, lrho), fmaf(-t * (1.0f + phv), a.inv_rho_b0, lrho));
+    const float2 l = make_float2(fmaf(t * (1.0f - phv), a.inv_rho_r0, lrho), fmaf(-t * (1.0f + phv), a.inv_rho_b0, lrho));
+    if (g.mom) {  // a reverse step: into the record
+        float2 *r = reinterpret_cast<float2 *>(g.rec_out.p[0] + nb.n);
+        const float2 d = *r;
+        *r = make_float2(d.x + l.x, d.y + l.y);
+    } else {
+        g.lr_out[nb.n] = l;
+    }
 }
 
 // ----------------------------------------------- inlet gradients and outflow transpose
@@ -594,6 +541,14 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// lambda_f of node n's own pull of direction c (components known at run time).
+__device__ __forceinline__ float2 adj_pull_any(const AdjRec &r, size_t n, int c0, int c1, int c2) {
+    const float4 v0 = r.p[0][n], v1 = r.p[1][n], v2 = r.p[2][n];
+    const float x = (float)c0, y = (float)c1, z = (float)c2;
+    const float t = x * v0.z + y * v0.w + z * v1.x + x * x * v1.y + y * y * v1.z + z * z * v1.w + x * y * v2.x + x * z * v2.y + y * z * v2.z;
+    return make_float2(v0.x + t, v0.y + t);
 }
 
 __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g) {
@@ -618,15 +573,11 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
         if (ys < 0 || ys >= a.ny) {
             if (a.wall_y) { ys = y; cys = -cyi; } else ys = wrapi(ys, a.ny);
         }
-        const int ii = dir_of(cxs, cys, czi);
         const int q = cxi * cxi + cyi * cyi + czi * czi;
         const float w_i = q == 0 ? 8.0f / 27.0f : q == 1 ? 2.0f / 27.0f : q == 2 ? 1.0f / 54.0f : 1.0f / 216.0f;
         if (a.bc_zlo == BC_INLET && lane < 27 && czi == 1) {
             if (a.disc[(size_t)ys * a.nx + xs]) {
-                // rank of i among the c_z = +1 directions
-                int zr = 0;
-                for (int j = 0; j < i; ++j) zr += ((int)((kPackZ >> (2 * j)) & 3ull) - 1) == 1;
-                const float lam = g.li[(size_t)zr * P + pxy] + g.lr_out[pxy].x;
+                const float lam = adj_pull_any(g.rec_out, pxy, cxi, cyi, czi).x;
                 InletVel iv;
                 inlet_velocity(a.u_in, a.noise_amp, a.fourier, a.xc, a.yc, a.seed, a.step, xs, ys, a.nx, a.ny, iv);
                 const float c0 = (float)cxs, c1 = (float)cys, c2 = (float)czi;  // direction leaving the ghost
@@ -648,10 +599,7 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
             }
         }
         if (a.bc_zhi == BC_CONVECTIVE) {
-            const int N = a.nz - 1, zm = N - 1;
-            const Nbr nbm(a, x, y, zm);
-            // the source of f_i(x, y, N-1) (plain pull in z: 1 <= N-1; reflected at side walls)
-            const int src = nbm.zo[czi + 1] + nbm.yo[cyi + 1] + nbm.xo[cxi + 1];
+            const int N = a.nz - 1;
             float fr = 0.0f, fb = 0.0f;
             if (lane < 27) {  // f(N-1) as the forward step pulled it
                 fr = __ldg(g.fm + (size_t)i * P + pxy);
@@ -663,12 +611,12 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
             const float lam_raw = (jz + 0.5f * Fz) / rho;
             const float lam = fminf(fmaxf(lam_raw, 0.0f), 1.0f);
             const float inv = 1.0f / (1.0f + lam);
-            const float2 lrN = g.lr_out[(size_t)N * P + pxy];
             float lvr = 0.0f, lvb = 0.0f, part_l = 0.0f;
             const size_t hr = (size_t)i * P + pxy, hb = (size_t)(27 + i) * P + pxy;
             if (lane < 27) {
-                lvr = g.lc[hr] + lrN.x + g.lh_in[hr];
-                lvb = g.lc[hb] + lrN.y + g.lh_in[hb];
+                const float2 lN = adj_pull_any(g.rec_out, (size_t)N * P + pxy, cxi, cyi, czi);
+                lvr = lN.x + g.lh_in[hr];
+                lvb = lN.y + g.lh_in[hb];
                 g.lh_out[hr] = lvr * inv;
                 g.lh_out[hb] = lvb * inv;
                 part_l = fmaf(lvr, fr - a.hist_out[hr], lvb * (fb - a.hist_out[hb]));
@@ -677,11 +625,8 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
             if (lane < 27) {
                 const bool active = lam_raw > 0.0f && lam_raw < 1.0f;
                 const float dl = active ? llam * ((float)czi + 0.5f * a.gz - lam_raw) / rho : 0.0f;
-                float2 *slot = g.lp_out + (size_t)ii * a.NN + src;
-                float2 v = *slot;
-                v.x += fmaf(lvr, lam * inv, dl);
-                v.y += fmaf(lvb, lam * inv, dl);
-                *slot = v;
+                g.lx[hr] = fmaf(lvr, lam * inv, dl);
+                g.lx[hb] = fmaf(lvb, lam * inv, dl);
             }
         }
     }
@@ -755,9 +700,9 @@ __global__ void __launch_bounds__(128) obj_pen_sum_kernel(StepArgs a, const floa
     block_accumulate<1>(part, acc, block_id());
 }
 
-// lambda_S(T)(n, k, i) = dL/dphi_n dphi/drho_k for every i; clears the deferred part.
+// lambda_S(T)(n, k, i) = dL/dphi_n dphi/drho_k for every i.
 __global__ void __launch_bounds__(256) obj_pen_adjoint_kernel(StepArgs a, const float2 *ph, const double *Z,
-                                                             float2 *lp, float2 *lr, float inv_delta, float delta) {
+                                                             float2 *lr, float inv_delta, float delta) {
     const float inv_Z = (float)(1.0 / *Z);
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.NN; n += (long long)gridDim.x * blockDim.x) {
         const float2 v = ph[n];
@@ -765,20 +710,7 @@ __global__ void __launch_bounds__(256) obj_pen_adjoint_kernel(StepArgs a, const 
         const float lphi = delta * 0.5f * (1.0f + v.x) * expf((float)(z - (a.nz - 1)) * inv_delta) * inv_Z;
         const float S_ = v.y / (a.rho_r0 * 0.5f * (1.0f + v.x) + a.rho_b0 * 0.5f * (1.0f - v.x));
         const float q = lphi / S_;
-        const float2 o = make_float2(q * (1.0f - v.x) * a.inv_rho_r0, -q * (1.0f + v.x) * a.inv_rho_b0);
-#pragma unroll
-        for (int i = 0; i < 27; ++i) lp[(size_t)i * a.NN + n] = o;
-        lr[n] = make_float2(0.0f, 0.0f);
-    }
-}
-
-// lambda_S(T)(n, k, i) = lr_obj(n, k) for every i (density adjoint of the objective).
-__global__ void __launch_bounds__(256) obj_fill_kernel(long long NN, const float2 *lr_obj, float2 *lp, float2 *lr) {
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < NN; n += (long long)gridDim.x * blockDim.x) {
-        const float2 o = lr_obj[n];
-#pragma unroll
-        for (int i = 0; i < 27; ++i) lp[(size_t)i * NN + n] = o;
-        lr[n] = make_float2(0.0f, 0.0f);
+        lr[n] = make_float2(q * (1.0f - v.x) * a.inv_rho_r0, -q * (1.0f + v.x) * a.inv_rho_b0);
     }
 }
 
@@ -811,7 +743,7 @@ __global__ void __launch_bounds__(256) adj_state_kernel(StepArgs a, AdjArgs g, f
         const bool own_in_disc = a.bc_zlo == BC_INLET && z == 0 && a.disc[nb.pxy];
 #pragma unroll
         for (int i = 0; i < 27; ++i) {
-            const float2 v = adj_slot(a, g, nb, i, z, own_in_disc);
+            const float2 v = adj_slot<true, true>(a, g, nb, i, z, own_in_disc);
             out[(size_t)i * a.NN + n] = v.x;
             out[(size_t)(27 + i) * a.NN + n] = v.y;
         }
@@ -833,28 +765,18 @@ long long adj_boundary_blocks(const StepArgs &a) {
     return (long long)gr.x * gr.y * gr.z;
 }
 
-constexpr int kAdjSmem = 2 * 27 * 128 * (int)sizeof(float2);
-
 cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_t s, long long *launches) {
     const bool force = a.gx != 0.0f || a.gy != 0.0f || a.gz != 0.0f;
     const bool walls = a.wall_x || a.wall_y;
-    static bool attr = false;  // the dynamic shared memory exceeds the 48 KB default
-    if (!attr) {
-        cudaFuncSetAttribute(adj_collide_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmem);
-        cudaFuncSetAttribute(adj_collide_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmem);
-        cudaFuncSetAttribute(adj_collide_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmem);
-        cudaFuncSetAttribute(adj_collide_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmem);
-        attr = true;
-    }
     const dim3 gr = node_grid(a), bl = node_block();
     if (force && walls)
-        launch_chained(adj_collide_kernel<true, true>, gr, bl, kAdjSmem, s, a, g);
+        launch_chained(adj_collide_kernel<true, true>, gr, bl, 0, s, a, g);
     else if (force)
-        launch_chained(adj_collide_kernel<true, false>, gr, bl, kAdjSmem, s, a, g);
+        launch_chained(adj_collide_kernel<true, false>, gr, bl, 0, s, a, g);
     else if (walls)
-        launch_chained(adj_collide_kernel<false, true>, gr, bl, kAdjSmem, s, a, g);
+        launch_chained(adj_collide_kernel<false, true>, gr, bl, 0, s, a, g);
     else
-        launch_chained(adj_collide_kernel<false, false>, gr, bl, kAdjSmem, s, a, g);
+        launch_chained(adj_collide_kernel<false, false>, gr, bl, 0, s, a, g);
     if (walls)
         launch_chained(adj_stencil_kernel<true>, gr, bl, 0, s, a, g);
     else
@@ -888,16 +810,14 @@ cudaError_t launch_objective(const StepArgs &a, const AdjArgs &g, int objective,
             adj_stencil_kernel<true><<<node_grid(a), node_block(), 0, s>>>(ao, o);
         else
             adj_stencil_kernel<false><<<node_grid(a), node_block(), 0, s>>>(ao, o);
-        obj_fill_kernel<<<stride_grid(a.NN), 256, 0, s>>>(a.NN, lr_obj, g.lp_out, g.lr_out);
         adj_reduce_kernel<<<1, 1024, 0, s>>>(acc_obj, nblk, 1, 0, scalar);
-        *launches += 4;
+        *launches += 3;
     } else {  // penetration length
         const double delta = args[0];
         obj_pen_sum_kernel<<<node_grid(a), node_block(), 0, s>>>(a, ph, acc_obj, (float)(1.0 / delta));
         adj_reduce_kernel<<<1, 1024, 0, s>>>(acc_obj, nblk, 1, 0, scalar + 1);
         obj_pen_value_kernel<<<1, 32, 0, s>>>(scalar + 1, scalar, (double)(a.nz - 1), delta);
-        obj_pen_adjoint_kernel<<<stride_grid(a.NN), 256, 0, s>>>(a, ph, scalar + 1, g.lp_out, g.lr_out,
-                                                                 (float)(1.0 / delta), (float)delta);
+        obj_pen_adjoint_kernel<<<stride_grid(a.NN), 256, 0, s>>>(a, ph, scalar + 1, lr_obj, (float)(1.0 / delta), (float)delta);
         *launches += 4;
     }
     return cudaGetLastError();

@@ -160,10 +160,11 @@ struct lb_ctx {
     struct {
         void *base = nullptr;
         size_t bytes = 0;
-        float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lp[2] = {}, *lr[2] = {}, *lgb = nullptr, *objph = nullptr,
+        float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lr_obj = nullptr, *lgb = nullptr, *objph = nullptr,
                *phase2 = nullptr;
-        float *ckpt_hist = nullptr, *seg_fm[2] = {}, *seg_hist[2] = {}, *lc = nullptr, *li = nullptr, *lh[2] = {};
+        float *ckpt_hist = nullptr, *seg_fm[2] = {}, *seg_hist[2] = {}, *lx = nullptr, *lh[2] = {};
         float4 *lga = nullptr, *seg_mom[2] = {}, *seg_g4[2] = {};
+        lbcm::AdjRec rec[2] = {};
         float2 *seg_g2[2] = {};
         // a second stream recomputes the next segment while the context's stream steps back
         // through the current one; events order the two
@@ -1341,7 +1342,7 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     const size_t pb = 27 * NN * sizeof(float2), hb = 54 * P * sizeof(float), nb2 = NN * sizeof(float2);
     StepArgs a0 = make_args(c);
     const long long nblk_coll = adj_collide_blocks(a0), nblk_inlet = adj_boundary_blocks(a0);
-    constexpr int kParts = 29;
+    constexpr int kParts = 27;
     auto layout = [&](long long k, size_t (&parts)[kParts]) {
         const long long nseg = (T + k - 1) / k;
         const size_t one = nseg > 1 ? 1 : 0, ku = (size_t)k;
@@ -1349,7 +1350,7 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         const size_t v[kParts] = {one * nseg * pb, one * nseg * hb, one * 2 * pb,
                                   rec[0], rec[1], rec[2], rec[3], rec[4],
                                   one * rec[0], one * rec[1], one * rec[2], one * rec[3], one * rec[4],
-                                  pb, pb, nb2, nb2, NN * sizeof(float4), nb2, hb, 9 * P * sizeof(float), hb, hb,
+                                  3 * NN * sizeof(float4), 3 * NN * sizeof(float4), nb2, NN * sizeof(float4), nb2, hb, hb, hb,
                                   nblk_coll * 3 * sizeof(double), nblk_inlet * 17 * sizeof(double),
                                   nblk_coll * sizeof(double), 32 * sizeof(double), nb2, nb2};
         size_t need = 0;
@@ -1403,11 +1404,13 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
             w.seg_g2[r] = (float2 *)v[5 + 5 * r]; w.seg_fm[r] = (float *)v[6 + 5 * r];
             w.seg_hist[r] = (float *)v[7 + 5 * r];
         }
-        w.lp[0] = (float2 *)v[13]; w.lp[1] = (float2 *)v[14]; w.lr[0] = (float2 *)v[15];
-        w.lr[1] = (float2 *)v[16]; w.lga = (float4 *)v[17]; w.lgb = (float2 *)v[18]; w.lc = (float *)v[19];
-        w.li = (float *)v[20]; w.lh[0] = (float *)v[21]; w.lh[1] = (float *)v[22]; w.acc_coll = (double *)v[23];
-        w.acc_inlet = (double *)v[24]; w.acc_obj = (double *)v[25]; w.out = (double *)v[26];
-        w.objph = (float2 *)v[27]; w.phase2 = (float2 *)v[28];
+        for (int r = 0; r < 2; ++r)
+            for (int q = 0; q < 3; ++q) w.rec[r].p[q] = (float4 *)v[13 + r] + q * NN;
+        w.lr_obj = (float2 *)v[15];
+        w.lga = (float4 *)v[16]; w.lgb = (float2 *)v[17]; w.lx = (float *)v[18];
+        w.lh[0] = (float *)v[19]; w.lh[1] = (float *)v[20]; w.acc_coll = (double *)v[21];
+        w.acc_inlet = (double *)v[22]; w.acc_obj = (double *)v[23]; w.out = (double *)v[24];
+        w.objph = (float2 *)v[25]; w.phase2 = (float2 *)v[26];
         w.nblk_coll = nblk_coll;
         w.nblk_inlet = nblk_inlet;
     }
@@ -1428,8 +1431,6 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     LB_CUDA(cudaMemsetAsync(w.acc_obj, 0, nblk_coll * sizeof(double), st));
     LB_CUDA(cudaMemsetAsync(w.out, 0, 32 * sizeof(double), st));
     LB_CUDA(cudaMemsetAsync(w.lh[0], 0, hb, st));
-    LB_CUDA(cudaMemsetAsync(w.lc, 0, hb, st));
-    LB_CUDA(cudaMemsetAsync(w.li, 0, 9 * P * sizeof(float), st));
 
     // what the reverse needs of step t of a segment (record set r = segment index & 1): the
     // collision inputs, f(N-1) and the outflow history before and after the step
@@ -1509,14 +1510,11 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
 
     // objective of S(T) and its adjoint
     AdjArgs g{};
-    g.lga = w.lga; g.lgb = w.lgb; g.lc = w.lc; g.li = w.li;
+    g.lga = w.lga; g.lgb = w.lgb; g.lx = w.lx;
     g.acc_coll = w.acc_coll; g.acc_inlet = w.acc_inlet;
     int cl = 0, ch = 0;
     {
-        AdjArgs go = g;
-        go.lp_out = w.lp[cl];
-        go.lr_out = w.lr[cl];
-        cudaError_t e = launch_objective(state_args(c), go, objective, obj_args, w.objph, w.lr[cl ^ 1], w.acc_obj,
+        cudaError_t e = launch_objective(state_args(c), g, objective, obj_args, w.objph, w.lr_obj, w.acc_obj,
                                          w.out + 24, st, &c->launches);
         if (e != cudaSuccess) return cuda_fail(e, "launch_objective");
     }
@@ -1561,8 +1559,8 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
             gs.grad4 = w.seg_g4[r] + t * NN;
             gs.grad2 = w.seg_g2[r] + t * NN;
             gs.fm = w.seg_fm[r] + t * 54 * P;
-            gs.lp_in = w.lp[cl]; gs.lr_in = w.lr[cl];
-            gs.lp_out = w.lp[cl ^ 1]; gs.lr_out = w.lr[cl ^ 1];
+            gs.rec_in = w.rec[cl]; gs.rec_out = w.rec[cl ^ 1];
+            gs.lr_obj = sg == nseg - 1 && t == len - 1 ? w.lr_obj : nullptr;
             gs.lh_in = w.lh[ch]; gs.lh_out = w.lh[ch ^ 1];
             cudaError_t e = launch_adjoint_step(seg_args(t, step0 + n0 + t, r), gs, st, &c->launches);
             if (e != cudaSuccess) return cuda_fail(e, "launch_adjoint_step");
@@ -1698,10 +1696,10 @@ lb_status lb_adjoint_state(lb_ctx *c, float *out, int32_t on_device) {
     if (!c->adj.valid) return fail(LB_ESTATE, "lb_adjoint_state before a successful lb_adjoint");
     auto &w = c->adj;
     AdjArgs g{};
-    g.lp_in = w.lp[w.cl];
-    g.lr_in = w.lr[w.cl];
+    g.rec_in = w.rec[w.cl];
+    g.lx = w.lx;
     const size_t bytes = 54 * (size_t)c->nn * sizeof(float);
-    float *dst = on_device ? out : (float *)w.lp[w.cl ^ 1];
+    float *dst = on_device ? out : (float *)c->pop[c->cur ^ 1];  // the idle population buffer stages host output
     cudaError_t e = launch_adjoint_state(make_args(c), g, dst, c->stream, &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "launch_adjoint_state");
     if (!on_device) LB_CUDA(cudaMemcpyAsync(out, dst, bytes, cudaMemcpyDeviceToHost, c->stream));

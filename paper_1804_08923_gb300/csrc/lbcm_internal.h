@@ -95,13 +95,19 @@ cudaError_t launch_fused_step(const StepArgs &a, int storage, const FusedCtl &f,
 // the wait's limit and sets *f.err; *ns receives the time it waited.
 cudaError_t launch_fused_wait_probe(const FusedCtl &f, unsigned long long *ns, cudaStream_t s);
 
+// Record of lambda_f of every node's pulls, lambda_f_i^k = l_j . c_i + c_i Lambda c_i + l_k:
+// p[0] = (l_r, l_b, l_jx, l_jy), p[1] = (l_jz, L_xx, L_yy, L_zz), p[2] = (L_xy, L_xz, L_yz, -), [NN] each.
+struct AdjRec {
+    float4 *p[3];
+};
 // Adjoint state and scratch of one reverse step (FP32 populations, paper rates).
-//   lp_in / lr_in   lambda of S(n+1): pushed part [27][NN] float2 and deferred density part [NN]
-//   lp_out / lr_out the same for S(n)
+//   rec_in / rec_out  records of step n+1 (lambda of S(n+1)) and of step n
+//   lr_obj          NULL, or, on the first reverse step, dJ/drho_k of S(T) [NN] in place of rec_in
 //   lga, lgb        lambda of (grad phi, grad rho) per node: (gpx, gpy, gpz, grx), (gry, grz)
-//   lc              direct lambda of f(N) on a convective top [54][nx ny]
-//   li              direct lambda of the red inlet populations that come from the disc [9][nx ny]
+//   lx              the outflow's part of lambda_f of the pulls of plane N - 1 [54][nx ny]: read as
+//                   step n+1 left it, then written by step n
 //   lh_in / lh_out  lambda of the outflow history hist(n+1) / hist(n) [54][nx ny]
+//   lr_out          launch_objective alone: receives dJ/drho_k
 //   acc_coll        FP64 per-block sums of dJ/d(sigma, nu_r, nu_b) [blocks][3]
 //   acc_inlet       FP64 per-block sums of dJ/d(u_in, a_1, b_1, ..., a_8, b_8) [blocks][17]
 //   mom             the forward step's collision moments per node, [3][NN] float4 as the moment
@@ -112,11 +118,12 @@ struct AdjArgs {
     const float4 *mom, *grad4;
     const float2 *grad2;
     const float *fm;
-    const float2 *lp_in, *lr_in;
-    float2 *lp_out, *lr_out;
+    AdjRec rec_in, rec_out;
+    const float2 *lr_obj;
+    float2 *lr_out;
     float4 *lga;
     float2 *lgb;
-    float *lc, *li;
+    float *lx;
     const float *lh_in;
     float *lh_out;
     double *acc_coll, *acc_inlet;
@@ -130,13 +137,13 @@ long long adj_boundary_blocks(const StepArgs &a);
 // step n).
 cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_t s, long long *launches);
 // Objective of the state a.pin (0 interface area, args[0] = eps; 1 penetration length,
-// args[0] = delta): scalar[0] = J; writes lambda_S(T) into g.lp_out / g.lr_out.
+// args[0] = delta): scalar[0] = J; writes dJ/drho_k, lambda of every direction of S(T), into lr_obj.
 cudaError_t launch_objective(const StepArgs &a, const AdjArgs &g, int objective, const double *args, float2 *ph,
                              float2 *lr_obj, double *acc_obj, double *scalar, cudaStream_t s, long long *launches);
 // out[1] = dJ/du_in, out[2..4] = dJ/d(sigma, nu_r, nu_b), out[5..20] = dJ/d(a_1, b_1, ..., b_8).
 cudaError_t launch_adjoint_reduce(const AdjArgs &g, long long nblk_coll, long long nblk_inlet, double *out,
                                   cudaStream_t s, long long *launches);
-// dJ/dS in the canonical layout [k][i][z][y][x] from (g.lp_in, g.lr_in).
+// dJ/dS in the canonical layout [k][i][z][y][x] from g.rec_in and g.lx.
 cudaError_t launch_adjoint_state(const StepArgs &a, const AdjArgs &g, float *out, cudaStream_t s, long long *launches);
 
 // Fragment labelling of the state a.pin (stored as `storage`): union-find labels (smallest node
