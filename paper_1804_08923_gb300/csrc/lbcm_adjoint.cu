@@ -23,10 +23,10 @@
 // pulls it, evaluated when it is needed.  On a convective lattice the outflow adds lx, 54 numbers
 // a column, to the pulls of plane N - 1, and Lh = dJ/dhist(n).  Parameter gradients are summed per
 // block in FP64 into one accumulator slot per block (deterministic, no atomics).
+#include "lbcm_collide.cuh"
 #include "lbcm_device.cuh"
 #include "lbcm_internal.h"
 #include "lbcm_node.cuh"
-#include "lbcm_pairs.cuh"
 
 #include <algorithm>
 
@@ -65,18 +65,38 @@ __device__ __forceinline__ long long block_id() {
     return blockIdx.x + (long long)gridDim.x * (blockIdx.y + (long long)gridDim.y * blockIdx.z);
 }
 
-// lambda_f of the pull of direction i by node n, with the signs of c as given: the record's polynomial.
-// i selects which components are there at compile time; sx, sy, sz are their signs.
-__device__ __forceinline__ float2 adj_pull(const AdjRec &r, int i, int n, float sx, float sy, float sz) {
-    const float4 v0 = __ldg(r.p[0] + n);  // (l_r, l_b, l_jx, l_jy)
+// The record of the node x + c_i: through L1 (RecNbr) or from the block's ring of planes in shared
+// memory (RecRing; p[cz + 1] points at the node's own cell in the plane z + cz).
+struct RecNbr {
+    const AdjRec &r;
+    const Nbr &nb;
+    __device__ __forceinline__ float4 ld(int q, int i) const { return __ldg(r.p[q] + nb.nbr(i)); }
+};
+// Tile of the marching collide adjoint: TX x 128 / TX nodes and one more on each side.
+template <int TX>
+struct AdjTile {
+    static constexpr int kTY = 128 / TX, kX = TX + 2, kN = kX * (kTY + 2);
+};
+template <int TX>
+struct RecRing {
+    using T = AdjTile<TX>;
+    const float4 *p[3];
+    __device__ __forceinline__ float4 ld(int q, int i) const { return p[cz(i) + 1][q * T::kN + cy(i) * T::kX + cx(i)]; }
+};
+
+// lambda_f of the pull of direction i by the node x + c_i, with the signs of c as given: the record's
+// polynomial.  i selects which components are there at compile time; sx, sy, sz are their signs.
+template <class R>
+__device__ __forceinline__ float2 adj_pull(const R &r, int i, float sx, float sy, float sz) {
+    const float4 v0 = r.ld(0, i);  // (l_r, l_b, l_jx, l_jy)
     if (i == 0) return make_float2(v0.x, v0.y);
-    const float4 v1 = __ldg(r.p[1] + n);  // (l_jz, L_xx, L_yy, L_zz)
+    const float4 v1 = r.ld(1, i);  // (l_jz, L_xx, L_yy, L_zz)
     float t = 0.0f, q = 0.0f;
     if (cx(i) != 0) { t = sx * v0.z; q = v1.y; }
     if (cy(i) != 0) { t = fmaf(sy, v0.w, t); q += v1.z; }
     if (cz(i) != 0) { t = fmaf(sz, v1.x, t); q += v1.w; }
     if (csq(i) > 1) {
-        const float4 v2 = __ldg(r.p[2] + n);  // (L_xy, L_xz, L_yz, -), off-diagonal entries doubled
+        const float4 v2 = r.ld(2, i);  // (L_xy, L_xz, L_yz, -), off-diagonal entries doubled
         if (cx(i) != 0 && cy(i) != 0) q = fmaf(sx * sy, v2.x, q);
         if (cx(i) != 0 && cz(i) != 0) q = fmaf(sx * sz, v2.y, q);
         if (cy(i) != 0 && cz(i) != 0) q = fmaf(sy * sz, v2.z, q);
@@ -90,14 +110,15 @@ __device__ __forceinline__ float2 adj_pull(const AdjRec &r, int i, int n, float 
 // reversed).  The inlet disc and the convective plane pull nothing; the pulls of plane N - 1 have the
 // outflow's part too.  kEdge = false: the caller knows that 0 < z < N - 2.  On the first reverse step
 // (g.lr_obj) S(T)'s own lambda, the objective's density adjoint, is the same for every direction.
-template <bool W, bool kEdge>
-__device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int i, int z, bool own_in_disc) {
+template <bool W, bool kEdge, class R>
+__device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, const R &r, const Nbr &nb, int i, int z,
+                                           bool own_in_disc) {
     const float sx = W && nb.gx(i) ? -(float)cx(i) : (float)cx(i), sy = W && nb.gy(i) ? -(float)cy(i) : (float)cy(i);
-    if (!kEdge || a.bc_zlo == BC_PERIODIC) return adj_pull(g.rec_in, i, nb.nbr(i), sx, sy, (float)cz(i));
+    if (!kEdge || a.bc_zlo == BC_PERIODIC) return adj_pull(r, i, sx, sy, (float)cz(i));
     const int zr = z + cz(i), N = a.nz - 1;
     if ((zr < 0 && own_in_disc) || (a.bc_zhi == BC_CONVECTIVE && zr >= N)) return make_float2(0.0f, 0.0f);
     const float sz = zr < 0 || zr > N ? -(float)cz(i) : (float)cz(i);
-    float2 v = adj_pull(g.rec_in, i, nb.nbr(i), sx, sy, sz);
+    float2 v = adj_pull(r, i, sx, sy, sz);
     if (a.bc_zhi == BC_CONVECTIVE && zr == N - 1) {
         const size_t P = (size_t)a.plane;
         const float *x = g.lx + dir_of((int)sx, (int)sy, cz(i)) * P + (nb.nbr(i) - (N - 1) * (int)P);
@@ -107,27 +128,42 @@ __device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, 
     return v;
 }
 
-// 1-D transpose of the inverse sweep: M_a = sum_c v_c G_a[c](u) for a = 0, 1, 2.
-__device__ __forceinline__ void sweep_inv_T(float &a0, float &a1, float &a2, const InvAxis &A) {
-    const float v0 = a0, v1 = a1, v2 = a2;
-    a0 = fmaf(A.g0[0], v0, fmaf(A.g0[1], v1, A.g0[2] * v2));
-    a1 = fmaf(A.g1[0], v0, fmaf(A.g1[1], v1, A.g1[2] * v2));
-    a2 = fmaf(0.5f, v0 + v2, -v1);
+// Asynchronous global -> shared copies (no register holds the value in flight).
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
+// 1-D transpose of the inverse transform of central moments about u (values v(+-1) = (t +- o)/2,
+// v(0) = m0 - t with t = u^2 m0 + 2 u m1 + m2, o = u m0 + m1), two fields at once: (v0, v1, v2) become
+// lambda of m0, twice that of m1 and twice that of m2.
+__device__ __forceinline__ void sweep_inv_T(float2 &v0, float2 &v1, float2 &v2, float u) {
+    const float2 s = __fadd2_rn(v2, v0), d = sub2(v2, v0), e = __ffma2_rn(both(-2.0f), v1, s);
+    v0 = __ffma2_rn(both(0.5f * u * u), e, __ffma2_rn(both(0.5f * u), d, v1));
+    v1 = __ffma2_rn(both(2.0f * u), e, d);
+    v2 = e;
 }
 
 // Weighted raw moments m_pqr = sum_i v_i w_i cx^p cy^q cz^r (p, q, r <= 2) of 27 values in the
 // tensor layout [cx+1][cy+1][cz+1], by 1-D sweeps: D3Q27's w_i is the product of the 1-D weights
-// (1/6, 2/3, 1/6).  Only the moments of total order <= 3 are kept (c^3 = c on the lattice).
+// (1/6, 2/3, 1/6), here times 6 an axis.  Only the moments of total order <= 3 are kept (c^3 = c on the
+// lattice).
 struct RawMom {
     float m000, m100, m010, m001, m200, m020, m002, m110, m101, m011, m210, m201, m120, m021, m102, m012, m111;
 };
-__device__ __forceinline__ void wsweep(float &v0, float &v1, float &v2) {
-    const float s = (v2 + v0) * (1.0f / 6.0f), d = (v2 - v0) * (1.0f / 6.0f);
-    v0 = fmaf(2.0f / 3.0f, v1, s);
+__device__ __forceinline__ void wsweep(float2 &v0, float2 &v1, float2 &v2) {
+    const float2 s = __fadd2_rn(v2, v0), d = sub2(v2, v0);
+    v0 = __ffma2_rn(both(4.0f), v1, s);
     v1 = d;
     v2 = s;
 }
-__device__ __forceinline__ void raw_moments(float (&t)[27], RawMom &M) {
+// of two fields at once: A of the .x, B of the .y
+__device__ __forceinline__ void raw_moments(float2 (&t)[27], RawMom &A, RawMom &B) {
 #pragma unroll
     for (int q = 0; q < 9; ++q) wsweep(t[q], t[9 + q], t[18 + q]);
 #pragma unroll
@@ -136,11 +172,18 @@ __device__ __forceinline__ void raw_moments(float (&t)[27], RawMom &M) {
         for (int c = 0; c < 3; ++c) wsweep(t[p * 9 + c], t[p * 9 + 3 + c], t[p * 9 + 6 + c]);
 #pragma unroll
     for (int p = 0; p < 9; ++p) wsweep(t[p * 3], t[p * 3 + 1], t[p * 3 + 2]);
-#define T_(p, q, r) t[(p) * 9 + (q) * 3 + (r)]
-    M = RawMom{T_(0, 0, 0), T_(1, 0, 0), T_(0, 1, 0), T_(0, 0, 1), T_(2, 0, 0), T_(0, 2, 0), T_(0, 0, 2), T_(1, 1, 0),
-               T_(1, 0, 1), T_(0, 1, 1), T_(2, 1, 0), T_(2, 0, 1), T_(1, 2, 0), T_(0, 2, 1), T_(1, 0, 2), T_(0, 1, 2),
-               T_(1, 1, 1)};
-#undef T_
+    auto get = [&](int p, int q, int r, float &x, float &y) {
+        const float2 v = __fmul2_rn(both(1.0f / 216.0f), t[p * 9 + q * 3 + r]);
+        x = v.x;
+        y = v.y;
+    };
+    get(0, 0, 0, A.m000, B.m000);
+    get(1, 0, 0, A.m100, B.m100); get(0, 1, 0, A.m010, B.m010); get(0, 0, 1, A.m001, B.m001);
+    get(2, 0, 0, A.m200, B.m200); get(0, 2, 0, A.m020, B.m020); get(0, 0, 2, A.m002, B.m002);
+    get(1, 1, 0, A.m110, B.m110); get(1, 0, 1, A.m101, B.m101); get(0, 1, 1, A.m011, B.m011);
+    get(2, 1, 0, A.m210, B.m210); get(2, 0, 1, A.m201, B.m201); get(1, 2, 0, A.m120, B.m120);
+    get(0, 2, 1, A.m021, B.m021); get(1, 0, 2, A.m102, B.m102); get(0, 1, 2, A.m012, B.m012);
+    get(1, 1, 1, A.m111, B.m111);
 }
 // M2 v (the second-moment tensor applied to a vector) and v.M2.w
 __device__ __forceinline__ void m2v(const RawMom &M, float vx, float vy, float vz, float &ox, float &oy, float &oz) {
@@ -162,20 +205,16 @@ __device__ __forceinline__ void m3uu(const RawMom &M, float ux, float uy, float 
 // proportional to w_i (varphi_i(alpha) = 27/19 (1 - alpha) w_i, the Phi coefficient 9 w_i and
 // B_i = w_i for i >= 1), so it is a combination of the weighted raw moments of a and b up to
 // third order.  Only the recolouring's 1/|c_i| is not separable and is summed directly.
-template <bool kForce, bool W>
-__device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArgs &g, int x, int y, int z,
-                                                 float (&part)[3], float2 *L_s) {
-    const Nbr nb(a, x, y, z);
+template <bool kForce, bool W, class Ring, class Next>
+__device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int z, const Ring &ring,
+                                                 const float4 (*own)[128], const float2 *own2, float (&part)[3],
+                                                 float2 *L_s, Next &&fetch_next) {
     const int N = a.nz - 1;
 
-    // ---- the forward step's collision inputs of this node (recorded in the recompute)
-    const size_t NN = (size_t)a.NN;
-    const Moments mo = load_moments(g.mom, NN, nb.n);
-    const float4 r3 = __ldg(g.grad4 + nb.n);
-    const float2 r4 = __ldg(g.grad2 + nb.n);
-    const float gpx = r3.x, gpy = r3.y, gpz = r3.z, grx = r3.w, gry = r4.x, grz = r4.y;
+    // ---- the forward step's collision inputs of this node
+    const Moments mo = unpack_moments(own[0][0], own[1][0], own[2][0]);
     const float rr = mo.rho_r, rb = mo.rho_b;
-    const float rho = rr + rb, inv_rho = 1.0f / rho;
+    const float rho = rr + rb, inv_rho = rcp_newton(rho);
     float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
     if (kForce) {
         const float fo = rho - a.rho_b0;
@@ -186,36 +225,38 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     const float phi = order_parameter(rr, rb, a.inv_rho_r0, a.inv_rho_b0);
     const float hp = 0.5f * (1.0f + phi), hm = 0.5f * (1.0f - phi);
     const float oma = one_minus_alpha_bar(a.alpha_mix, rr, rb, inv_rho, hp, hm, a.oma_r, a.oma_b), alpha = 1.0f - oma;
-    const float nu = 1.0f / (hp * a.inv_nu_r + hm * a.inv_nu_b);
-    const float tau = 3.0f * nu + 0.5f, s2nu = 1.0f / tau;
-    const float Acoef = 2.25f * a.sigma / tau;
+    const float nu = rcp_newton(hp * a.inv_nu_r + hm * a.inv_nu_b);
+    const float tau = 3.0f * nu + 0.5f, s2nu = rcp_newton(tau);
+    const float Acoef = 2.25f * a.sigma * s2nu;
     const float usq = ux * ux + uy * uy + uz * uz;
-    const float ugr = ux * grx + uy * gry + uz * grz;
     const float uF = ux * Fx + uy * Fy + uz * Fz;
     const float cs2 = oma * (9.0f / 19.0f);
-    // Q: second central moment of f - f^e + F'/2 (Pi(f^e), Pi(F') in closed form)
-    float Qxx = (mo.pzz + mo.dxz) - (rho * cs2 + rho * ux * ux + nu * (2.0f * ux * grx + ugr));
-    float Qyy = (mo.pzz + mo.dyz) - (rho * cs2 + rho * uy * uy + nu * (2.0f * uy * gry + ugr));
-    float Qzz = mo.pzz - (rho * cs2 + rho * uz * uz + nu * (2.0f * uz * grz + ugr));
-    float Qxy = mo.pxy - (rho * ux * uy + nu * (ux * gry + uy * grx));
-    float Qxz = mo.pxz - (rho * ux * uz + nu * (ux * grz + uz * grx));
-    float Qyz = mo.pyz - (rho * uy * uz + nu * (uy * grz + uz * gry));
-    if (kForce) {
-        Qxx += ux * Fx; Qyy += uy * Fy; Qzz += uz * Fz;
-        Qxy += 0.5f * (ux * Fy + uy * Fx); Qxz += 0.5f * (ux * Fz + uz * Fx); Qyz += 0.5f * (uy * Fz + uz * Fy);
-    }
+    float gpx, gpy, gpz, grx, gry, grz, ugr, Qxx, Qyy, Qzz, Qxy, Qxz, Qyz;
+    // gradients and Q, the second central moment of f - f^e + F'/2 (Pi(f^e), Pi(F') in closed form)
+    auto load_q = [&] {
+        const float4 r1 = own[1][0], r2 = own[2][0], r3 = own[3][0];
+        const float2 r4 = own2[0];
+        const float dxz = r1.z, dyz = r1.w, pzz = r2.x;
+        gpx = r3.x; gpy = r3.y; gpz = r3.z; grx = r3.w; gry = r4.x; grz = r4.y;
+        ugr = ux * grx + uy * gry + uz * grz;
+        Qxx = (pzz + dxz) - (rho * cs2 + rho * ux * ux + nu * (2.0f * ux * grx + ugr));
+        Qyy = (pzz + dyz) - (rho * cs2 + rho * uy * uy + nu * (2.0f * uy * gry + ugr));
+        Qzz = pzz - (rho * cs2 + rho * uz * uz + nu * (2.0f * uz * grz + ugr));
+        Qxy = r2.y - (rho * ux * uy + nu * (ux * gry + uy * grx));
+        Qxz = r2.z - (rho * ux * uz + nu * (ux * grz + uz * grx));
+        Qyz = r2.w - (rho * uy * uz + nu * (uy * grz + uz * gry));
+        if (kForce) {
+            Qxx += ux * Fx; Qyy += uy * Fy; Qzz += uz * Fz;
+            Qxy += 0.5f * (ux * Fy + uy * Fx); Qxz += 0.5f * (ux * Fz + uz * Fx); Qyz += 0.5f * (uy * Fz + uz * Fy);
+        }
+    };
+    load_q();
     const float o2 = 1.0f - s2nu, o2b = 1.0f - a.s2b, third = 1.0f / 3.0f;
-    const float trQ = Qxx + Qyy + Qzz;
+    float trQ = Qxx + Qyy + Qzz;
     const float k200 = o2 * (Qxx - trQ * third) + o2b * trQ * third;
     const float k020 = o2 * (Qyy - trQ * third) + o2b * trQ * third;
     const float k002 = o2 * (Qzz - trQ * third) + o2b * trQ * third;
     const float k110 = o2 * Qxy, k101 = o2 * Qxz, k011 = o2 * Qyz;
-    const InvAxis Ax(ux), Ay(uy), Az(uz);
-    const float g2 = gpx * gpx + gpy * gpy + gpz * gpz;
-    const float inv_gm = 1.0f / sqrtf(g2 + a.eps2);
-    const float pert = Acoef * inv_gm;
-    const float R = a.beta * rr * rb * inv_rho;
-
     // ---- a_i and b_i into this thread's column of shared memory (tensor layout): 54 registers less
     auto put = [&](int i, float2 l) { L_s[cell(i) * 128] = make_float2((rr * l.x + rb * l.y) * inv_rho, l.x - l.y); };
     if (g.lr_obj) {
@@ -225,41 +266,72 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     } else if (z == 0 || z >= N - 2) {
         const bool own_in_disc = a.bc_zlo == BC_INLET && z == 0 && a.disc[nb.pxy];
 #pragma unroll
-        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, true>(a, g, nb, i, z, own_in_disc));
+        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, true>(a, g, ring, nb, i, z, own_in_disc));
     } else {
 #pragma unroll
-        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, false>(a, g, nb, i, z, false));
+        for (int i = 0; i < 27; ++i) put(i, adj_slot<W, false>(a, g, ring, nb, i, z, false));
     }
     const float a0 = L_s[13 * 128].x, b0 = L_s[13 * 128].y;  // rest direction: cell 13
     const float w0 = 8.0f / 27.0f, k27 = 27.0f / 19.0f;
 
-    // ---- moments of b: the recolouring weight D = sum_i f**_i b_i and the flux direction Q1
-    float Dsum, Q1x = 0.0f, Q1y = 0.0f, Q1z = 0.0f;
+    // ---- h_i = sum_t C_t psi_t,i(u): lambda_C_t, d/du and sum_i b_i h_i by the transposed 1-D sweeps
+    float l200, l020, l002, l110, l101, l011, lux, luy, luz, bh;
     {
-        float t[27];
+        float2 t[27];
 #pragma unroll
-        for (int c = 0; c < 27; ++c) t[c] = L_s[c * 128].y;
-        // Q1 = 27/19 sum_{i>=1} b_i w_i c_i / |c_i|
+        for (int c = 0; c < 27; ++c) t[c] = L_s[c * 128];
 #pragma unroll
-        for (int i = 1; i < 27; ++i) {
-            const float v = t[cell(i)] * (k27 * wgt(i) * inv_cnorm(i));
-            Q1x += (float)cx(i) * v; Q1y += (float)cy(i) * v; Q1z += (float)cz(i) * v;
-        }
-        // sum_i b_i h_i = sum_t C_t (psi moments of b)
-        float tb[27];
-#pragma unroll
-        for (int c = 0; c < 27; ++c) tb[c] = t[c];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) sweep_inv_T(tb[q], tb[9 + q], tb[18 + q], Ax);
+        for (int q = 0; q < 9; ++q) sweep_inv_T(t[q], t[9 + q], t[18 + q], ux);
 #pragma unroll
         for (int p = 0; p < 3; ++p)
 #pragma unroll
-            for (int c = 0; c < 3; ++c) sweep_inv_T(tb[p * 9 + c], tb[p * 9 + 3 + c], tb[p * 9 + 6 + c], Ay);
+            for (int c = 0; c < 3; ++c) sweep_inv_T(t[p * 9 + c], t[p * 9 + 3 + c], t[p * 9 + 6 + c], uy);
 #pragma unroll
-        for (int p = 0; p < 9; ++p) sweep_inv_T(tb[p * 3], tb[p * 3 + 1], tb[p * 3 + 2], Az);
-        const float bh = k200 * tb[18] + k020 * tb[6] + k002 * tb[2] + k110 * tb[12] + k101 * tb[10] + k011 * tb[4];
-        RawMom B;
-        raw_moments(t, B);
+        for (int p = 0; p < 9; ++p) sweep_inv_T(t[p * 3], t[p * 3 + 1], t[p * 3 + 2], uz);
+        // an entry holds 2^(number of its nonzero orders) times its moment
+        const float h200 = 0.5f * k200, h020 = 0.5f * k020, h002 = 0.5f * k002, h110 = 0.25f * k110, h101 = 0.25f * k101,
+                    h011 = 0.25f * k011;
+        bh = h200 * t[18].y + h020 * t[6].y + h002 * t[2].y + h110 * t[12].y + h101 * t[10].y + h011 * t[4].y;
+#define MM(p, q, r) t[(p) * 9 + (q) * 3 + (r)].x
+        l200 = 0.5f * MM(2, 0, 0); l020 = 0.5f * MM(0, 2, 0); l002 = 0.5f * MM(0, 0, 2);
+        l110 = 0.25f * MM(1, 1, 0); l101 = 0.25f * MM(1, 0, 1); l011 = 0.25f * MM(0, 1, 1);
+        // with the values G_a[c](u) of the transform: dG0/du = G1, dG1/du = 2 G2, dG2/du = 0
+        lux = 0.5f * (h020 * MM(1, 2, 0) + h002 * MM(1, 0, 2) + h011 * MM(1, 1, 1)) + 2.0f * (h110 * MM(2, 1, 0) + h101 * MM(2, 0, 1));
+        luy = 0.5f * (h200 * MM(2, 1, 0) + h002 * MM(0, 1, 2) + h101 * MM(1, 1, 1)) + 2.0f * (h110 * MM(1, 2, 0) + h011 * MM(0, 2, 1));
+        luz = 0.5f * (h200 * MM(2, 0, 1) + h020 * MM(0, 2, 1) + h110 * MM(1, 1, 1)) + 2.0f * (h101 * MM(1, 0, 2) + h011 * MM(0, 1, 2));
+#undef MM
+    }
+
+    // ---- the gradients and Q once more: read again, they take no registers while the sweeps need them all
+    asm volatile("" ::: "memory");
+    load_q();
+    trQ = Qxx + Qyy + Qzz;
+    fetch_next();  // everything of this node is in registers or in L_s now
+    const float g2 = gpx * gpx + gpy * gpy + gpz * gpz;
+    const float inv_gm = rsqrt_newton(fmaxf(g2 + a.eps2, 1.1754944e-38f));  // of a normal number
+    const float pert = Acoef * inv_gm;
+    const float R = a.beta * rr * rb * inv_rho;
+
+    // ---- moments of a and b
+    RawMom A, B;
+    float Dsum, Q1x, Q1y, Q1z;
+    {
+        float2 t[27];
+#pragma unroll
+        for (int c = 0; c < 27; ++c) t[c] = L_s[c * 128];
+        // Q1 = 27/19 sum_{i>=1} b_i w_i c_i / |c_i|, opposite directions and the speed classes first
+        auto d = [&](int i) { return t[cell(i)].y - t[cell(i + 1)].y; };  // c_{i+1} = -c_i
+        const float d7 = d(7), d9 = d(9), d11 = d(11), d13 = d(13), d15 = d(15), d17 = d(17);
+        const float d19 = d(19), d21 = d(21), d23 = d(23), d25 = d(25);  // (1,1,1) (1,1,-1) (1,-1,1) (-1,1,1)
+        const float p = d19 + d21, q = d23 - d25, q1 = k27 * wgt(1) * inv_cnorm(1), q2 = k27 * wgt(7) * inv_cnorm(7),
+                    q3 = k27 * wgt(19) * inv_cnorm(19);
+        Q1x = fmaf(q1, d(1), fmaf(q2, (d7 + d9) + (d15 + d17), q3 * (p + q)));    // (1,1,0) (1,-1,0) (1,0,1) (1,0,-1)
+        Q1y = fmaf(q1, d(3), fmaf(q2, (d7 - d9) + (d11 + d13), q3 * (p - q)));    // (0,1,1) (0,1,-1)
+        Q1z = fmaf(q1, d(5), fmaf(q2, (d11 - d13) + (d15 - d17), q3 * ((d19 - d21) + (d23 + d25))));
+        raw_moments(t, A, B);
+    }
+    // ---- of b: the recolouring weight D = sum_i f**_i b_i
+    {
         const float B1u = B.m100 * ux + B.m010 * uy + B.m001 * uz;
         float Bux, Buy, Buz;
         m2v(B, ux, uy, uz, Bux, Buy, Buz);
@@ -293,13 +365,8 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     float lgm = -R * lR * inv_gm;
 
     // ---- moments of a: perturbation, equilibrium, forcing
-    float lux, luy, luz, lnu, lgrx, lgry, lgrz, lFx = 0.0f, lFy = 0.0f, lFz = 0.0f, lA;
+    float lnu, lgrx, lgry, lgrz, lFx = 0.0f, lFy = 0.0f, lFz = 0.0f, lA;
     {
-        float t[27];
-#pragma unroll
-        for (int c = 0; c < 27; ++c) t[c] = L_s[c * 128].x;
-        RawMom A;
-        raw_moments(t, A);
         const float sB = A.m000 - (2.0f / 3.0f) * a0;  // sum_i a_i B_i
         float Agx, Agy, Agz, Aux, Auy, Auz, Arx, Ary, Arz;
         m2v(A, gpx, gpy, gpz, Agx, Agy, Agz);
@@ -316,7 +383,7 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
         lgpx = fmaf(2.0f * gpx, lg2, lgpx);
         lgpy = fmaf(2.0f * gpy, lg2, lgpy);
         lgpz = fmaf(2.0f * gpz, lg2, lgpz);
-        part[0] += lA * 2.25f / tau;
+        part[0] += lA * 2.25f * s2nu;
         // equilibrium f^e_i = rho (varphi_i(alpha) + w_i poly_i(u)) + Phi_i(nu, u, grad rho)
         const float A1u = A.m100 * ux + A.m010 * uy + A.m001 * uz;
         float A3x, A3y, A3z;
@@ -327,9 +394,9 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
                 4.5f * A3uuu - 4.5f * usq * A1u;
         lalpha = fmaf(rho, a0 - k27 * (A.m000 - w0 * a0), lalpha);
         const float c3 = 3.0f - 4.5f * usq, s_u = -3.0f * A.m000 - 9.0f * A1u;
-        lux = rho * (c3 * A.m100 + 9.0f * Aux + 13.5f * A3x + ux * s_u);
-        luy = rho * (c3 * A.m010 + 9.0f * Auy + 13.5f * A3y + uy * s_u);
-        luz = rho * (c3 * A.m001 + 9.0f * Auz + 13.5f * A3z + uz * s_u);
+        lux += rho * (c3 * A.m100 + 9.0f * Aux + 13.5f * A3x + ux * s_u);
+        luy += rho * (c3 * A.m010 + 9.0f * Auy + 13.5f * A3y + uy * s_u);
+        luz += rho * (c3 * A.m001 + 9.0f * Auz + 13.5f * A3z + uz * s_u);
         lnu = -3.0f * a0 * ugr + 9.0f * (ux * Arx + uy * Ary + uz * Arz);
         lux = fmaf(nu, fmaf(-3.0f * a0, grx, 9.0f * Arx), lux);
         luy = fmaf(nu, fmaf(-3.0f * a0, gry, 9.0f * Ary), luy);
@@ -348,29 +415,6 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
             lFy = 0.5f * (3.0f * A.m010 - 3.0f * uy * A.m000 + 9.0f * Auy);
             lFz = 0.5f * (3.0f * A.m001 - 3.0f * uz * A.m000 + 9.0f * Auz);
         }
-    }
-    // ---- h_i = sum_t C_t psi_t,i(u): lambda_C_t and d/du via the transposed 1-D sweeps
-    float l200, l020, l002, l110, l101, l011;
-    {
-        float lh[27];
-#pragma unroll
-        for (int c = 0; c < 27; ++c) lh[c] = L_s[c * 128].x;
-#pragma unroll
-        for (int q = 0; q < 9; ++q) sweep_inv_T(lh[q], lh[9 + q], lh[18 + q], Ax);
-#pragma unroll
-        for (int a0_ = 0; a0_ < 3; ++a0_)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sweep_inv_T(lh[a0_ * 9 + 0 + c], lh[a0_ * 9 + 3 + c], lh[a0_ * 9 + 6 + c], Ay);
-#pragma unroll
-        for (int p = 0; p < 9; ++p) sweep_inv_T(lh[p * 3 + 0], lh[p * 3 + 1], lh[p * 3 + 2], Az);
-#define MM(p, q, r) lh[(p) * 9 + (q) * 3 + (r)]
-        l200 = MM(2, 0, 0); l020 = MM(0, 2, 0); l002 = MM(0, 0, 2);
-        l110 = MM(1, 1, 0); l101 = MM(1, 0, 1); l011 = MM(0, 1, 1);
-        // dG0/du = G1, dG1/du = 2 G2, dG2/du = 0
-        lux += k020 * MM(1, 2, 0) + k002 * MM(1, 0, 2) + 2.0f * k110 * MM(2, 1, 0) + 2.0f * k101 * MM(2, 0, 1) + k011 * MM(1, 1, 1);
-        luy += k200 * MM(2, 1, 0) + k002 * MM(0, 1, 2) + 2.0f * k110 * MM(1, 2, 0) + k101 * MM(1, 1, 1) + 2.0f * k011 * MM(0, 2, 1);
-        luz += k200 * MM(2, 0, 1) + k020 * MM(0, 2, 1) + k110 * MM(1, 1, 1) + 2.0f * k101 * MM(1, 0, 2) + 2.0f * k011 * MM(0, 1, 2);
-#undef MM
     }
     // ---- relaxation C = (1 - s2nu) dev Q + (1 - s2b) (tr Q / 3) I
     const float trl = l200 + l020 + l002;
@@ -405,7 +449,7 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     lgry -= nu * fmaf(2.0f, Luy, Ltr * uy);
     lgrz -= nu * fmaf(2.0f, Luz, Ltr * uz);
     // ---- sigma, tau, nu (harmonic mean), alpha-bar
-    const float ltau = -lA * Acoef / tau - ls2nu * s2nu * s2nu;
+    const float ltau = -lA * Acoef * s2nu - ls2nu * s2nu * s2nu;
     lnu = fmaf(3.0f, ltau, lnu);
     const float lH = -lnu * nu * nu;
     float lphi = lH * 0.5f * (a.inv_nu_r - a.inv_nu_b);
@@ -429,7 +473,7 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     // ---- phi = (A - B)/(A + B), A = rho_r / rho_r0, B = rho_b / rho_b0
     {
         const float S_ = rr * a.inv_rho_r0 + rb * a.inv_rho_b0;
-        const float t = lphi / S_;
+        const float t = lphi * rcp_newton(S_);
         lrr = fmaf(t * (1.0f - phi), a.inv_rho_r0, lrr);
         lrb = fmaf(-t * (1.0f + phi), a.inv_rho_b0, lrb);
     }
@@ -444,19 +488,99 @@ __device__ __forceinline__ void adj_collide_node(const StepArgs &a, const AdjArg
     g.rec_out.p[2][nb.n] = make_float4(lQxy, lQxz, lQyz, 0.0f);
 }
 
-#ifndef LBCM_ADJ_MIN_BLOCKS
-#define LBCM_ADJ_MIN_BLOCKS 3
-#endif
-template <bool kForce, bool W>
-__global__ void __launch_bounds__(128, LBCM_ADJ_MIN_BLOCKS) adj_collide_kernel(StepArgs a, AdjArgs g) {
+// Shared memory of a block of adj_collide_kernel: a ring of four planes of the tile's records, a_i and
+// b_i of every node of the plane in hand, and the forward step's record of that node.
+template <int TX>
+struct AdjSmem {
+    float4 ring[4][3 * AdjTile<TX>::kN];
+    float4 own[4][128];
+    float2 own2[128];
+    float2 ab[27 * 128];
+};
+
+// A block marches chunk planes of a tile of TX x 128 / TX columns upwards.  While a plane is worked on, the
+// tile's records of the plane after next and the own record of the next one arrive by cp.async.  What
+// bounds it is the latency of the node's arithmetic (1700 instructions in 158 registers, three warps a
+// scheduler; a fourth block an SM does not fit the registers), so memory is kept out of it: gathered
+// straight from memory, the 73 16-byte loads of a node were 40% of the stall cycles and moved 650 bytes a
+// node through L2.  64x64x256: 144 us gathered; 110 in the ring with a and b as pairs; 104 with the own
+// record fetched before the arithmetic; 98 without spills (load_q reads twice); 83 with the reciprocals
+// of lbcm_collide.cuh.
+template <bool kForce, bool W, int TX>
+__global__ void __launch_bounds__(128, 3) adj_collide_kernel(StepArgs a, AdjArgs g, int chunk) {
     chain_begin();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    __shared__ float2 adj_sm[27 * 128];  // a_i, b_i
-    const int t = threadIdx.y * 32 + threadIdx.x;
-    float part[3] = {0.0f, 0.0f, 0.0f};
-    if (x < a.nx && y < a.ny) adj_collide_node<kForce, W>(a, g, x, y, z, part, adj_sm + t);
+    extern __shared__ float4 adj_dsm[];
+    using T = AdjTile<TX>;
+    AdjSmem<TX> &S = *reinterpret_cast<AdjSmem<TX> *>(adj_dsm);
+    const int t = threadIdx.x, tx = t % TX, ty = t / TX, P = (int)a.plane;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * T::kTY, z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, a.nz);
+    const int x = x0 + tx, y = y0 + ty;
+    const bool live = x < a.nx && y < a.ny;
+    // this thread's two cells of the tile, wrapped or reflected at the sides as Nbr does; cells beyond
+    // the node after the last are never read
+    int cell0[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int c = t + 128 * k, xs = x0 - 1 + c % T::kX, ys = y0 - 1 + c / T::kX;
+        const int xw = a.wall_x ? min(max(xs, 0), a.nx - 1) : (xs < 0 ? a.nx - 1 : (xs < a.nx ? xs : 0));
+        const int yw = a.wall_y ? min(max(ys, 0), a.ny - 1) : (ys < 0 ? a.ny - 1 : (ys < a.ny ? ys : 0));
+        cell0[k] = yw * a.nx + xw;
+    }
+    auto fetch_plane = [&](int z) {  // z in [-1, nz]
+        int zs = z;
+        if (a.bc_zlo == BC_PERIODIC) zs = wrapi(z, a.nz);
+        zs = min(max(zs, 0), a.nz - 1);
+        float4 *dst = S.ring[(z + 1) & 3];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c = t + 128 * k;
+            if (c < T::kN) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) cp_async16(dst + q * T::kN + c, g.rec_in.p[q] + (size_t)zs * P + cell0[k]);
+            }
+        }
+    };
+    const size_t NN = (size_t)a.NN;
+    auto fetch_own = [&](int z) {
+        if (!live) return;
+        const size_t n = (size_t)z * P + (size_t)y * a.nx + x;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) cp_async16(&S.own[q][t], g.mom + q * NN + n);
+        cp_async16(&S.own[3][t], g.grad4 + n);
+        cp_async8(&S.own2[t], g.grad2 + n);
+    };
+    const bool gather = g.lr_obj == nullptr;
+    if (gather) {
+        fetch_plane(z0 - 1);
+        fetch_plane(z0);
+        fetch_plane(z0 + 1);
+    }
+    fetch_own(z0);
+    // parameter sums of this thread's column, compensated: the sum over a block keeps the rounding of a
+    // sum of one term a thread
+    float sum[3] = {0.0f, 0.0f, 0.0f}, low[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+    for (int z = z0; z < z1; ++z) {
+        cp_async_wait_all();
+        __syncthreads();  // plane z + 1 is there for every thread, and nobody reads plane z - 2 any more
+        if (gather && z + 1 < z1) fetch_plane(z + 2);
+        if (live) {
+            const Nbr nb(a, x, y, z);
+            const int c = (ty + 1) * T::kX + tx + 1;
+            const RecRing<TX> ring{{S.ring[z & 3] + c, S.ring[(z + 1) & 3] + c, S.ring[(z + 2) & 3] + c}};
+            float part[3] = {0.0f, 0.0f, 0.0f};
+            adj_collide_node<kForce, W>(a, g, nb, z, ring, reinterpret_cast<const float4 (*)[128]>(&S.own[0][t]), S.own2 + t, part, S.ab + t, [&] { if (z + 1 < z1) fetch_own(z + 1); });
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float s = sum[k] + part[k], bb = s - sum[k];
+                low[k] += (sum[k] - (s - bb)) + (part[k] - bb);
+                sum[k] = s;
+            }
+        }
+    }
+    float part[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) part[k] = sum[k] + low[k];
     block_accumulate<3>(part, g.acc_coll, block_id());
 }
 
@@ -743,7 +867,7 @@ __global__ void __launch_bounds__(256) adj_state_kernel(StepArgs a, AdjArgs g, f
         const bool own_in_disc = a.bc_zlo == BC_INLET && z == 0 && a.disc[nb.pxy];
 #pragma unroll
         for (int i = 0; i < 27; ++i) {
-            const float2 v = adj_slot<true, true>(a, g, nb, i, z, own_in_disc);
+            const float2 v = adj_slot<true, true>(a, g, RecNbr{g.rec_in, nb}, nb, i, z, own_in_disc);
             out[(size_t)i * a.NN + n] = v.x;
             out[(size_t)(27 + i) * a.NN + n] = v.y;
         }
@@ -765,22 +889,56 @@ long long adj_boundary_blocks(const StepArgs &a) {
     return (long long)gr.x * gr.y * gr.z;
 }
 
+static long long tile_columns(const StepArgs &a, int tx) {
+    return (long long)((a.nx + tx - 1) / tx) * ((a.ny + 128 / tx - 1) / (128 / tx));
+}
+// Tile width of the collide adjoint: 32, or 16 where that takes fewer tiles (an 80 x 80
+// plane: 50 against 60; a step of 80x80x300, forward and reverse, 473 -> 402 us).
+static int tile_width(const StepArgs &a) { return tile_columns(a, 16) < tile_columns(a, 32) ? 16 : 32; }
+
+// Planes a block of the collide adjoint marches: the length with the least estimated time.  A plane
+// takes 3.8 us where a block has an SM to itself and 6.0 us where three share it; starting a block
+// costs a tenth of a plane (the others on the SM hide it).  Step of 64x64x256 by length: 1 248 us, 5
+// 259, 10 251, 19 (chosen) 249, 32 327; of 25x23x60: 1 (chosen) 50, 2 56, 5 65.
+static int adj_chunk(const StepArgs &a, int tx) {
+    const long long cols = tile_columns(a, tx), slots = 3 * 152;
+    auto us = [&](long long blocks, int len) {
+        const long long r = blocks % slots;
+        return ((float)(blocks / slots) * 6.0f + (r ? 3.8f + 2.2f * (float)r / (float)slots : 0.0f)) * ((float)len + 0.1f);
+    };
+    int best = 1;
+    float cost = 1e30f;
+    for (int len = 1; len <= a.nz && len <= 64; ++len) {
+        const long long full = cols * (a.nz / len);
+        const int rest = a.nz % len;  // the last chunk; alongside the others where slots are left
+        const float t = us(full, len) + (rest && full % slots + cols > slots ? us(cols, rest) : 0.0f);
+        if (t < 0.985f * cost) { cost = t; best = len; }  // the shorter where it makes no difference
+    }
+    return best;
+}
+
+template <bool kForce, bool W, int TX>
+static cudaError_t launch_adj_collide(const StepArgs &a, const AdjArgs &g, cudaStream_t s) {
+    auto *fn = adj_collide_kernel<kForce, W, TX>;
+    const int smem = (int)sizeof(AdjSmem<TX>), chunk = adj_chunk(a, TX);
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 gr((a.nx + TX - 1) / TX, (a.ny + 128 / TX - 1) / (128 / TX), (a.nz + chunk - 1) / chunk);
+    launch_chained(fn, gr, dim3(128, 1, 1), smem, s, a, g, chunk);
+    return cudaSuccess;
+}
+template <int TX>
+static cudaError_t launch_adj_collide(const StepArgs &a, const AdjArgs &g, bool force, bool walls, cudaStream_t s) {
+    return force ? (walls ? launch_adj_collide<true, true, TX>(a, g, s) : launch_adj_collide<true, false, TX>(a, g, s))
+                 : (walls ? launch_adj_collide<false, true, TX>(a, g, s) : launch_adj_collide<false, false, TX>(a, g, s));
+}
+
 cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_t s, long long *launches) {
     const bool force = a.gx != 0.0f || a.gy != 0.0f || a.gz != 0.0f;
     const bool walls = a.wall_x || a.wall_y;
-    const dim3 gr = node_grid(a), bl = node_block();
-    if (force && walls)
-        launch_chained(adj_collide_kernel<true, true>, gr, bl, 0, s, a, g);
-    else if (force)
-        launch_chained(adj_collide_kernel<true, false>, gr, bl, 0, s, a, g);
-    else if (walls)
-        launch_chained(adj_collide_kernel<false, true>, gr, bl, 0, s, a, g);
-    else
-        launch_chained(adj_collide_kernel<false, false>, gr, bl, 0, s, a, g);
-    if (walls)
-        launch_chained(adj_stencil_kernel<true>, gr, bl, 0, s, a, g);
-    else
-        launch_chained(adj_stencil_kernel<false>, gr, bl, 0, s, a, g);
+    const cudaError_t e = tile_width(a) == 16 ? launch_adj_collide<16>(a, g, force, walls, s) : launch_adj_collide<32>(a, g, force, walls, s);
+    if (e != cudaSuccess) return e;
+    launch_chained(walls ? adj_stencil_kernel<true> : adj_stencil_kernel<false>, node_grid(a), node_block(), 0, s, a, g);
     *launches += 2;
     if (a.bc_zlo == BC_INLET || a.bc_zhi == BC_CONVECTIVE) {
         launch_chained(adj_boundary_kernel, col_grid(a), col_block(), 0, s, a, g);
@@ -806,10 +964,7 @@ cudaError_t launch_objective(const StepArgs &a, const AdjArgs &g, int objective,
         ao.phase = ph;
         const float eps = (float)args[0];
         obj_area_kernel<<<node_grid(a), node_block(), 0, s>>>(a, ph, g.lga, g.lgb, acc_obj, eps * eps);
-        if (a.wall_x || a.wall_y)
-            adj_stencil_kernel<true><<<node_grid(a), node_block(), 0, s>>>(ao, o);
-        else
-            adj_stencil_kernel<false><<<node_grid(a), node_block(), 0, s>>>(ao, o);
+        (a.wall_x || a.wall_y ? adj_stencil_kernel<true> : adj_stencil_kernel<false>)<<<node_grid(a), node_block(), 0, s>>>(ao, o);
         adj_reduce_kernel<<<1, 1024, 0, s>>>(acc_obj, nblk, 1, 0, scalar);
         *launches += 3;
     } else {  // penetration length
