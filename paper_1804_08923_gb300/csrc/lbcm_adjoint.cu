@@ -585,77 +585,104 @@ __global__ void __launch_bounds__(128, 3) adj_collide_kernel(StepArgs a, AdjArgs
 }
 
 // --------------------------------------------------- transposed gradient stencil (K3)
+// lambda_rho_k of node n from lambda_phi and lambda_rho.
+__device__ __forceinline__ void adj_stencil_out(const StepArgs &a, const AdjArgs &g, int n, float lphi, float lrho) {
+    float phv, S_;  // phi and rho_r/rho_r0 + rho_b/rho_b0 of this node
+    if (g.mom) {
+        const float4 r0 = __ldg(g.mom + n);  // (rho_r, rho_b, phi, jx)
+        phv = order_parameter(r0.x, r0.y, a.inv_rho_r0, a.inv_rho_b0);
+        S_ = r0.x * a.inv_rho_r0 + r0.y * a.inv_rho_b0;
+    } else {
+        const float2 ph = __ldg(a.phase + n);  // (phi, rho)
+        phv = ph.x;
+        S_ = ph.y / (a.rho_r0 * 0.5f * (1.0f + ph.x) + a.rho_b0 * 0.5f * (1.0f - ph.x));
+    }
+    const float t = lphi * rcp_newton(S_);
+    const float2 l = make_float2(fmaf(t * (1.0f - phv), a.inv_rho_r0, lrho), fmaf(-t * (1.0f + phv), a.inv_rho_b0, lrho));
+    if (g.mom) {  // a reverse step: into the record
+        float2 *r = reinterpret_cast<float2 *>(g.rec_out.p[0] + n);
+        const float2 d = *r;
+        *r = make_float2(d.x + l.x, d.y + l.y);
+    } else {
+        g.lr_out[n] = l;
+    }
+}
+
 // lambda_phi(y) = sum over the nodes x whose stencil reads y of 3 w_j c_j . lambda_gphi(x); a
 // node x on z = 0 (z = N) reads y through the mirror ghost with c_j's z component flipped,
 // except inside the inlet disc, where the ghost is a constant.  Same for rho.  Then
 // lambda_rho_k(y) = lambda_phi dphi/drho_k + lambda_rho.
-// The 52 neighbour loads are issued in two batches of 13 neighbours before they are used (the
-// loop with a use after every load kept few loads in flight and stalled on each); planes away
-// from z walls take the stencil's signs at compile time.
-template <bool W, bool kZWall>
-__device__ __forceinline__ void adj_stencil_sums(const StepArgs &a, const AdjArgs &g, const Nbr &nb, int z,
-                                                 float &lphi, float &lrho) {
-    const int N = a.nz - 1;
-    const bool pz = a.bc_zlo == BC_PERIODIC;
-    const bool lo_const = kZWall && !pz && z == 0 && a.bc_zlo == BC_INLET && a.disc[nb.pxy];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float4 A[13];
-        float2 B[13];
-#pragma unroll
-        for (int q = 0; q < 13; ++q) {
-            const int src = nb.src(1 + 13 * h + q);  // clamped onto the wall layer: the mirrored reader
-            A[q] = __ldg(g.lga + src);
-            B[q] = __ldg(g.lgb + src);
-        }
-#pragma unroll
-        for (int q = 0; q < 13; ++q) {
-            const int j = 1 + 13 * h + q;
-            const bool below = kZWall && !pz && z == 0 && cz(j) == 1;   // x = y - c_j would sit on z = -1
-            const bool above = kZWall && !pz && z == N && cz(j) == -1;  // ... on z = N + 1
-            // beyond a wall the reader is on this layer and reached y through its mirror ghost
-            // with that component of c reversed
-            const float czj = (below || above) ? -(float)cz(j) : (float)cz(j);
-            const float cxj = W && nb.fx(j) ? -(float)cx(j) : (float)cx(j);
-            const float cyj = W && nb.fy(j) ? -(float)cy(j) : (float)cy(j);
-            const float w3 = (below && lo_const) ? 0.0f : 3.0f * wgt(j);  // the disc ghost is a constant
-            lphi = fmaf(w3, cxj * A[q].x + cyj * A[q].y + czj * A[q].z, lphi);
-            lrho = fmaf(w3, cxj * A[q].w + cyj * B[q].x + czj * B[q].y, lrho);
-        }
-    }
-}
-
+// A thread marches chunk planes of its column.  The nine readers in a plane z enter the sums of z - 1,
+// z and z + 1 only as three numbers a field, so a plane's 18 loads are made once and not three times.
+struct StencilPart {
+    float2 in, xy, z;  // (phi, rho): sum for the plane itself; x, y and z terms for the planes next to it
+};
 template <bool W>
-__global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g) {
+__global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g, int chunk) {
     chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
     if (x >= a.nx || y >= a.ny) return;
-    const Nbr nb(a, x, y, z);
-    float lphi = 0.0f, lrho = 0.0f;
-    if (a.bc_zlo != BC_PERIODIC && (z == 0 || z == a.nz - 1))
-        adj_stencil_sums<W, true>(a, g, nb, z, lphi, lrho);
-    else
-        adj_stencil_sums<W, false>(a, g, nb, z, lphi, lrho);
-    float phv, S_;  // phi and rho_r/rho_r0 + rho_b/rho_b0 of this node
-    if (g.mom) {
-        const float4 r0 = __ldg(g.mom + nb.n);  // (rho_r, rho_b, phi, jx)
-        phv = order_parameter(r0.x, r0.y, a.inv_rho_r0, a.inv_rho_b0);
-        S_ = r0.x * a.inv_rho_r0 + r0.y * a.inv_rho_b0;
-    } else {
-        const float2 ph = __ldg(a.phase + nb.n);  // (phi, rho)
-        phv = ph.x;
-        S_ = ph.y / (a.rho_r0 * 0.5f * (1.0f + ph.x) + a.rho_b0 * 0.5f * (1.0f - ph.x));
-    }
-    const float t = lphi / S_;
-    const float2 l = make_float2(fmaf(t * (1.0f - phv), a.inv_rho_r0, lrho), fmaf(-t * (1.0f + phv), a.inv_rho_b0, lrho));
-    if (g.mom) {  // a reverse step: into the record
-        float2 *r = reinterpret_cast<float2 *>(g.rec_out.p[0] + nb.n);
-        const float2 d = *r;
-        *r = make_float2(d.x + l.x, d.y + l.y);
-    } else {
-        g.lr_out[nb.n] = l;
+    const int z0 = blockIdx.z * chunk, z1 = min(z0 + chunk, a.nz), N = a.nz - 1;
+    const bool pz = a.bc_zlo == BC_PERIODIC;
+    const Nbr nb(a, x, y, z0);
+    const bool lo_const = a.bc_zlo == BC_INLET && z0 == 0 && a.disc[nb.pxy];  // the disc ghost is a constant
+    auto plane = [&](int z) {
+        const size_t base = (size_t)z * (size_t)a.plane;
+        float4 A[9];
+        float2 B[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {  // the node x - c, clamped onto a side wall: the mirrored reader
+            const size_t n = base + nb.yo[q / 3] + nb.xo[q % 3];
+            A[q] = __ldg(g.lga + n);
+            B[q] = __ldg(g.lgb + n);
+        }
+        StencilPart o{{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int dx = q % 3 - 1, dy = q / 3 - 1, m = dx * dx + dy * dy;
+            // beyond a side wall the reader reached y through its mirror ghost with that component of c
+            // reversed
+            const float sx = W && (dx > 0 ? nb.wxl : dx < 0 && nb.wxh) ? -(float)dx : (float)dx;
+            const float sy = W && (dy > 0 ? nb.wyl : dy < 0 && nb.wyh) ? -(float)dy : (float)dy;
+            const float w0 = m == 1 ? 6.0f / 27.0f : 3.0f / 54.0f, w1 = m == 0 ? 6.0f / 27.0f : m == 1 ? 3.0f / 54.0f : 3.0f / 216.0f;
+            if (m > 0) {
+                const float tp = dx == 0 ? sy * A[q].y : dy == 0 ? sx * A[q].x : fmaf(sx, A[q].x, sy * A[q].y);
+                const float tr = dx == 0 ? sy * B[q].x : dy == 0 ? sx * A[q].w : fmaf(sx, A[q].w, sy * B[q].x);
+                o.in.x = fmaf(w0, tp, o.in.x);
+                o.in.y = fmaf(w0, tr, o.in.y);
+                o.xy.x = fmaf(w1, tp, o.xy.x);
+                o.xy.y = fmaf(w1, tr, o.xy.y);
+            }
+            o.z.x = fmaf(w1, A[q].z, o.z.x);
+            o.z.y = fmaf(w1, B[q].y, o.z.y);
+        }
+        return o;
+    };
+    StencilPart lo{}, cur = plane(z0), hi{};
+    if (z0 > 0 || pz) lo = plane(z0 > 0 ? z0 - 1 : N);
+#pragma unroll 1
+    for (int z = z0; z < z1; ++z) {
+        const int n = z * (int)a.plane + nb.pxy;
+        float lphi = cur.in.x, lrho = cur.in.y;
+        if (z < N || pz) {
+            hi = plane(z < N ? z + 1 : 0);
+            lphi += hi.xy.x - hi.z.x;
+            lrho += hi.xy.y - hi.z.y;
+        } else {  // beyond a wall the reader is on this layer, with the z component of c reversed
+            lphi += cur.xy.x + cur.z.x;
+            lrho += cur.xy.y + cur.z.y;
+        }
+        if (z > 0 || pz) {
+            lphi += lo.xy.x + lo.z.x;
+            lrho += lo.xy.y + lo.z.y;
+        } else if (!lo_const) {
+            lphi += cur.xy.x - cur.z.x;
+            lrho += cur.xy.y - cur.z.y;
+        }
+        adj_stencil_out(a, g, n, lphi, lrho);
+        lo = cur;
+        cur = hi;
     }
 }
 
@@ -892,7 +919,7 @@ long long adj_boundary_blocks(const StepArgs &a) {
 static long long tile_columns(const StepArgs &a, int tx) {
     return (long long)((a.nx + tx - 1) / tx) * ((a.ny + 128 / tx - 1) / (128 / tx));
 }
-// Tile width of the collide adjoint: 32, or 16 where that takes fewer tiles (an 80 x 80
+// Tile width of the collide adjoint and the stencil: 32, or 16 where that takes fewer tiles (an 80 x 80
 // plane: 50 against 60; a step of 80x80x300, forward and reverse, 473 -> 402 us).
 static int tile_width(const StepArgs &a) { return tile_columns(a, 16) < tile_columns(a, 32) ? 16 : 32; }
 
@@ -933,12 +960,27 @@ static cudaError_t launch_adj_collide(const StepArgs &a, const AdjArgs &g, bool 
                  : (walls ? launch_adj_collide<false, true, TX>(a, g, s) : launch_adj_collide<false, false, TX>(a, g, s));
 }
 
+// Grid of the stencil: a thread marches the longest chunk of 16, 8, 4, 2, 1 planes that leaves five
+// blocks an SM (a chunk reads two planes more than it writes).  Whole step of 64x64x256 by length: 1 245
+// us, 4 232, 8 (chosen) 231, 16 247; of 41x38x90: 1 (chosen) 77.5, 2 76.4, 4 79.5, 16 99.8.
+struct StencilGrid {
+    dim3 grid, block;
+    int chunk;
+    explicit StencilGrid(const StepArgs &a) : chunk(16) {
+        const int tx = tile_width(a), ty = 128 / tx;
+        while (chunk > 1 && tile_columns(a, tx) * ((a.nz + chunk - 1) / chunk) < 5 * 152) chunk /= 2;
+        block = dim3(tx, ty, 1);
+        grid = dim3((a.nx + tx - 1) / tx, (a.ny + ty - 1) / ty, (a.nz + chunk - 1) / chunk);
+    }
+};
+
 cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_t s, long long *launches) {
     const bool force = a.gx != 0.0f || a.gy != 0.0f || a.gz != 0.0f;
     const bool walls = a.wall_x || a.wall_y;
     const cudaError_t e = tile_width(a) == 16 ? launch_adj_collide<16>(a, g, force, walls, s) : launch_adj_collide<32>(a, g, force, walls, s);
     if (e != cudaSuccess) return e;
-    launch_chained(walls ? adj_stencil_kernel<true> : adj_stencil_kernel<false>, node_grid(a), node_block(), 0, s, a, g);
+    const StencilGrid sg(a);
+    launch_chained(walls ? adj_stencil_kernel<true> : adj_stencil_kernel<false>, sg.grid, sg.block, 0, s, a, g, sg.chunk);
     *launches += 2;
     if (a.bc_zlo == BC_INLET || a.bc_zhi == BC_CONVECTIVE) {
         launch_chained(adj_boundary_kernel, col_grid(a), col_block(), 0, s, a, g);
@@ -964,7 +1006,8 @@ cudaError_t launch_objective(const StepArgs &a, const AdjArgs &g, int objective,
         ao.phase = ph;
         const float eps = (float)args[0];
         obj_area_kernel<<<node_grid(a), node_block(), 0, s>>>(a, ph, g.lga, g.lgb, acc_obj, eps * eps);
-        (a.wall_x || a.wall_y ? adj_stencil_kernel<true> : adj_stencil_kernel<false>)<<<node_grid(a), node_block(), 0, s>>>(ao, o);
+        const StencilGrid sg(a);
+        (a.wall_x || a.wall_y ? adj_stencil_kernel<true> : adj_stencil_kernel<false>)<<<sg.grid, sg.block, 0, s>>>(ao, o, sg.chunk);
         adj_reduce_kernel<<<1, 1024, 0, s>>>(acc_obj, nblk, 1, 0, scalar);
         *launches += 3;
     } else {  // penetration length
