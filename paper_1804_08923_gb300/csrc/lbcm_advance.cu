@@ -9,7 +9,7 @@
 // sums the next moments.  lb_step(n) is one gather pass, n - 1 advances and one collision pass,
 // with the same bits as n gather and n collision passes.
 //
-// A block owns a 32 x TY tile of columns and a run of planes and marches along z.  Per plane k:
+// A block owns a TX x TY tile of columns and a run of planes and marches along z.  Per plane k:
 //   collide  a warp takes a row of the tile, its halo rows or its halo columns (of which only the nine
 //            populations that enter the tile are built), from prefetched moments and the gradients,
 //            and writes the populations to shared memory;
@@ -26,6 +26,7 @@
 // part of the collision before the second 22.4; both barriers split in two halves 21.5.  Two
 // population buffers and one barrier (32 x 11, 14 warps) 16.3 when the first form had 17.2.
 #include <algorithm>
+#include <iterator>
 #include <type_traits>
 
 #include "lbcm_collide.cuh"
@@ -35,19 +36,19 @@
 
 namespace lbcm {
 
-template <int TY>
+template <int TX, int TY>
 struct AdvanceTile {
-    static constexpr int BX = 34, RX = 36, RY = TY + 4;    // row of collided nodes, ring of phase nodes
+    static constexpr int BX = TX + 2, RX = TX + 4, RY = TY + 4;  // row of collided nodes, ring of phase nodes
     static constexpr int NB = BX * (TY + 2), NR = RX * RY;
-    // warps: TY rows of the tile, the two halo rows, the halo columns with the corners
-    static constexpr int NT = 32 * (TY + 2) + (2 * (TY + 2) + 31) / 32 * 32;
+    // threads: the nodes of the tile, the two halo rows, the halo columns with the corners, in whole warps
+    static constexpr int kRows = TX * TY, kHaloY = 2 * TX, NT = kRows + kHaloY + (2 * (TY + 2) + 31) / 32 * 32;
     // bytes: populations [27][NB] float2, moments [3][NT] float4, ring [4][NR] float2, inlet velocities [NB] float4
     static constexpr int kMom = (27 * NB * (int)sizeof(float2) + 15) / 16 * 16;
     static constexpr int kRing = kMom + 3 * NT * (int)sizeof(float4);
     static constexpr int kInflow = kRing + 4 * NR * (int)sizeof(float2);
     static constexpr int kBar = kInflow + NB * (int)sizeof(float4);
     static constexpr int kBytes = kBar + 16;
-    static_assert(kBytes <= 227 * 1024 && NR <= 2 * NT, "shared memory layout");
+    static_assert(kBytes <= 227 * 1024 && NR <= 2 * NT && kRows % 32 == 0 && kHaloY % 32 == 0, "layout");
 };
 
 template <int B>
@@ -93,10 +94,10 @@ __device__ __forceinline__ int pmod(int a, int n) {
     return r < 0 ? r + n : r;
 }
 
-template <bool kForce, bool W, int TY, int MB>
-__global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepArgs a, AdvanceArgs v) {
+template <bool kForce, bool W, int TX, int TY, int MB>
+__global__ void __launch_bounds__(AdvanceTile<TX, TY>::NT, MB) advance_kernel(StepArgs a, AdvanceArgs v) {
     chain_begin();
-    using T = AdvanceTile<TY>;
+    using T = AdvanceTile<TX, TY>;
     constexpr int BX = T::BX, RX = T::RX, NB = T::NB, NT = T::NT;
     extern __shared__ __align__(16) unsigned char smem[];
     float4 *mb = reinterpret_cast<float4 *>(smem + T::kMom);
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
 
     const int t = threadIdx.x;
     const int tile = blockIdx.x % v.tiles, chunk = blockIdx.x / v.tiles;
-    const int x0 = (tile % v.tiles_x) * 32, y0 = (tile / v.tiles_x) * TY;
+    const int x0 = (tile % v.tiles_x) * TX, y0 = (tile / v.tiles_x) * TY;
     const int nx = a.nx, ny = a.ny, N = a.nz - 1, P = (int)a.plane;
     const bool pz = a.bc_zlo == BC_PERIODIC, conv = a.bc_zhi == BC_CONVECTIVE;
     const int z0 = (int)((long long)v.planes * chunk / v.chunks), z1 = (int)((long long)v.planes * (chunk + 1) / v.chunks);
@@ -114,9 +115,10 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
 
     // the node this thread collides, at position (bx, by) of the tile with its halo, wrapped where
     // periodic; nothing lies beyond a side wall
-    const int warp = t >> 5, lane = t & 31, e = t - 32 * (TY + 2);
-    const bool row = warp < TY, halo_y = !row && warp < TY + 2;
-    const int bx = e < 0 ? lane + 1 : (e & 1 ? BX - 1 : 0), by = row ? warp + 1 : (halo_y ? (warp == TY ? 0 : TY + 1) : e >> 1);
+    const int line = t / TX, lane = t % TX, e = t - T::kRows - T::kHaloY;
+    const bool row = line < TY, halo_y = !row && line < TY + 2;  // warp-uniform
+    const int bx = e < 0 ? lane + 1 : (e & 1 ? BX - 1 : 0),
+              by = row ? line + 1 : (halo_y ? (line == TY ? 0 : TY + 1) : e >> 1);
     const float side = e < 0 ? (by == 0 ? 1.0f : -1.0f) : (bx == 0 ? 1.0f : -1.0f);  // halo: the component that enters
     int xs = x0 + bx - 1, ys = y0 + by - 1;
     const bool wx = W && a.wall_x, wy = W && a.wall_y;
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
     // comes from the wall node itself, with that velocity component reversed (half-way specular
     // reflection).  Blocks without wall nodes take the plain form.
     const bool wxl = wx && x == 0, wxh = wx && x == nx - 1, wyl = wy && y == 0, wyh = wy && y == ny - 1;
-    const bool walled = (wx && (x0 == 0 || x0 + 32 >= nx)) || (wy && (y0 == 0 || y0 + TY >= ny));
+    const bool walled = (wx && (x0 == 0 || x0 + TX >= nx)) || (wy && (y0 == 0 || y0 + TY >= ny));
     auto gather = [&](int k, float2 rest, auto wall) {
         constexpr bool kWall = decltype(wall)::value;
         auto fx = [&](int i) { return kWall && (cx(i) > 0 ? wxl : (cx(i) < 0 ? wxh : false)); };
@@ -319,13 +321,13 @@ __global__ void __launch_bounds__(AdvanceTile<TY>::NT, MB) advance_kernel(StepAr
 }
 
 // ------------------------------------------------------------------------ launchers
-template <bool kForce, bool W, int TY, int MB>
+template <bool kForce, bool W, int TX, int TY, int MB>
 static cudaError_t launch_tile(const StepArgs &a, AdvanceArgs v, int chunks, cudaStream_t s) {
-    using T = AdvanceTile<TY>;
-    auto *fn = advance_kernel<kForce, W, TY, MB>;
+    using T = AdvanceTile<TX, TY>;
+    auto *fn = advance_kernel<kForce, W, TX, TY, MB>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kBytes);
     if (e != cudaSuccess) return e;
-    v.tiles_x = (a.nx + 31) / 32;
+    v.tiles_x = (a.nx + TX - 1) / TX;
     v.tiles = v.tiles_x * ((a.ny + TY - 1) / TY);
     v.planes = a.bc_zhi == BC_CONVECTIVE ? a.nz - 1 : a.nz;
     v.chunks = std::min(chunks, v.planes);
@@ -336,32 +338,42 @@ static cudaError_t launch_tile(const StepArgs &a, AdvanceArgs v, int chunks, cud
     return launch_chained(fn, dim3((unsigned)v.tiles * v.chunks), dim3(T::NT), T::kBytes, s, a, v);
 }
 
-template <int TY, int MB>
-static cudaError_t launch_ty(const StepArgs &a, const AdvanceArgs &v, int chunks, cudaStream_t s) {
+template <int TX, int TY, int MB>
+static cudaError_t launch_shape(const StepArgs &a, const AdvanceArgs &v, int chunks, cudaStream_t s) {
     const bool force = a.gx != 0.0f || a.gy != 0.0f || a.gz != 0.0f;
     if (a.wall_x || a.wall_y)
-        return force ? launch_tile<true, true, TY, MB>(a, v, chunks, s) : launch_tile<false, true, TY, MB>(a, v, chunks, s);
-    return force ? launch_tile<true, false, TY, MB>(a, v, chunks, s) : launch_tile<false, false, TY, MB>(a, v, chunks, s);
+        return force ? launch_tile<true, true, TX, TY, MB>(a, v, chunks, s) : launch_tile<false, true, TX, TY, MB>(a, v, chunks, s);
+    return force ? launch_tile<true, false, TX, TY, MB>(a, v, chunks, s) : launch_tile<false, false, TX, TY, MB>(a, v, chunks, s);
 }
 
 constexpr int kSMs = 152;
 
-// Which tile and how many runs of planes: the estimated time of the last wave's end, with the
-// measured time a plane takes a resident block (us, 256 x 256 x 512 periodic, FP32): 3.15 for the
-// 32 x 16 tile (one block of 20 warps on an SM), 3.1 for the 32 x 7 tile (two blocks of 10 warps;
-// 1.9 when a block has the SM to itself).  They reach 22 and 20 G nodes/s on large lattices; the small
-// tile wastes less on planes that are no multiple of 16 rows and fills the chip with fewer columns.  A
-// run collides one plane more at each end, and about 12 us go into filling and draining it.
+// The tiles.  Per plane and resident block (us, from 256 x 256 x 512 periodic and the jets): 3.15 for
+// 32 x 16 (one block of 20 warps on an SM), 2.9 for 16 x 30 (18 warps), 2.85 for 16 x 14 (two blocks of
+// 9 warps; 1.9 when a block has the SM to itself).  They reach 21.7, 21.5 and 20.9 G nodes/s on that
+// lattice; the 16-wide ones waste less on extents that are no multiple of 32, and the smallest fills the
+// chip with fewer columns (it replaced 32 x 7, 10 warps for the same 224 nodes, 18.4).  Over lattices of
+// 48 to 192 nodes a side the estimate is 7% (up to 23%) below that of 32 x 16 and 32 x 7 alone; the
+// walled 120 x 120 x 600 jet takes 512 us a step in 16 x 30 and 530 in 32 x 16.
+struct TileShape {
+    int tx, ty, resident;
+    float plane_us, alone_us;
+};
+constexpr TileShape kShapes[] = {{32, 16, 1, 3.15f, 3.15f}, {16, 30, 1, 2.9f, 2.9f}, {16, 14, 2, 2.85f, 1.9f}};
+
+// Which tile and how many runs of planes: the least estimated time of the last wave's end.  A run
+// collides one plane more at each end, and about 12 us go into filling and draining it.
 AdvancePlan plan_advance(const StepArgs &a) {
     const int planes = a.bc_zhi == BC_CONVECTIVE ? a.nz - 1 : a.nz;
     AdvancePlan best{0, 1, 1e30f};
-    for (int ty : {16, 7}) {
-        const long long tiles = (long long)((a.nx + 31) / 32) * ((a.ny + ty - 1) / ty);
+    for (int k = 0; k < (int)std::size(kShapes); ++k) {
+        const TileShape &h = kShapes[k];
+        const long long tiles = (long long)((a.nx + h.tx - 1) / h.tx) * ((a.ny + h.ty - 1) / h.ty), slots = h.resident * kSMs;
         for (int chunks = 1; chunks <= planes && chunks <= 4 * kSMs; ++chunks) {
-            const long long blocks = tiles * chunks, slots = ty == 16 ? kSMs : 2 * kSMs;
-            const float plane_us = ty == 16 ? 3.15f : (blocks <= kSMs ? 1.9f : 3.1f);
-            const float us = (float)((blocks + slots - 1) / slots) * (float)((planes + chunks - 1) / chunks + 2) * plane_us + 12.0f;
-            if (us < best.us) best = AdvancePlan{ty, chunks, us};
+            const long long blocks = tiles * chunks;
+            const float us = (float)((blocks + slots - 1) / slots) * (float)((planes + chunks - 1) / chunks + 2) *
+                                 (blocks <= kSMs ? h.alone_us : h.plane_us) + 12.0f;
+            if (us < best.us) best = AdvancePlan{k, chunks, us};
         }
     }
     return best;
@@ -370,7 +382,11 @@ AdvancePlan plan_advance(const StepArgs &a) {
 cudaError_t launch_advance(const StepArgs &a, const AdvancePlan &p, const AdvanceArgs &v, cudaStream_t s,
                            long long *launches) {
     *launches += 1;
-    return p.ty == 16 ? launch_ty<16, 1>(a, v, p.chunks, s) : launch_ty<7, 2>(a, v, p.chunks, s);
+    switch (p.shape) {
+        case 0: return launch_shape<kShapes[0].tx, kShapes[0].ty, kShapes[0].resident>(a, v, p.chunks, s);
+        case 1: return launch_shape<kShapes[1].tx, kShapes[1].ty, kShapes[1].resident>(a, v, p.chunks, s);
+        default: return launch_shape<kShapes[2].tx, kShapes[2].ty, kShapes[2].resident>(a, v, p.chunks, s);
+    }
 }
 
 }  // namespace lbcm

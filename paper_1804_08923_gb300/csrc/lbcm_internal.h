@@ -45,9 +45,10 @@ struct AdvanceArgs {
     int *err;              // set if a wait inside the kernel ran out
     int tiles_x, tiles, planes, chunks;  // set by the launcher: column tiles, planes marched, runs of planes
 };
-// Tile rows and runs of planes of an advance, and its estimated time (us).
+// Tile shape (index into the list of lbcm_advance.cu) and runs of planes of an advance, and its estimated
+// time (us).
 struct AdvancePlan {
-    int ty, chunks;
+    int shape, chunks;
     float us;
 };
 AdvancePlan plan_advance(const StepArgs &a);
