@@ -372,7 +372,7 @@ def kernel_source_sha(kernel: str, src: str = None) -> str:
     unchanged."""
     import hashlib
     src = src or os.path.join(ROOT, "paper_1804_08923_gb300", "csrc")
-    units = KERNEL_SOURCES.get(kernel, ("lbcm_adjoint.cu",) if kernel.startswith("adj_") else ("lbcm_step.cu",))
+    units = KERNEL_SOURCES.get(kernel, ("lbcm_adjoint.cu",) if kernel.startswith("adj_") else ("lbcm_half.cu", "lbcm_step.cu"))
     h = hashlib.sha256()
     for f in sorted(os.listdir(src)):
         if f.endswith((".cuh", ".h")) or f in units:

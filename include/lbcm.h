@@ -261,7 +261,7 @@ LB_API lb_status lb_load(lb_ctx *ctx, const void *buf, size_t nbytes);
  * moments), phase_field_kernel otherwise; 2 the collision pass; 3 the fused step kernel, which
  * runs both passes in one launch (params.step_kernel = 1); 4 advance_kernel, which takes the
  * place of a collision pass and the next gather pass inside an lb_step call of several steps
- * (paper rates, FP32 and FP16 storage). */
+ * (paper rates, FP32 storage). */
 enum { LB_KERNEL_BOUNDARY = 0, LB_KERNEL_GATHER = 1, LB_KERNEL_COLLIDE = 2, LB_KERNEL_STEP = 3, LB_KERNEL_ADVANCE = 4,
        LB_NKERNELS = 5,
        LB_KERNEL_PHASE_FIELD = LB_KERNEL_GATHER };
@@ -294,7 +294,9 @@ LB_API lb_status lb_set_params(lb_ctx *ctx, const lb_params *params);
  * reverse-mode differentiation of the step of Section II with the boundaries of Section
  * IV.A, transposed by hand).  The forward pass runs T steps from the context's state,
  * keeping a checkpoint every k steps; the reverse pass recomputes each k-step segment from
- * its checkpoint and steps back through it, so device memory holds about T/k + k states.
+ * its checkpoint and steps back through it (k = T: every step recorded, none recomputed).  Device
+ * memory: T/k checkpoints of 216 bytes a node (k < T), records of 72 bytes a node for 2k steps (k for
+ * k = T), about 160 bytes a node besides.
  * Adjoint arithmetic is FP32, parameter gradients are accumulated in FP64.
  *
  * objective:

@@ -886,7 +886,7 @@ __global__ void obj_pen_value_kernel(const double *Z, double *out, double N, dou
     if (threadIdx.x == 0 && blockIdx.x == 0) out[0] = N + delta * log(*Z);
 }
 
-// dJ/dS(n) in the canonical layout [k][i][z][y][x] from the split adjoint state.
+// dJ/dS(n) in the canonical layout [k][i][z][y][x] from the records.
 __global__ void __launch_bounds__(256) adj_state_kernel(StepArgs a, AdjArgs g, float *out) {
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.NN; n += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(n % a.nx), y = (int)((n / a.nx) % a.ny), z = (int)(n / a.plane);

@@ -1010,7 +1010,7 @@ static cudaEvent_t *profile_record(lb_ctx *c, ProfKind kind) {
 // of through the populations: the paper's rates, FP32 storage and the default step kernel, where an
 // advance is estimated faster than the two passes it replaces.  Those run at 12.7 G nodes/s on large
 // lattices and take 6 us on the smallest (two dependent launches; 32^3: 8.5 us in all, against
-// 14 us for an advance, whose blocks collide three planes for each that they own), 3 us more where
+// 12 us for an advance, whose blocks collide three planes for each that they own), 3 us more where
 // boundary planes are computed first.
 static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
     const lb_params &p = c->p;

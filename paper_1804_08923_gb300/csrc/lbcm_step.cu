@@ -5,12 +5,12 @@
 //   1. boundary_plane_kernel  incoming z = 0 populations (inlet disc / free-slip mirror),
 //                             free-slip top, and the convective outflow plane
 //                             f(N, t+1) = [f(N, t) + lambda f(N-1, t+1)] / (1 + lambda)
-//                             (Section IV.A).  One warp per (x, y) column.
+//                             (Section IV.A).
 //   2. moment_kernel          pull-gathers the 54 post-stream populations of a node (the
 //                             step's only gather) and writes its order parameter phi
 //                             (Eq. (23)) and total density rho (Section II, densities) for
-//                             the gradient stencil, and the 12 moments the collision needs
-//                             (colour densities, mass, momentum, raw second moment).  One
+//                             the gradient stencil, and the moments the collision needs
+//                             (colour densities, phi, momentum, raw second moment).  One
 //                             thread per node.
 //   3. collide_kernel         reads a node's moments, takes the isotropic gradients of phi
 //                             and rho from the fields of step 2 (end of Section II), and
