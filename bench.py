@@ -510,7 +510,7 @@ def config_block(cfg, storage):
     nx, ny, nz = cfg["grid"]
     return {"workload": f"{cfg['name']}: {cfg['text']}", "lattice": [nx, ny, nz], "nodes": nx * ny * nz,
             "storage": {0: "fp32 SoA populations [i][z][y][x] of (red, blue) pairs"}.get(storage, STORAGE_TEXT.get(storage)),
-            "l2": "state >> 129 MB L2 (every population is read and written once per step); no flush between steps",
+            "l2": "state >> 129 MB L2 (every node's state is read and written once per step); no flush between steps",
             "parallelism": "one lattice per GPU (replicas, no exchange)"}
 
 
@@ -608,7 +608,7 @@ def main():
             "data": "synthetic", "config": config_block(cfg, st),
             "hbm_pct_of_peak": 100.0 * value * 1e6 * bytes_step / (peak[0] * 1e9) / world,
             "bytes_per_node_algorithmic": bytes_step,
-            "bytes_per_node_design": 2 * BYTES[st][1]["collide_kernel"] if st == 0 else
+            "bytes_per_node_design": BYTES[st][1]["advance_kernel"] if st == 0 else
             BYTES[st][1]["collide_kernel"] + BYTES[st][1]["moment_kernel"],
             "roofline": roofline, "kernels": kernels, "gpu_launches": launches, "clocks": clocks}
     if args.only_main:
