@@ -18,9 +18,10 @@
 //   gather   each thread of the tile reads the 27 pulls that come from plane k: c_z = -1 completes
 //            the node of plane k - 1, c_z = 0 is joined to plane k, c_z = +1 starts plane k + 1
 //            (z_class, join_classes, finish_moments; 22 registers hold the two open planes).
-// What bounds it: instruction issue and the shared-memory pipe, in turn rather than together (issue
-// slots 61%, FMA pipe 49%, shared memory 49% of the time; DRAM 103 bytes a node, a quarter of its
-// bandwidth), because the warps of a block go through the same phase at the same time.  Tried on
+// What bounds it: instruction issue and the shared-memory pipe, in turn rather than together (96 x 96 x
+// 384 jet: issue slots 71%, FMA pipe 55%, 1206 instructions a node with its share of the halo; DRAM 104
+// bytes a node, a third of its bandwidth), because the warps of a block go through the same phase at
+// the same time.  Tried on
 // 256 x 256 x 512, G nodes/s: 32 x 16 tile, 20 warps, a barrier after each phase 19.2; halo warps of
 // their own 20.2; gradient moved between arriving at and waiting on the first barrier, the scalar
 // part of the collision before the second 22.4; both barriers split in two halves 21.5.  Two
@@ -94,6 +95,11 @@ __device__ __forceinline__ int pmod(int a, int n) {
     return r < 0 ? r + n : r;
 }
 
+// The run that ends at a convective top computes the outflow after its march, as long as six planes take;
+// it gets that many fewer.  By that number of planes (us a step): 64x64x256 jet 0 72.5, 2 66.3, 4 60.8, 6
+// 56.5, 8 57.2; 96x96x384 jet 180, 177, 171, 167.0, 167.4; runs shorter than 8 planes stay equal.
+constexpr int kTail = 6;
+
 template <bool kForce, bool W, int TX, int TY, int MB>
 __global__ void __launch_bounds__(AdvanceTile<TX, TY>::NT, MB) advance_kernel(StepArgs a, AdvanceArgs v) {
     chain_begin();
@@ -109,7 +115,9 @@ __global__ void __launch_bounds__(AdvanceTile<TX, TY>::NT, MB) advance_kernel(St
     const int x0 = (tile % v.tiles_x) * TX, y0 = (tile / v.tiles_x) * TY;
     const int nx = a.nx, ny = a.ny, N = a.nz - 1, P = (int)a.plane;
     const bool pz = a.bc_zlo == BC_PERIODIC, conv = a.bc_zhi == BC_CONVECTIVE;
-    const int z0 = (int)((long long)v.planes * chunk / v.chunks), z1 = (int)((long long)v.planes * (chunk + 1) / v.chunks);
+    const int tail = conv && v.planes >= 8 * v.chunks ? kTail : 0;
+    auto cut = [&](int c) { return min((int)((long long)(v.planes + tail) * c / v.chunks), v.planes); };
+    const int z0 = cut(chunk), z1 = cut(chunk + 1);
     const bool top = !pz && z1 == v.planes;  // the run that ends at z = N (conv: planes = N)
     const int kb = pz ? z0 - 1 : max(z0 - 1, 0), ke = pz ? z1 : min(z1, N);
 
@@ -354,7 +362,7 @@ constexpr int kSMs = 152;
 // lattice; the 16-wide ones waste less on extents that are no multiple of 32, and the smallest fills the
 // chip with fewer columns (it replaced 32 x 7, 10 warps for the same 224 nodes, 18.4).  Over lattices of
 // 48 to 192 nodes a side the estimate is 7% (up to 23%) below that of 32 x 16 and 32 x 7 alone; the
-// walled 120 x 120 x 600 jet takes 512 us a step in 16 x 30 and 530 in 32 x 16.
+// walled 120 x 120 x 600 jet takes 507 us a step in 16 x 30 and 530 in 32 x 16.
 struct TileShape {
     int tx, ty, resident;
     float plane_us, alone_us;
