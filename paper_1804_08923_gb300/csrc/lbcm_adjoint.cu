@@ -585,27 +585,36 @@ __global__ void __launch_bounds__(128, 3) adj_collide_kernel(StepArgs a, AdjArgs
 }
 
 // --------------------------------------------------- transposed gradient stencil (K3)
-// lambda_rho_k of node n from lambda_phi and lambda_rho.
-__device__ __forceinline__ void adj_stencil_out(const StepArgs &a, const AdjArgs &g, int n, float lphi, float lrho) {
+// lambda_rho_k of node n from lambda_phi and lambda_rho; what it needs of the node is loaded ahead.
+struct StencilNode {
+    float4 r0;  // a reverse step: (rho_r, rho_b, phi, jx); the objective: (phi, rho, -, -)
+    float2 l;   // the record's (l_r, l_b)
+    __device__ __forceinline__ void load(const StepArgs &a, const AdjArgs &g, int n) {
+        if (g.mom) {
+            r0 = __ldg(g.mom + n);
+            l = *reinterpret_cast<const float2 *>(g.rec_out.p[0] + n);
+        } else {
+            const float2 ph = __ldg(a.phase + n);
+            r0 = make_float4(ph.x, ph.y, 0.0f, 0.0f);
+        }
+    }
+};
+__device__ __forceinline__ void adj_stencil_out(const StepArgs &a, const AdjArgs &g, int n, const StencilNode &s, float lphi,
+                                                float lrho) {
     float phv, S_;  // phi and rho_r/rho_r0 + rho_b/rho_b0 of this node
     if (g.mom) {
-        const float4 r0 = __ldg(g.mom + n);  // (rho_r, rho_b, phi, jx)
-        phv = order_parameter(r0.x, r0.y, a.inv_rho_r0, a.inv_rho_b0);
-        S_ = r0.x * a.inv_rho_r0 + r0.y * a.inv_rho_b0;
+        phv = order_parameter(s.r0.x, s.r0.y, a.inv_rho_r0, a.inv_rho_b0);
+        S_ = s.r0.x * a.inv_rho_r0 + s.r0.y * a.inv_rho_b0;
     } else {
-        const float2 ph = __ldg(a.phase + n);  // (phi, rho)
-        phv = ph.x;
-        S_ = ph.y / (a.rho_r0 * 0.5f * (1.0f + ph.x) + a.rho_b0 * 0.5f * (1.0f - ph.x));
+        phv = s.r0.x;
+        S_ = s.r0.y / (a.rho_r0 * 0.5f * (1.0f + phv) + a.rho_b0 * 0.5f * (1.0f - phv));
     }
     const float t = lphi * rcp_newton(S_);
     const float2 l = make_float2(fmaf(t * (1.0f - phv), a.inv_rho_r0, lrho), fmaf(-t * (1.0f + phv), a.inv_rho_b0, lrho));
-    if (g.mom) {  // a reverse step: into the record
-        float2 *r = reinterpret_cast<float2 *>(g.rec_out.p[0] + n);
-        const float2 d = *r;
-        *r = make_float2(d.x + l.x, d.y + l.y);
-    } else {
+    if (g.mom)  // into the record
+        *reinterpret_cast<float2 *>(g.rec_out.p[0] + n) = make_float2(s.l.x + l.x, s.l.y + l.y);
+    else
         g.lr_out[n] = l;
-    }
 }
 
 // lambda_phi(y) = sum over the nodes x whose stencil reads y of 3 w_j c_j . lambda_gphi(x); a
@@ -627,16 +636,24 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g,
     const bool pz = a.bc_zlo == BC_PERIODIC;
     const Nbr nb(a, x, y, z0);
     const bool lo_const = a.bc_zlo == BC_INLET && z0 == 0 && a.disc[nb.pxy];  // the disc ghost is a constant
-    auto plane = [&](int z) {
-        const size_t base = (size_t)z * (size_t)a.plane;
+    struct Readers {
         float4 A[9];
         float2 B[9];
+    };
+    auto load = [&](int z) {
+        const size_t base = (size_t)z * (size_t)a.plane;
+        Readers r;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {  // the node x - c, clamped onto a side wall: the mirrored reader
             const size_t n = base + nb.yo[q / 3] + nb.xo[q % 3];
-            A[q] = __ldg(g.lga + n);
-            B[q] = __ldg(g.lgb + n);
+            r.A[q] = __ldg(g.lga + n);
+            r.B[q] = __ldg(g.lgb + n);
         }
+        return r;
+    };
+    auto sums = [&](const Readers &r) {
+        const float4(&A)[9] = r.A;
+        const float2(&B)[9] = r.B;
         StencilPart o{{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
@@ -659,14 +676,16 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g,
         }
         return o;
     };
-    StencilPart lo{}, cur = plane(z0), hi{};
-    if (z0 > 0 || pz) lo = plane(z0 > 0 ? z0 - 1 : N);
+    StencilPart lo{}, cur = sums(load(z0)), hi{};
+    if (z0 > 0 || pz) lo = sums(load(z0 > 0 ? z0 - 1 : N));
 #pragma unroll 1
     for (int z = z0; z < z1; ++z) {
         const int n = z * (int)a.plane + nb.pxy;
+        StencilNode node;
+        node.load(a, g, n);
         float lphi = cur.in.x, lrho = cur.in.y;
         if (z < N || pz) {
-            hi = plane(z < N ? z + 1 : 0);
+            hi = sums(load(z < N ? z + 1 : 0));
             lphi += hi.xy.x - hi.z.x;
             lrho += hi.xy.y - hi.z.y;
         } else {  // beyond a wall the reader is on this layer, with the z component of c reversed
@@ -680,7 +699,7 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g,
             lphi += cur.xy.x - cur.z.x;
             lrho += cur.xy.y - cur.z.y;
         }
-        adj_stencil_out(a, g, n, lphi, lrho);
+        adj_stencil_out(a, g, n, node, lphi, lrho);
         lo = cur;
         cur = hi;
     }
