@@ -706,7 +706,8 @@ __global__ void __launch_bounds__(128) adj_stencil_kernel(StepArgs a, AdjArgs g,
 }
 
 // ----------------------------------------------- inlet gradients and outflow transpose
-// One warp per (x, y) column, lane i < 27 handling direction i (both colours).
+// One warp per (x, y) column and plane (blockIdx.y = 0: z = 0, 1: z = N), lane i < 27 handling direction i
+// (both colours).  Bound by the chain of its loads.
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -745,9 +746,9 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
         }
         const int q = cxi * cxi + cyi * cyi + czi * czi;
         const float w_i = q == 0 ? 8.0f / 27.0f : q == 1 ? 2.0f / 27.0f : q == 2 ? 1.0f / 54.0f : 1.0f / 216.0f;
-        if (a.bc_zlo == BC_INLET && lane < 27 && czi == 1) {
+        if (blockIdx.y == 0 && a.bc_zlo == BC_INLET && lane < 27 && czi == 1) {
+            const float lam = adj_pull_any(g.rec_out, pxy, cxi, cyi, czi).x;
             if (a.disc[(size_t)ys * a.nx + xs]) {
-                const float lam = adj_pull_any(g.rec_out, pxy, cxi, cyi, czi).x;
                 InletVel iv;
                 inlet_velocity(a.u_in, a.noise_amp, a.fourier, a.xc, a.yc, a.seed, a.step, xs, ys, a.nx, a.ny, iv);
                 const float c0 = (float)cxs, c1 = (float)cys, c2 = (float)czi;  // direction leaving the ghost
@@ -768,10 +769,16 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
                 }
             }
         }
-        if (a.bc_zhi == BC_CONVECTIVE) {
+        if (blockIdx.y == 1 && a.bc_zhi == BC_CONVECTIVE) {
             const int N = a.nz - 1;
-            float fr = 0.0f, fb = 0.0f;
-            if (lane < 27) {  // f(N-1) as the forward step pulled it
+            const size_t hr = (size_t)i * P + pxy, hb = (size_t)(27 + i) * P + pxy;
+            float fr = 0.0f, fb = 0.0f, lvr = 0.0f, lvb = 0.0f, hist_r = 0.0f, hist_b = 0.0f;
+            if (lane < 27) {  // f(N-1) as the forward step pulled it; every load before the sums
+                const float2 lN = adj_pull_any(g.rec_out, (size_t)N * P + pxy, cxi, cyi, czi);
+                lvr = lN.x + g.lh_in[hr];
+                lvb = lN.y + g.lh_in[hb];
+                hist_r = a.hist_out[hr];
+                hist_b = a.hist_out[hb];
                 fr = __ldg(g.fm + (size_t)i * P + pxy);
                 fb = __ldg(g.fm + (size_t)(27 + i) * P + pxy);
             }
@@ -781,15 +788,11 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
             const float lam_raw = (jz + 0.5f * Fz) / rho;
             const float lam = fminf(fmaxf(lam_raw, 0.0f), 1.0f);
             const float inv = 1.0f / (1.0f + lam);
-            float lvr = 0.0f, lvb = 0.0f, part_l = 0.0f;
-            const size_t hr = (size_t)i * P + pxy, hb = (size_t)(27 + i) * P + pxy;
+            float part_l = 0.0f;
             if (lane < 27) {
-                const float2 lN = adj_pull_any(g.rec_out, (size_t)N * P + pxy, cxi, cyi, czi);
-                lvr = lN.x + g.lh_in[hr];
-                lvb = lN.y + g.lh_in[hb];
                 g.lh_out[hr] = lvr * inv;
                 g.lh_out[hb] = lvb * inv;
-                part_l = fmaf(lvr, fr - a.hist_out[hr], lvb * (fb - a.hist_out[hb]));
+                part_l = fmaf(lvr, fr - hist_r, lvb * (fb - hist_b));
             }
             const float llam = warp_sum(part_l) * inv;
             if (lane < 27) {
@@ -1002,7 +1005,7 @@ cudaError_t launch_adjoint_step(const StepArgs &a, const AdjArgs &g, cudaStream_
     launch_chained(walls ? adj_stencil_kernel<true> : adj_stencil_kernel<false>, sg.grid, sg.block, 0, s, a, g, sg.chunk);
     *launches += 2;
     if (a.bc_zlo == BC_INLET || a.bc_zhi == BC_CONVECTIVE) {
-        launch_chained(adj_boundary_kernel, col_grid(a), col_block(), 0, s, a, g);
+        launch_chained(adj_boundary_kernel, dim3(col_grid(a).x, 2), col_block(), 0, s, a, g);
         *launches += 1;
     }
     return cudaGetLastError();

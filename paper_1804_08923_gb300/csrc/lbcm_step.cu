@@ -42,9 +42,9 @@ namespace lbcm {
 //   z = N free-slip top: the 9 incoming c_z = -1 populations -> zout
 //   z = N convective: hist(t+1) from hist(t) and the post-stream f(N-1, t+1) (Section IV.A)
 // Two kernels with the same results, bit for bit.
-// boundary_plane_kernel: one warp per (x, y) column, lane i < 27 handles direction i.  Many
-// warps with few instructions each: the faster of the two on planes of fewer than
-// kColumnKernelPlane columns.
+// boundary_plane_kernel: one warp per (x, y) column and plane (blockIdx.y = 0: z = 0, 1: z = N), lane
+// i < 27 handles direction i.  Many warps with few instructions each: the faster of the two on planes of
+// fewer than kColumnKernelPlane columns.
 __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
     chain_begin();
     const int lane = threadIdx.x & 31;
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
     }
     const int ii = dir_of(cxs, cys, czi);
 
-    if ((a.bc_zlo == BC_INLET || a.bc_zlo == BC_FREESLIP) && mine && czi == 1) {
+    if (blockIdx.y == 0 && (a.bc_zlo == BC_INLET || a.bc_zlo == BC_FREESLIP) && mine && czi == 1) {
         float vr, vb;
         if (a.bc_zlo == BC_INLET && a.disc[(long long)ys * a.nx + xs]) {
             vr = inlet_population_at(a, i, cxs, cys, xs, ys);
@@ -80,17 +80,20 @@ __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
         a.zin[(long long)zrank(i) * P + pxy] = vr;
         a.zin[(long long)(9 + zrank(i)) * P + pxy] = vb;
     }
-    if (a.bc_zhi == BC_FREESLIP && mine && czi == -1) {
+    if (blockIdx.y == 1 && a.bc_zhi == BC_FREESLIP && mine && czi == -1) {
         const float2 v = load_pop<STORE_FP32>(a, mirror_z(ii), (N * a.ny + ys) * a.nx + xs,
                                      no_shift());
         a.zout[(long long)zrank(i) * P + pxy] = v.x;
         a.zout[(long long)(9 + zrank(i)) * P + pxy] = v.y;
     }
-    if (a.bc_zhi == BC_CONVECTIVE) {
+    if (blockIdx.y == 1 && a.bc_zhi == BC_CONVECTIVE) {
         // post-stream populations of node (x, y, N-1) at t+1 (N-1 >= 1: plain pulls)
         const int z = N - 1;
-        float fr = 0.0f, fb = 0.0f;
+        float fr = 0.0f, fb = 0.0f, hist_r = 0.0f, hist_b = 0.0f;
+        const long long hr = (long long)i * P + pxy, hb = (long long)(27 + i) * P + pxy;
         if (mine) {
+            hist_r = __ldg(a.hist_in + hr);
+            hist_b = __ldg(a.hist_in + hb);
             const int zs = z - czi;
             const float2 v = load_pop<STORE_FP32>(a, ii, (zs * a.ny + ys) * a.nx + xs, no_shift());
             fr = v.x;
@@ -104,9 +107,8 @@ __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
         const float lam = outflow_lambda(a, moments_of(a, [&](int k) { return all[k]; }));
         const float inv = 1.0f / (1.0f + lam);
         if (mine) {
-            const long long hr = (long long)i * P + pxy, hb = (long long)(27 + i) * P + pxy;
-            a.hist_out[hr] = outflow_blend(__ldg(a.hist_in + hr), fr, lam, inv);
-            a.hist_out[hb] = outflow_blend(__ldg(a.hist_in + hb), fb, lam, inv);
+            a.hist_out[hr] = outflow_blend(hist_r, fr, lam, inv);
+            a.hist_out[hb] = outflow_blend(hist_b, fb, lam, inv);
             if (a.fm_out) {
                 a.fm_out[hr] = fr;
                 a.fm_out[hb] = fb;
@@ -208,7 +210,7 @@ static void launch_boundary(const StepArgs &a, cudaStream_t s) {
     if (a.plane >= kColumnKernelPlane)
         launch_chained(boundary_column_kernel, dim3((unsigned)((a.plane + 127) / 128)), dim3(128), 0, s, a);
     else
-        launch_chained(boundary_plane_kernel, dim3((unsigned)((a.plane + 3) / 4)), dim3(128), 0, s, a);
+        launch_chained(boundary_plane_kernel, dim3((unsigned)((a.plane + 3) / 4), 2), dim3(128), 0, s, a);
 }
 
 // ------------------------------------------- moment pass (K_A with the paper's rates)
