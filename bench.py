@@ -340,14 +340,14 @@ def adjoint_leg(lb, torch, name="jet64", T=500, objective="area", args=(1e-3,), 
     ev[3].record(lat.stream)
     torch.cuda.synchronize()
     fwd, adj = ev[0].elapsed_time(ev[1]), ev[2].elapsed_time(ev[3])
-    k = checkpoint if checkpoint > 0 else int(np.ceil(np.sqrt(T)))
     lat.close()
     del lat
     torch.cuda.empty_cache()
-    return {"workload": cfg["text"], "T": T, "checkpoint_interval": k, "objective": objective,
+    return {"workload": cfg["text"], "T": T, "checkpoint_interval": checkpoint or "automatic", "objective": objective,
             "objective_args": list(args), "J": J, "grad_norm": float(np.linalg.norm(g)),
             "forward_ms": fwd, "adjoint_ms": adj, "ratio": adj / fwd,
-            "work": "T forward steps with checkpoints + T recomputed forward steps + T reverse steps",
+            "work": "T forward steps, recorded, + T reverse steps; with checkpoints, where the records do not fit or an "
+                    "interval is given, also the recomputed segments",
             "precision": "FP32 kernels, FP64 parameter-gradient accumulation"}
 
 

@@ -307,8 +307,8 @@ LB_API lb_status lb_set_params(lb_ctx *ctx, const lb_params *params);
  *                          a smooth maximum of z over the red region (H = 1 in pure red, 0 in
  *                          pure blue); obj_args[0] = delta > 0.
  * obj_args[1] and obj_args[3] unused (0); obj_args[2] = checkpoint interval k (0: k = T, every step
- *   recorded and none recomputed, where the records (72 bytes a node and step) take no more than an
- *   eighth of the free device memory, else ceil(sqrt(T))).
+ *   recorded and none recomputed, where the records (72 bytes a node and step) take no more than a
+ *   sixth of the free device memory, else ceil(sqrt(T))).
  * grad_out (n_grad >= LB_ADJ_NOUT doubles): [0] J, [1] dJ/du_in, [2] dJ/dsigma, [3] dJ/dnu_r,
  *   [4] dJ/dnu_b, [5 + 2(m-1)] dJ/da_m, [6 + 2(m-1)] dJ/db_m for m = 1..8.
  * On return the context holds S(T) (as after lb_step(T)).  Requires FP32 storage and

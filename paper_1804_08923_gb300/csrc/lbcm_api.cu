@@ -1409,17 +1409,17 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         c->adj.bytes = need;
         return true;
     };
-    // k = 0: every step recorded where that takes no more than an eighth of the free device memory
+    // k = 0: every step recorded where that takes no more than a sixth of the free device memory
     // (what a previous call left allocated counts as free), else ceil(sqrt(T)).  The recompute that this
     // saves costs as much as the forward pass; run beside the reverse sweep it hid nothing (64x64x256
-    // jet, 50 steps: 20.2 ms with it).
+    // jet, 50 steps: 20.2 ms with it; 500 steps, 38 GB of records: 116 ms with it, 87 without).
     long long k = obj_args[2] >= 1 ? std::min<long long>((long long)obj_args[2], T) : 0;
     bool have = false;
     if (k == 0) {
         size_t free_b = 0, total_b = 0;
         LB_CUDA(cudaMemGetInfo(&free_b, &total_b));
         const size_t all = layout(T, parts);
-        have = all <= (free_b + c->adj.bytes) / 8 && allocate(all);
+        have = all <= (free_b + c->adj.bytes) / 6 && allocate(all);
         k = have ? T : std::max(1ll, std::min<long long>((long long)std::ceil(std::sqrt((double)T)), T));
     }
     const long long nseg = (T + k - 1) / k;
