@@ -12,8 +12,9 @@
 namespace lbcm {
 
 // 1/x and 1/sqrt(x) of normal positive x: the hardware approximation and one Newton step in FMA
-// arithmetic (within 2 ulp; three and five instructions where the IEEE forms take about ten, with
-// a branch for the special cases).
+// arithmetic, three and five instructions where the IEEE forms take about ten, with a branch for the
+// special cases.  Over every mantissa 1/x is the IEEE division's result; 1/sqrt(x) is off by at most 1
+// ulp, 0.33 rms (a division by the square root: 1.49 and 0.43).
 __device__ __forceinline__ float rcp_newton(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -197,7 +198,11 @@ struct Collision {
     template <bool kSecond>
     __device__ __forceinline__ float2 one(int i, float ev, float cu, float cF, float cgp, float sg, float r) const {
         const float od = odd(cu, cF), seg = sg * cgp;
-        const float s = fmaf(wgt(i), kSecond ? ev - od : ev + od, r);
+        // One rounding at the population's size, where ev + od would be rounded at that of rho.  Distance
+        // of u after one step from double precision, against a collision that adds even and odd part by
+        // direction, mean of seven scenes: 0.88 (0.97 with ev + od; 1.2 to 1.3 on a static droplet, whose
+        // velocities are below FP32 resolution either way).
+        const float s = fmaf(wgt(i), ev, fmaf(wgt(i), kSecond ? -od : od, r));
         return kSecond ? make_float2(fmaf(frac_r, s, -seg), fmaf(frac_b, s, seg))
                        : make_float2(fmaf(frac_r, s, seg), fmaf(frac_b, s, -seg));
     }

@@ -128,17 +128,26 @@ struct Moments {
 // marches along z and meets the classes of a node one plane after another (advance_kernel) gives
 // the same bits as one that holds all 27.  Within a class mirrored directions are subtracted
 // before they are added up, and the differences dxz and dyz are taken class by class, so that a
-// resting uniform node has exactly zero momentum and no second moment but its trace; the axis
-// population, the largest, is kept apart (a) from the others (b) until the classes c_z = +-1 are
-// subtracted.  The colour masses of a class are one running sum: at a density ratio of 1000 a node's
-// rest population holds all but 0.05% of its mass, FP32 resolves what moves only down to 6% of the
-// Laplace jump, and how a droplet settles depends on the association (100^3, R = 25, 1e5 steps, jump
-// off by 1.2% when all 13 pairs were added up in one sum, red and blue mass by -6e-5 and 1.3e-4; by
-// 1.3%, 1e-5 and 3e-5 with this order, by 3.5% with balanced trees).
+// resting uniform node has exactly zero momentum and no second moment but its trace.  The axis
+// population (a), the two pairs of faces (fx, fy) and the corners (k, with what the sums fx and fy
+// rounded off) are kept apart until the classes c_z = +-1 are subtracted: their differences are nearly
+// exact, where a class's sum is rounded at the size of the class.  Error of j_z of populations about
+// equilibrium, against that of differences taken pair by pair: 0.96 so, 1.14 without the
+// remainders in k, 1.64 with faces and corners added up in one sum, which made u_z after one step of a
+// jet 1.27 times as far from double precision.  The colour masses of a class are one running sum: at
+// a density ratio of 1000 a node's rest population holds all but 0.05% of its mass, FP32 resolves what
+// moves only down to 6% of the Laplace jump, and how a droplet settles depends on the association
+// (100^3, R = 25, 1e5 steps, jump off by 1.2% when all 13 pairs were added up in one sum, red and blue
+// mass by -6e-5 and 1.3e-4; by 1.2%, -5e-5 and 3e-5 with this order, by 3.5% with balanced trees).
 struct ZClass {
     float2 m;  // colour masses of the class's moving populations
-    float a, b, X, Y, XY;
-    float ex, ey;  // c_z = 0: the class's part of dxz, dyz; c_z = +-1: minus that part
+    float a, fx, fy, k, X, Y, XY;
+    __device__ __forceinline__ float b() const { return (fx + fy) + k; }
+    // c_z = 0: the class's part of dxz, dyz; c_z = +-1: minus that part
+    template <int cz>
+    __device__ __forceinline__ float ex() const { return cz == 0 ? fx + k : a + fy; }
+    template <int cz>
+    __device__ __forceinline__ float ey() const { return cz == 0 ? fy + k : a + fx; }
 };
 // at(i) is (red, blue) of direction i; cz = 0 leaves the rest direction out (a = 0).
 template <int cz, class L>
@@ -156,26 +165,30 @@ __device__ __forceinline__ ZClass z_class(L &&at) {
     }
     o.m = __fadd2_rn(__fadd2_rn(__fadd2_rn(o.m, v_x), vmy), vmx);
     o.m = __fadd2_rn(__fadd2_rn(__fadd2_rn(__fadd2_rn(o.m, v_k), v_q), vmk), vmq);
-    const float y0 = v_y.x + v_y.y, y1 = vmy.x + vmy.y, x0 = v_x.x + v_x.y, x1 = vmx.x + vmx.y;
+    const float y0 = v_y.x + v_y.y;
+    const float y1 = vmy.x + vmy.y;
+    const float x0 = v_x.x + v_x.y;
+    const float x1 = vmx.x + vmx.y;
     const float k0 = v_k.x + v_k.y, k1 = vmk.x + vmk.y, q0 = v_q.x + v_q.y, q1 = vmq.x + vmq.y;
-    const float fx = x0 + x1, fy = y0 + y1, ks = k0 + k1, qs = q0 + q1, kk = ks + qs;
-    const float kd = k0 - k1, qd = q0 - q1;
-    o.b = (fx + fy) + kk;
+    const float ks = k0 + k1, qs = q0 + q1, kd = k0 - k1, qd = q0 - q1;
+    o.fx = x0 + x1;
+    o.fy = y0 + y1;
+    o.k = ks + qs;
+    // what x0 + x1 and y0 + y1 rounded off (x0 and x1 lie within a factor of two, so it is exact)
+    if constexpr (cz != 0) o.k += (x1 - (o.fx - x0)) + (y1 - (o.fy - y0));
     o.X = (x0 - x1) + (kd + qd);
     o.Y = (y0 - y1) + (kd - qd);
     o.XY = ks - qs;
-    o.ex = cz == 0 ? fx + kk : o.a + fy;
-    o.ey = cz == 0 ? fy + kk : o.a + fx;
     return o;
 }
 // The classes c_z = +1 and 0 of a node, and its rest population.
 struct HalfNode {
     float2 f0, m;
-    float a, b, X, Y, jx, jy, dx, dy, XY;
+    float a, fx, fy, k, X, Y, jx, jy, dx, dy, XY;
 };
 __device__ __forceinline__ HalfNode join_classes(const ZClass &p, const ZClass &o, float2 f0) {
-    return HalfNode{f0,       __fadd2_rn(o.m, p.m), p.a,         p.b,         p.X,        p.Y,
-                    o.X + p.X, o.Y + p.Y,            o.ex - p.ex, o.ey - p.ey, o.XY + p.XY};
+    return HalfNode{f0,        __fadd2_rn(o.m, p.m), p.a, p.fx, p.fy, p.k, p.X, p.Y,
+                    o.X + p.X, o.Y + p.Y, o.ex<0>() - p.ex<1>(), o.ey<0>() - p.ey<1>(), o.XY + p.XY};
 }
 // All 27: the colour masses are f_0 + ((class 0 + class +1) + class -1), the association in which
 // the collision sums the moving populations it writes before it takes the rest population as the
@@ -188,10 +201,10 @@ __device__ __forceinline__ Moments finish_moments(const StepArgs &a, const HalfN
     m.phi = order_parameter(rho.x, rho.y, a.inv_rho_r0, a.inv_rho_b0);
     m.jx = h.jx + n.X;
     m.jy = h.jy + n.Y;
-    m.jz = (h.a - n.a) + (h.b - n.b);
-    m.dxz = h.dx - n.ex;
-    m.dyz = h.dy - n.ey;
-    m.pzz = (h.a + n.a) + (h.b + n.b);
+    m.jz = (h.a - n.a) + (((h.fx - n.fx) + (h.fy - n.fy)) + (h.k - n.k));
+    m.dxz = h.dx - n.ex<-1>();
+    m.dyz = h.dy - n.ey<-1>();
+    m.pzz = (h.a + n.a) + (((h.fx + h.fy) + h.k) + n.b());
     m.pxy = h.XY + n.XY;
     m.pxz = h.X - n.X;
     m.pyz = h.Y - n.Y;
