@@ -812,17 +812,14 @@ __global__ void __launch_bounds__(128) adj_boundary_kernel(StepArgs a, AdjArgs g
 }
 
 // ------------------------------------------------------------------- objectives
-// (phi, rho) of a post-collision state: rho_k = sum_i S_i^k.
+// (phi, rho) of a post-collision state: rho_k = sum_i S_i^k, as the collision summed.
 __global__ void __launch_bounds__(256) obj_fields_kernel(StepArgs a, float2 *ph) {
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.NN; n += (long long)gridDim.x * blockDim.x) {
-        MassAcc mr, mb;
+        float2 f[27];
 #pragma unroll
-        for (int i = 0; i < 27; ++i) {
-            const float2 v = load_pop<STORE_FP32>(a, i, (int)n, no_shift());
-            mr.add(i, v.x);
-            mb.add(i, v.y);
-        }
-        const float rr = mr.total(), rb = mb.total();
+        for (int i = 0; i < 27; ++i) f[i] = load_pop<STORE_FP32>(a, i, (int)n, no_shift());
+        const float2 s = moving_mass([&](int i) { return f[i]; });
+        const float rr = f[0].x + s.x, rb = f[0].y + s.y;
         ph[n] = make_float2(order_parameter(rr, rb, a.inv_rho_r0, a.inv_rho_b0), rr + rb);
     }
 }

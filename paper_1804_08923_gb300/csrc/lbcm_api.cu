@@ -14,6 +14,7 @@
 #include "lbcm.h"
 #include "lbcm_device.cuh"
 #include "lbcm_internal.h"
+#include "lbcm_node.cuh"
 
 namespace {
 
@@ -181,7 +182,8 @@ namespace lbcm {
 
 // ------------------------------------------------------------ initial populations
 // f_i^k = rho_k [varphi_i(alpha_k) + w_i P(c_i.u, u^2)]  (Eq. (18) per colour, Phi = 0); the
-// rest population takes each colour's remainder of the stored moving ones.
+// rest population takes each colour's remainder of the stored moving ones, summed as the step's
+// readers will sum them (kPaper: FP32 storage and the paper's rates).
 struct InitArgs {
     float *hist;
     const float *fr, *fb, *fu;
@@ -243,7 +245,7 @@ __global__ void init_phase_kernel(InitArgs ia, StepArgs sa) {
     }
 }
 
-template <int S>
+template <int S, bool kPaper>
 __global__ void init_kernel(InitArgs ia, StepArgs sa) {
     const long long NN = sa.NN;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < NN; n += (long long)gridDim.x * blockDim.x) {
@@ -252,6 +254,7 @@ __global__ void init_kernel(InitArgs ia, StepArgs sa) {
         const Nbr nb = node_nbr(sa, n);
         const float usq = ux * ux + uy * uy + uz * uz;
         MassAcc sr, sb;
+        float2 moving[27];
         const bool top = nb.zo[1] == (ia.nz - 1) * (int)sa.plane;
         const long long h = nb.pxy, P = sa.plane;
 #pragma unroll
@@ -261,14 +264,20 @@ __global__ void init_kernel(InitArgs ia, StepArgs sa) {
             const float2 f = make_float2(rr * (varphi(i, ia.alpha_r, ia.oma_r) + pw),
                                          rb * (varphi(i, ia.alpha_b, ia.oma_b) + pw));
             const float2 d = store_pop<S>(sa, i, (int)n, f, dest_shift<S>(sa, nb, i));
-            sr.add(i, d.x);
-            sb.add(i, d.y);
+            if constexpr (kPaper) {
+                moving[i] = d;
+            } else {
+                sr.add(i, d.x);
+                sb.add(i, d.y);
+            }
             if (top) {
                 ia.hist[(long long)i * P + h] = d.x;
                 ia.hist[(long long)(27 + i) * P + h] = d.y;
             }
         }
-        const float2 f0 = make_float2(rr - sr.s, rb - sb.s);
+        float2 s = make_float2(sr.s, sb.s);
+        if constexpr (kPaper) s = moving_mass([&](int i) { return moving[i]; });
+        const float2 f0 = make_float2(rr - s.x, rb - s.y);
         store_pop<S>(sa, 0, (int)n, f0, no_shift());
         if (top) {
             ia.hist[h] = f0.x;
@@ -282,13 +291,14 @@ struct FieldOut {
     float *o[LB_NFIELDS];
 };
 
-template <int S>
-__global__ void fields_kernel(StepArgs sa, FieldOut fo, float gx, float gy, float gz) {
+// Densities are summed as the collision that wrote the state took its rest populations (kPaper: FP32
+// storage and the paper's rates), so that the fields are the densities of the step, to the bit.
+template <int S, bool kPaper>
+__global__ void __launch_bounds__(256) fields_kernel(StepArgs sa, FieldOut fo, float gx, float gy, float gz) {
     chain_begin();
     const long long NN = sa.NN;
     for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < NN; n += (long long)gridDim.x * blockDim.x) {
-        MassAcc mr, mb;
-        float jx = 0.0f, jy = 0.0f, jz = 0.0f;
+        float rr, rb, jx = 0.0f, jy = 0.0f, jz = 0.0f;
         float2 f[27];
         if constexpr (S == STORE_FP32) {  // all loads in flight before the first sum
 #pragma unroll
@@ -298,16 +308,24 @@ __global__ void fields_kernel(StepArgs sa, FieldOut fo, float gx, float gy, floa
 #pragma unroll
             for (int i = 0; i < 27; ++i) f[i] = stored_pop<S>(sa, nb, i);
         }
+        if constexpr (kPaper) {
+            const Moments m = moments_of(sa, [&](int i) { return f[i]; });
+            rr = m.rho_r; rb = m.rho_b;
+            jx = m.jx; jy = m.jy; jz = m.jz;
+        } else {
+            MassAcc mr, mb;
 #pragma unroll
-        for (int i = 0; i < 27; ++i) {
-            const float2 v = f[i];
-            mr.add(i, v.x);
-            mb.add(i, v.y);
-            if (cx(i) != 0) jx += cx(i) * (v.x + v.y);
-            if (cy(i) != 0) jy += cy(i) * (v.x + v.y);
-            if (cz(i) != 0) jz += cz(i) * (v.x + v.y);
+            for (int i = 0; i < 27; ++i) {
+                const float2 v = f[i];
+                mr.add(i, v.x);
+                mb.add(i, v.y);
+                if (cx(i) != 0) jx += cx(i) * (v.x + v.y);
+                if (cy(i) != 0) jy += cy(i) * (v.x + v.y);
+                if (cz(i) != 0) jz += cz(i) * (v.x + v.y);
+            }
+            rr = mr.total();
+            rb = mb.total();
         }
-        const float rr = mr.total(), rb = mb.total();
         const float rho = rr + rb;
         const float phi = order_parameter(rr, rb, sa.inv_rho_r0, sa.inv_rho_b0);
         const float fc = rho - sa.rho_b0;
@@ -464,6 +482,8 @@ namespace {
 
 using namespace lbcm;
 
+
+bool paper_rates(const lb_params &p) { return p.s3 == 1.0 && p.s4 == 1.0 && p.s5 == 1.0 && p.s6 == 1.0; }
 
 // Inlet disc membership for the current d_in, and cleared boundary planes.
 lb_status upload_disc(lb_ctx *c) {
@@ -803,14 +823,14 @@ lb_status lb_init(lb_ctx *c, int32_t kind, const double *args, int32_t nargs, co
                 a[0], a[1], a[2], a[3], a[4], sa.rho_r0, sa.rho_b0, sa.alpha_r, sa.alpha_b, sa.oma_r, sa.oma_b};
     if (c->p.storage == LB_STORE_FP16) {
         init_phase_kernel<STORE_FP16><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
-        init_kernel<STORE_FP16><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
+        init_kernel<STORE_FP16, false><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
         c->launches += 2;
     } else if (c->p.storage == LB_STORE_FP16_FIT) {
         init_phase_kernel<STORE_FP16_FIT><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
-        init_kernel<STORE_FP16_FIT><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
+        init_kernel<STORE_FP16_FIT, false><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
         c->launches += 2;
     } else {
-        init_kernel<STORE_FP32><<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
+        (paper_rates(c->p) ? init_kernel<STORE_FP32, true> : init_kernel<STORE_FP32, false>)<<<grid_for(c->nn, 256), 256, 0, c->stream>>>(ia, sa);
         c->launches += 1;
     }
     LB_CUDA(cudaGetLastError());
@@ -824,7 +844,7 @@ lb_status lb_init(lb_ctx *c, int32_t kind, const double *args, int32_t nargs, co
 // Whether lb_step runs the fused step kernel: selected (step_kernel = 1) and the paper's rates.
 static bool use_fused(const lb_ctx *c) {
     const lb_params &p = c->p;
-    return p.step_kernel == 1 && p.s3 == 1.0 && p.s4 == 1.0 && p.s5 == 1.0 && p.s6 == 1.0;
+    return p.step_kernel == 1 && paper_rates(p);
 }
 
 // A collision item of the fused kernel comes kFusedLeadPct / 100 rounds of the grid's blocks
@@ -1014,7 +1034,7 @@ static cudaEvent_t *profile_record(lb_ctx *c, ProfKind kind) {
 // boundary planes are computed first.
 static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
     const lb_params &p = c->p;
-    if (p.step_kernel != 0 || p.storage != LB_STORE_FP32 || p.s3 != 1.0 || p.s4 != 1.0 || p.s5 != 1.0 || p.s6 != 1.0) return false;
+    if (p.step_kernel != 0 || p.storage != LB_STORE_FP32 || !paper_rates(p)) return false;
     *plan = plan_advance(a);
     const bool planes = c->g.bc_zlo != LB_BC_PERIODIC || c->g.bc_zhi != LB_BC_PERIODIC;
     return plan->us < 6.0f + (planes ? 3.0f : 0.0f) + 7.87e-5f * (float)c->nn;
@@ -1137,11 +1157,11 @@ lb_status lb_fields(lb_ctx *c, uint32_t mask, float *const *outs, int32_t on_dev
     FieldOut fo;
     for (int j = 0; j < LB_NFIELDS; ++j) fo.o[j] = dst[j];
     if (c->p.storage == LB_STORE_FP16)
-        launch_chained(fields_kernel<STORE_FP16>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(fields_kernel<STORE_FP16, false>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     else if (c->p.storage == LB_STORE_FP16_FIT)
-        launch_chained(fields_kernel<STORE_FP16_FIT>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(fields_kernel<STORE_FP16_FIT, false>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     else
-        launch_chained(fields_kernel<STORE_FP32>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
+        launch_chained(paper_rates(c->p) ? fields_kernel<STORE_FP32, true> : fields_kernel<STORE_FP32, false>, dim3(grid_for(c->nn, 256)), dim3(256), 0, c->stream, sa, fo, sa.gx, sa.gy, sa.gz);
     c->launches += 1;
     LB_CUDA(cudaGetLastError());
     if (!on_device) {
@@ -1354,7 +1374,7 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     if (!c->initialized) return fail(LB_ESTATE, "lb_adjoint before lb_init/lb_load");
     if (c->half) return fail(LB_ESTATE, "lb_adjoint inside a split step");
     if (c->p.storage != LB_STORE_FP32) return fail(LB_EINVAL, "lb_adjoint needs FP32 population storage");
-    if (c->p.s3 != 1.0 || c->p.s4 != 1.0 || c->p.s5 != 1.0 || c->p.s6 != 1.0)
+    if (!paper_rates(c->p))
         return fail(LB_EINVAL, "lb_adjoint needs the paper's rates s3 = s4 = s5 = s6 = 1");
     if (T < 1) return fail(LB_EINVAL, "T must be >= 1");
     if (n_grad < LB_ADJ_NOUT) return fail(LB_EINVAL, "grad_out must hold LB_ADJ_NOUT doubles");

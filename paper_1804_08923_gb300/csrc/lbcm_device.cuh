@@ -171,9 +171,11 @@ __device__ __forceinline__ float one_minus_alpha_bar(int mix, float rho_r, float
 
 // Sum of one colour's 27 populations of a node in one fixed association,
 //   f_0 + (((f_1 + f_2) + (f_3 + f_4)) + ... + (f_25 + f_26)),
-// the one the collision uses when it writes the rest population as the remainder rho_k - s of
-// the moving ones.  A reader that gathers the same moving values therefore gets rho_k back
-// (fl(fl(rho - s) + s) = rho up to a rounding tie), so a uniform state is an exact fixed point
+// the one the collision of the half-precision storages and of rates other than the paper's uses when it
+// writes the rest population as the remainder rho_k - s of the moving ones (the FP32 collision with
+// the paper's rates has its own, z_class and finish_moments of lbcm_node.cuh).  A reader that adds the
+// same moving values up in the writer's order therefore gets rho_k back (fl(fl(rho - s) + s) = rho
+// up to a rounding tie), so a uniform state is an exact fixed point
 // of the FP32 step instead of drifting by an ulp of density now and then; a drift that, being
 // the same at every node, would not average out and, against the frozen convective plane,
 // would drive a spurious outflow velocity.  add(i, v) must be called in the order i = 0..26

@@ -210,6 +210,11 @@ __device__ __forceinline__ Moments finish_moments(const StepArgs &a, const HalfN
     m.pyz = h.Y - n.Y;
     return m;
 }
+// Colour masses of the 26 moving populations in that association.
+template <class L>
+__device__ __forceinline__ float2 moving_mass(L &&at) {
+    return __fadd2_rn(__fadd2_rn(z_class<0>(at).m, z_class<1>(at).m), z_class<-1>(at).m);
+}
 template <class L>
 __device__ __forceinline__ Moments moments_of(const StepArgs &a, L &&at) {
     return finish_moments(a, join_classes(z_class<1>(at), z_class<0>(at), at(0)), z_class<-1>(at));
