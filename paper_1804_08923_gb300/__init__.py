@@ -156,8 +156,15 @@ class Lattice:
     def selftest_fused_wait(self):
         """Runs the fused step kernel's plane wait against a target nothing reaches (lb_selftest):
         returns (status the host read, milliseconds the wait lasted)."""
+        return self._selftest(_abi.SELFTEST_FUSED_WAIT)
+
+    def selftest_advance_wait(self):
+        """The same of the barrier wait inside the kernel that takes several steps of one call."""
+        return self._selftest(_abi.SELFTEST_ADVANCE_WAIT)
+
+    def _selftest(self, which):
         res, ms = C.c_int32(), C.c_double()
-        _abi.check(self.lib.lb_selftest(self._ctx, _abi.SELFTEST_FUSED_WAIT, C.byref(res), C.byref(ms)))
+        _abi.check(self.lib.lb_selftest(self._ctx, which, C.byref(res), C.byref(ms)))
         return int(res.value), float(ms.value)
 
     @property

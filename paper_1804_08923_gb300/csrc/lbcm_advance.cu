@@ -63,25 +63,45 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Barrier of the block's warps in two halves: a warp arrives when it has written what it shares, goes
-// on with work of its own and waits when it needs the others'.  The wait is bounded; a wait that runs
-// out (none does while every warp arrives once a phase) sets *err and goes on.
+// on with work of its own and waits when it needs the others'.  The wait is bounded by the number of
+// tries (1.4 us each when they fail); a wait that runs out (none does while every warp arrives once a
+// phase) sets *err and the word after the barrier and goes on, and later waits of the block that find
+// that word set try once.
+constexpr int kWaitTries = 1 << 20;  // 1.5 s
 __device__ __forceinline__ void warps_init(unsigned bar, int warps) {
     asm volatile("mbarrier.init.shared.b64 [%0], %1;\n" ::"r"(bar), "r"(warps) : "memory");
+    asm volatile("st.shared.u32 [%0 + 8], 0;\n" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void warps_arrive(unsigned bar) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void warps_wait(unsigned bar, int phase, int *err) {
-    for (int n = 0; n < (1 << 22); ++n) {
-        unsigned done;
+__device__ __forceinline__ void warps_wait(unsigned bar, int phase, int *err, int tries = kWaitTries) {
+    for (int n = 0; n < tries; ++n) {
+        unsigned done, given_up;
         asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                      : "=r"(done)
                      : "r"(bar), "r"(phase & 1)
                      : "memory");
         if (done) return;
+        asm volatile("ld.volatile.shared.u32 %0, [%1 + 8];\n" : "=r"(given_up) : "r"(bar) : "memory");
+        if (given_up) return;
     }
     *err = 1;
+    asm volatile("st.volatile.shared.u32 [%0 + 8], 1;\n" ::"r"(bar) : "memory");
+}
+
+// That wait on a barrier at which only one of two warps arrives, twice; *ns receives the time both took.
+__global__ void __launch_bounds__(64) advance_wait_probe_kernel(int *err, int tries, unsigned long long *ns) {
+    __shared__ __align__(16) unsigned char smem[16];
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(smem);
+    if (threadIdx.x == 0) warps_init(bar, 2);
+    __syncthreads();
+    const unsigned long long t0 = global_ns();
+    if (threadIdx.x < 32) warps_arrive(bar);
+    warps_wait(bar, 0, err, tries);
+    warps_wait(bar, 0, err, tries);
+    if (threadIdx.x == 0) *ns = global_ns() - t0;
 }
 
 // Barrier of the whole block that the warps may reach at different places of the code.
@@ -329,6 +349,11 @@ __global__ void __launch_bounds__(AdvanceTile<TX, TY>::NT, MB) advance_kernel(St
 }
 
 // ------------------------------------------------------------------------ launchers
+cudaError_t launch_advance_wait_probe(int *err, int tries, unsigned long long *ns, cudaStream_t s) {
+    advance_wait_probe_kernel<<<1, 64, 0, s>>>(err, tries, ns);
+    return cudaGetLastError();
+}
+
 template <bool kForce, bool W, int TX, int TY, int MB>
 static cudaError_t launch_tile(const StepArgs &a, AdvanceArgs v, int chunks, cudaStream_t s) {
     using T = AdvanceTile<TX, TY>;

@@ -613,6 +613,21 @@ StepArgs state_args(const lb_ctx *c) {
     return a;
 }
 
+// Reads and clears the flag that a bounded wait inside a step kernel sets when it runs out, with what the
+// stream holds before it; the call that reads results back synchronises with this.
+lb_status settle_flag(lb_ctx *c, int err) {
+    if (!err) return LB_OK;
+    LB_CUDA(cudaMemsetAsync(c->ferr, 0, sizeof(int), c->stream));
+    return fail(LB_ETIMEOUT, "a wait inside a step kernel ran out: the state is not to be trusted");
+}
+
+lb_status settle(lb_ctx *c) {
+    int err = 0;
+    LB_CUDA(cudaMemcpyAsync(&err, c->ferr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    LB_CUDA(cudaStreamSynchronize(c->stream));
+    return settle_flag(c, err);
+}
+
 // FP64 colour masses of planes [z0, z1) of the current state (store-aware first stage).
 lb_status run_mass(lb_ctx *c, double out[2], int z0 = 0, int z1 = -1) {
     const StepArgs sa = state_args(c);
@@ -629,14 +644,7 @@ lb_status run_mass(lb_ctx *c, double out[2], int z0 = 0, int z1 = -1) {
     c->launches += 2;
     LB_CUDA(cudaGetLastError());
     LB_CUDA(cudaMemcpyAsync(out, c->partial + 2 * kMassBlocks, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    int err = 0;
-    LB_CUDA(cudaMemcpyAsync(&err, c->ferr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    LB_CUDA(cudaStreamSynchronize(c->stream));
-    if (err) {
-        cudaMemsetAsync(c->ferr, 0, sizeof(int), c->stream);
-        return fail(LB_ETIMEOUT, "a wait inside a step kernel ran out: the state is not to be trusted");
-    }
-    return LB_OK;
+    return settle(c);
 }
 
 int grid_for(long long n, int threads) {
@@ -834,6 +842,7 @@ lb_status lb_init(lb_ctx *c, int32_t kind, const double *args, int32_t nargs, co
         c->launches += 1;
     }
     LB_CUDA(cudaGetLastError());
+    LB_CUDA(cudaMemsetAsync(c->ferr, 0, sizeof(int), c->stream));  // of a state that is gone
     if (kind == LB_INIT_FIELDS && !fields_on_device) LB_CUDA(cudaStreamSynchronize(c->stream));
     c->step = 0;
     c->initialized = true;
@@ -1002,7 +1011,8 @@ lb_status lb_halo_pack(lb_ctx *c, int32_t kind, int32_t z, void *dst, int32_t on
     lb_status s = halo_check(c, kind, z);
     if (s != LB_OK) return s;
     if (!dst) return fail(LB_EINVAL, "dst must not be NULL");
-    return halo_copy(c, kind, z, (char *)dst, true, on_device);
+    s = halo_copy(c, kind, z, (char *)dst, true, on_device);
+    return s == LB_OK && !on_device ? settle(c) : s;
 }
 
 lb_status lb_halo_unpack(lb_ctx *c, int32_t kind, int32_t z, const void *src, int32_t on_device) {
@@ -1167,9 +1177,8 @@ lb_status lb_fields(lb_ctx *c, uint32_t mask, float *const *outs, int32_t on_dev
     if (!on_device) {
         for (int j = 0; j < LB_NFIELDS; ++j)
             if (dst[j]) LB_CUDA(cudaMemcpyAsync(outs[j], dst[j], c->nn * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-        LB_CUDA(cudaStreamSynchronize(c->stream));
     }
-    return LB_OK;
+    return on_device ? LB_OK : settle(c);
 }
 
 lb_status lb_populations(lb_ctx *c, float *out, int32_t on_device) {
@@ -1196,8 +1205,7 @@ lb_status lb_populations(lb_ctx *c, float *out, int32_t on_device) {
             LB_CUDA(cudaMemcpyAsync(both ? out : out + (size_t)k * 27 * c->nn, dst, both ? 2 * cbytes : cbytes,
                                     cudaMemcpyDeviceToHost, c->stream));
     }
-    if (!on_device) LB_CUDA(cudaStreamSynchronize(c->stream));
-    return LB_OK;
+    return on_device ? LB_OK : settle(c);
 }
 
 lb_status lb_history(lb_ctx *c, float *out, int32_t on_device) {
@@ -1205,8 +1213,7 @@ lb_status lb_history(lb_ctx *c, float *out, int32_t on_device) {
     if (!c->initialized) return fail(LB_ESTATE, "lb_history before lb_init/lb_load");
     LB_CUDA(cudaMemcpyAsync(out, c->hist[c->hcur], (size_t)54 * c->plane * sizeof(float),
                             on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
-    if (!on_device) LB_CUDA(cudaStreamSynchronize(c->stream));
-    return LB_OK;
+    return on_device ? LB_OK : settle(c);
 }
 
 lb_status lb_mass_noalloc(const float *pop, int64_t nodes, double *out, void *stream) {
@@ -1270,9 +1277,8 @@ lb_status lb_save(lb_ctx *c, void *buf, size_t *nbytes) {
     LB_CUDA(cudaMemcpyAsync(p, c->pop[c->cur], pb, cudaMemcpyDeviceToHost, c->stream));
     if (sb) LB_CUDA(cudaMemcpyAsync(p + pb, c->ph4[c->cur], sb, cudaMemcpyDeviceToHost, c->stream));
     LB_CUDA(cudaMemcpyAsync(p + pb + sb, c->hist[c->hcur], hb, cudaMemcpyDeviceToHost, c->stream));
-    LB_CUDA(cudaStreamSynchronize(c->stream));
     *nbytes = total;
-    return LB_OK;
+    return settle(c);
 }
 
 lb_status lb_load(lb_ctx *c, const void *buf, size_t nbytes) {
@@ -1291,6 +1297,7 @@ lb_status lb_load(lb_ctx *c, const void *buf, size_t nbytes) {
     LB_CUDA(cudaMemcpyAsync(c->pop[0], p, pb, cudaMemcpyHostToDevice, c->stream));
     if (sb) LB_CUDA(cudaMemcpyAsync(c->ph4[0], p + pb, sb, cudaMemcpyHostToDevice, c->stream));
     LB_CUDA(cudaMemcpyAsync(c->hist[0], p + pb + sb, hb, cudaMemcpyHostToDevice, c->stream));
+    LB_CUDA(cudaMemsetAsync(c->ferr, 0, sizeof(int), c->stream));  // of a state that is gone
     LB_CUDA(cudaStreamSynchronize(c->stream));
     c->step = h.step;
     c->initialized = true;
@@ -1345,16 +1352,20 @@ int64_t lb_kernel_launches(const lb_ctx *c) { return c ? c->launches : -1; }
 
 lb_status lb_selftest(lb_ctx *c, int32_t which, int32_t *result, double *ms) {
     if (!c || !result || !ms) return fail(LB_EINVAL, "ctx, result and ms must not be NULL");
-    if (which != LB_SELFTEST_FUSED_WAIT) return fail(LB_EINVAL, "unknown self-test");
+    if (which != LB_SELFTEST_FUSED_WAIT && which != LB_SELFTEST_ADVANCE_WAIT) return fail(LB_EINVAL, "unknown self-test");
     if (c->half) return fail(LB_ESTATE, "lb_selftest inside a split step");
-    // the fused kernel's wait on plane 0 with a target no counter reaches; the scratch of the
-    // mass reduction takes the waited time
-    FusedCtl f{};
-    f.done = c->fdone;
-    f.err = c->ferr;
-    f.target = ~0ull;
+    // the fused kernel's wait on plane 0 with a target no counter reaches, or the advance's on a
+    // barrier that lacks a warp; the scratch of the mass reduction takes the waited time
     unsigned long long *ns = reinterpret_cast<unsigned long long *>(c->partial);
-    LB_CUDA(launch_fused_wait_probe(f, ns, c->stream));
+    if (which == LB_SELFTEST_FUSED_WAIT) {
+        FusedCtl f{};
+        f.done = c->fdone;
+        f.err = c->ferr;
+        f.target = ~0ull;
+        LB_CUDA(launch_fused_wait_probe(f, ns, c->stream));
+    } else {
+        LB_CUDA(launch_advance_wait_probe(c->ferr, 1 << 14, ns, c->stream));
+    }
     c->launches += 1;
     unsigned long long waited = 0;
     int err = 0;
@@ -1636,14 +1647,9 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         if (e != cudaSuccess) return cuda_fail(e, "launch_adjoint_reduce");
     }
     double host[32];
-    int ran_out = 0;
     LB_CUDA(cudaMemcpyAsync(host, w.out, sizeof(host), cudaMemcpyDeviceToHost, st));
-    LB_CUDA(cudaMemcpyAsync(&ran_out, c->ferr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    LB_CUDA(cudaStreamSynchronize(st));
-    if (ran_out) {
-        cudaMemsetAsync(c->ferr, 0, sizeof(int), st);
-        return fail(LB_ETIMEOUT, "a wait inside a step kernel ran out: the state is not to be trusted");
-    }
+    const lb_status ran = settle(c);
+    if (ran != LB_OK) return ran;
     grad_out[0] = host[24];
     for (int j = 1; j < LB_ADJ_NOUT; ++j) grad_out[j] = host[j];
     w.cl = cl;
@@ -1659,10 +1665,10 @@ lb_status lb_fragments(lb_ctx *c, int32_t connectivity, int32_t exclude_inlet, i
     if (cap < 0) return fail(LB_EINVAL, "cap must be >= 0");
     const size_t NN = (size_t)c->nn;
     const long long nblk = ((long long)NN + 1023) / 1024;
-    // scratch: label, count (int32), touch (u8), block counts, block offsets, error flag, then the list
+    // scratch: label, count (int32), touch (u8), block counts, block offsets and error flags, then the list
     // of roots (17 bytes each), in the idle population buffer (at least 112 bytes a node); allocated
     // only for lattices so small that the parts' alignment exceeds it
-    const size_t parts[] = {NN * 4, NN * 4, NN, (size_t)nblk * 4, (size_t)(nblk + 1) * 8, 16, NN * 17 + 64};
+    const size_t parts[] = {NN * 4, NN * 4, NN, (size_t)nblk * 4, (size_t)(nblk + 2) * 8, NN * 17 + 64};
     size_t need = 0;
     for (size_t v : parts) need += align_up(v);
     struct Free { char *p = nullptr; ~Free() { if (p) cudaFree(p); } } guard;
@@ -1681,7 +1687,7 @@ lb_status lb_fragments(lb_ctx *c, int32_t connectivity, int32_t exclude_inlet, i
     uint8_t *touch = (uint8_t *)q; q += align_up(parts[2]);
     int *bc = (int *)q; q += align_up(parts[3]);
     long long *boff = (long long *)q; q += align_up(parts[4]);
-    int *err = (int *)q; q += align_up(parts[5]);
+    int *err = (int *)(boff + nblk + 1);  // the labelling's and, copied, the steps'
     cudaStream_t st = c->stream;
     LB_CUDA(cudaMemsetAsync(count, 0, NN * 4, st));
     LB_CUDA(cudaMemsetAsync(touch, 0, NN, st));
@@ -1690,12 +1696,17 @@ lb_status lb_fragments(lb_ctx *c, int32_t connectivity, int32_t exclude_inlet, i
     cudaError_t e = launch_fragments_label(sa, c->p.storage, connectivity, label, count, touch, bc, boff, err, st,
                                            &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "launch_fragments_label");
-    long long nroots = 0;
-    int herr = 0;
-    LB_CUDA(cudaMemcpyAsync(&nroots, boff + nblk, sizeof(nroots), cudaMemcpyDeviceToHost, st));
-    LB_CUDA(cudaMemcpyAsync(&herr, err, sizeof(herr), cudaMemcpyDeviceToHost, st));
+    struct {
+        long long nroots;
+        int err, ferr;
+    } found = {};
+    LB_CUDA(cudaMemcpyAsync(err + 1, c->ferr, sizeof(int), cudaMemcpyDeviceToDevice, st));
+    LB_CUDA(cudaMemcpyAsync(&found, boff + nblk, sizeof(found), cudaMemcpyDeviceToHost, st));
     LB_CUDA(cudaStreamSynchronize(st));
-    if (herr) return fail(LB_ECUDA, "fragment labelling exceeded its iteration bound");
+    const lb_status ran = settle_flag(c, found.ferr);
+    if (ran != LB_OK) return ran;
+    const long long nroots = found.nroots;
+    if (found.err) return fail(LB_ECUDA, "fragment labelling exceeded its iteration bound");
     std::vector<long long> hroot((size_t)nroots), hvol((size_t)nroots);
     std::vector<uint8_t> htouch((size_t)nroots);
     if (nroots > 0) {

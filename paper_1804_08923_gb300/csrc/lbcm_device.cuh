@@ -478,6 +478,13 @@ __device__ __forceinline__ float2 fit_even(const StepArgs &a, float rr, float rb
     return make_float2(rr * oma, rb * oma);
 }
 
+// Nanoseconds of the device's global timer.
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // First statement of every kernel of a step: lets the next kernel of the stream be scheduled while
 // this one runs (launch_chained, lbcm_internal.h), and waits until the kernel before it has completed
 // and its writes are visible.  Nothing is read or written before.

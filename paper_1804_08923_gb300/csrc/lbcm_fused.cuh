@@ -28,11 +28,6 @@ __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long
     return v;
 }
 
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 // Waits until the gathers of planes p0, p1, p2 are all counted complete (the three counters
 // are read together).  Bounded by time, kFusedWaitNs, and as a backstop by the number of

@@ -54,6 +54,9 @@ struct AdvancePlan {
 AdvancePlan plan_advance(const StepArgs &a);
 cudaError_t launch_advance(const StepArgs &a, const AdvancePlan &p, const AdvanceArgs &v, cudaStream_t s,
                            long long *launches);
+// The advance's wait on a barrier that is never completed, limited to so many tries: it gives up and sets
+// *err; *ns receives the time it took.
+cudaError_t launch_advance_wait_probe(int *err, int tries, unsigned long long *ns, cudaStream_t s);
 
 // The same with half-precision storage (lbcm_half.cu): a step, its boundary planes alone, and the fused
 // kernel (or, occ not NULL, its blocks per SM).
