@@ -156,7 +156,9 @@ typedef enum {
 LB_API lb_status lb_init(lb_ctx *ctx, int32_t kind, const double *args, int32_t nargs,
                   const float *rho_r, const float *rho_b, const float *u, int32_t fields_on_device);
 
-/* Advances the lattice by n >= 0 time steps (Eq. (9) with the operator split of Section II). */
+/* Advances the lattice by n >= 0 time steps (Eq. (9) with the operator split of Section II).  If a
+ * launch fails (LB_ECUDA), the context holds the last step completed, as lb_step_count says; if that is
+ * lost too, calls that need a state return LB_ESTATE until lb_init or lb_load. */
 LB_API lb_status lb_step(lb_ctx *ctx, int64_t n);
 
 /* ----------------------------------------------------------- z-slab decomposition

@@ -1053,7 +1053,8 @@ static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
 // n >= 2 steps: one gather pass, n - 1 advances, one collision pass.  Moment records and phase entries
 // alternate between their own buffers and the population buffer that does not hold the state.  With
 // n even the collision writes over S(t), with n odd over the records there, which it does not read
-// then.
+// then.  An advance that cannot be launched ends the run where it is: the context then holds the step
+// reached.
 static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
     const bool conv = c->g.bc_zhi == LB_BC_CONVECTIVE;
     char *spare = (char *)c->pop[c->cur ^ 1];
@@ -1063,9 +1064,10 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
     cudaError_t e = launch_step(a, c->p.storage, c->stream, profile_record(c, PROF_GATHER), &c->launches, PASS_GATHER);
     if (e != cudaSuccess) return cuda_fail(e, "launch_step (gather)");
     cudaEvent_t *ev = nullptr;
-    for (int64_t s = 1; s < n; ++s) {
-        const int in = (int)((s - 1) & 1), out = in ^ 1;
-        a.step = c->step + s;
+    int64_t done = 1;  // gathered steps
+    for (; done < n && e == cudaSuccess; ++done) {
+        const int in = (int)((done - 1) & 1), out = in ^ 1;
+        a.step = c->step + done;
         if (conv) {
             a.hist_in = c->hist[c->hcur ^ out];
             a.hist_out = c->hist[c->hcur ^ in];
@@ -1076,22 +1078,31 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
         v.phase = phase[in];
         v.phase_out = phase[out];
         v.err = c->ferr;
-        ev = profile_record(c, s == n - 1 ? PROF_ADVANCE_COLLIDE : PROF_ADVANCE);
+        ev = profile_record(c, done == n - 1 ? PROF_ADVANCE_COLLIDE : PROF_ADVANCE);
         if (ev) cudaEventRecord(ev[0], c->stream);
         e = launch_advance(a, plan, v, c->stream, &c->launches);
-        if (e != cudaSuccess) return cuda_fail(e, "launch_advance");
         if (ev) cudaEventRecord(ev[1], c->stream);
     }
-    const int last = (int)((n - 1) & 1), dst = c->cur ^ (int)(n & 1);
+    const lb_status advanced = e == cudaSuccess ? LB_OK : cuda_fail(e, "launch_advance");
+    if (advanced != LB_OK) {
+        done -= 1;
+        if (ev) c->prof_used -= 1;
+        ev = nullptr;
+    }
+    const int last = (int)((done - 1) & 1), dst = c->cur ^ (int)(done & 1);
     a.mom = mom[last];
     a.phase = phase[last];
     a.pout = c->pop[dst];
     e = launch_step(a, c->p.storage, c->stream, ev, &c->launches, PASS_COLLIDE);
-    if (e != cudaSuccess) return cuda_fail(e, "launch_step (collide)");
+    if (e != cudaSuccess) {  // the populations are those of S(t) still, its outflow plane may be written over
+        if (ev) c->prof_used -= 1;
+        if (conv && done > 1) c->initialized = false;
+        return cuda_fail(e, "launch_step (collide)");
+    }
     c->cur = dst;
-    if (conv) c->hcur ^= (int)(n & 1);
-    c->step += n;
-    return LB_OK;
+    if (conv) c->hcur ^= (int)(done & 1);
+    c->step += done;
+    return advanced;
 }
 
 // n steps by advances (plan not NULL, n >= 2) or one by one in two passes, without mass checks.
@@ -1514,7 +1525,10 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     // carries everything else of the first step
     AdvancePlan plan;
     const bool advance = use_advance(c, a0, &plan);
-    auto recorded_steps = [&](StepArgs a, cudaStream_t s, long long len, int64_t step, int r, void *const (&pops)[2]) -> lb_status {
+    // done: steps after which pops[done & 1] and the outflow plane recorded after them are a state
+    auto recorded_steps = [&](StepArgs a, cudaStream_t s, long long len, int64_t step, int r, void *const (&pops)[2],
+                              long long &done) -> lb_status {
+        done = 0;
         float2 *phase[2] = {c->phase, w.phase2};
         for (long long t = 0; t < len; ++t) {
             a.step = step + t;
@@ -1541,12 +1555,14 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
                 e = launch_advance(b, plan, v, s, &c->launches);
             }
             if (e != cudaSuccess) return cuda_fail(e, "recorded step");
+            if (!advance || len < 2) done = t + 1;
         }
         if (advance && len >= 2) {
             a.phase = phase[(len - 1) & 1];
             a.pout = pops[len & 1];
             cudaError_t e = launch_step(a, LB_STORE_FP32, s, nullptr, &c->launches, PASS_COLLIDE);
             if (e != cudaSuccess) return cuda_fail(e, "recorded step (collide)");
+            done = len;
         }
         return LB_OK;
     };
@@ -1567,12 +1583,13 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         } else {
             LB_CUDA(cudaMemcpyAsync(w.seg_hist[r], c->hist[c->hcur], hb, cudaMemcpyDeviceToDevice, st));
             void *const pops[2] = {c->pop[c->cur], c->pop[c->cur ^ 1]};
-            lb_status rs = recorded_steps(make_args(c), st, len, c->step, r, pops);
+            long long done;
+            lb_status rs = recorded_steps(make_args(c), st, len, c->step, r, pops, done);
+            c->cur ^= (int)(done & 1);
+            c->step += done;
+            if (conv && done > 0)
+                LB_CUDA(cudaMemcpyAsync(c->hist[c->hcur], w.seg_hist[r] + done * 54 * P, hb, cudaMemcpyDeviceToDevice, st));
             if (rs != LB_OK) return rs;
-            c->cur ^= (int)(len & 1);
-            c->step += len;
-            if (conv)
-                LB_CUDA(cudaMemcpyAsync(c->hist[c->hcur], w.seg_hist[r] + len * 54 * P, hb, cudaMemcpyDeviceToDevice, st));
         }
     }
 
@@ -1608,7 +1625,8 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         if (conv)
             LB_CUDA(cudaMemcpyAsync(w.seg_hist[r], w.ckpt_hist + sg * 54 * P, hb, cudaMemcpyDeviceToDevice, s2));
         void *const pops[2] = {w.seg_pop, w.seg_pop + 27 * NN};
-        lb_status rs = recorded_steps(make_args(c), s2, len, step0 + n0, r, pops);
+        long long done;
+        lb_status rs = recorded_steps(make_args(c), s2, len, step0 + n0, r, pops, done);
         if (rs != LB_OK) return rs;
         LB_CUDA(cudaEventRecord(w.ev_rec[r], s2));
         return LB_OK;

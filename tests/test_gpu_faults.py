@@ -88,3 +88,57 @@ def test_the_advance_s_wait_gives_up(lb):
     assert np.array_equal(lat.populations(device=False), ref.populations(device=False))
     lat.close()
     ref.close()
+
+
+def test_a_refused_launch_leaves_a_whole_state(lb):
+    """The k-th launch of a call of six steps fails.  What the context holds then, populations and
+    outflow plane, is the state of the step it names; where that is not to be had, it holds none."""
+    for bc in ((0, 0), (2, 3)):
+        lat, ref = lattice(lb, bc), lattice(lb, bc)
+        for k in range(1, 6):
+            blob, t = lat.save(), lat.step_count
+            lb.faults(0, k, 0)
+            with pytest.raises(lb.LBError) as e:
+                lat.step(6)
+            lb.faults(0, 0, 0)
+            assert e.value.status == LB_ECUDA
+            assert lat.step_count == t + k  # the first launch of the six is the gather pass
+            ref.load(blob)
+            for _ in range(k):
+                ref.step(1)
+            assert np.array_equal(lat.populations(device=False), ref.populations(device=False))
+            assert np.array_equal(lat.history(), ref.history())
+        blob = lat.save()
+        for n, call in ((4, 1), (2, 2), (3, 2)):  # the gather pass of four steps, the collision pass of two and three
+            lat.load(blob)
+            lb.faults(call, 0, 0)
+            with pytest.raises(lb.LBError) as e:
+                lat.step(n)
+            lb.faults(0, 0, 0)
+            assert e.value.status == LB_ECUDA
+            if call == 1 or bc[1] != 3:
+                assert lat.save() == blob
+            else:
+                with pytest.raises(lb.LBError):
+                    lat.populations()
+        lat.close()
+        ref.close()
+
+
+@pytest.mark.parametrize("grid,fail,done", [((24, 16, 20), (3, 0), 2), (GRID, (0, 2), 0), (GRID, (2, 0), 0)])
+def test_a_refused_launch_in_an_adjoint_leaves_a_whole_state(lb, grid, fail, done):
+    p = dict(rho_r0=1.0, rho_b0=0.5, nu_r=0.02, nu_b=0.05, sigma=0.003, u_in=0.05, d_in=8.0)
+    lat, ref = (lb.Lattice(grid, p, bc=(2, 3)) for _ in range(2))
+    for l in (lat, ref):
+        l.init_fields(*workloads.random_two_phase_fields(grid[::-1], 3, 1.0, 0.5, u_amp=0.03))
+    lb.faults(*fail, 0)
+    with pytest.raises(lb.LBError) as e:
+        lat.adjoint(4, "area", (1e-3,), checkpoint=4)
+    lb.faults(0, 0, 0)
+    assert e.value.status == LB_ECUDA
+    ref.step(done)
+    assert lat.step_count == done
+    assert np.array_equal(lat.populations(device=False), ref.populations(device=False))
+    assert np.array_equal(lat.history(), ref.history())
+    lat.close()
+    ref.close()
