@@ -1054,14 +1054,15 @@ static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
 // alternate between their own buffers and the population buffer that does not hold the state.  With
 // n even the collision writes over S(t), with n odd over the records there, which it does not read
 // then.  An advance that cannot be launched ends the run where it is: the context then holds the step
-// reached.
-static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
+// reached.  profile: whether the launches take profile records (those of lb_step do).
+static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n, bool profile) {
+    auto record = [&](ProfKind kind) { return profile ? profile_record(c, kind) : nullptr; };
     const bool conv = c->g.bc_zhi == LB_BC_CONVECTIVE;
     char *spare = (char *)c->pop[c->cur ^ 1];
     float4 *mom[2] = {c->mom, (float4 *)spare};
     float2 *phase[2] = {c->phase, (float2 *)(spare + align_up(48 * (size_t)c->nn))};
     StepArgs a = make_args(c);
-    cudaError_t e = launch_step(a, c->p.storage, c->stream, profile_record(c, PROF_GATHER), &c->launches, PASS_GATHER);
+    cudaError_t e = launch_step(a, c->p.storage, c->stream, record(PROF_GATHER), &c->launches, PASS_GATHER);
     if (e != cudaSuccess) return cuda_fail(e, "launch_step (gather)");
     cudaEvent_t *ev = nullptr;
     int64_t done = 1;  // gathered steps
@@ -1078,7 +1079,7 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
         v.phase = phase[in];
         v.phase_out = phase[out];
         v.err = c->ferr;
-        ev = profile_record(c, done == n - 1 ? PROF_ADVANCE_COLLIDE : PROF_ADVANCE);
+        ev = record(done == n - 1 ? PROF_ADVANCE_COLLIDE : PROF_ADVANCE);
         if (ev) cudaEventRecord(ev[0], c->stream);
         e = launch_advance(a, plan, v, c->stream, &c->launches);
         if (ev) cudaEventRecord(ev[1], c->stream);
@@ -1105,9 +1106,10 @@ static lb_status advance_steps(lb_ctx *c, const AdvancePlan &plan, int64_t n) {
     return advanced;
 }
 
-// n steps by advances (plan not NULL, n >= 2) or one by one in two passes, without mass checks.
+// n steps by advances (plan not NULL, n >= 2) or one by one in two passes, without mass checks and
+// profile records (lb_adjoint's).
 static lb_status steps_unchecked(lb_ctx *c, const AdvancePlan *plan, int64_t n) {
-    if (plan && n >= 2) return advance_steps(c, *plan, n);
+    if (plan && n >= 2) return advance_steps(c, *plan, n, false);
     for (int64_t s = 0; s < n; ++s) {
         cudaError_t e = launch_step(make_args(c), c->p.storage, c->stream, nullptr, &c->launches);
         if (e != cudaSuccess) return cuda_fail(e, "launch_step");
@@ -1129,7 +1131,7 @@ lb_status lb_step(lb_ctx *c, int64_t n) {
         if (advance) {  // up to the next mass check in one go
             const int64_t m = c->p.check_every > 0 ? std::min<int64_t>(n - s, c->p.check_every - c->step % c->p.check_every) : n - s;
             if (m >= 2) {
-                lb_status st = advance_steps(c, plan, m);
+                lb_status st = advance_steps(c, plan, m, true);
                 if (st == LB_OK) st = check_step(c);
                 if (st != LB_OK) return st;
                 s += m;
