@@ -157,10 +157,11 @@ struct lb_ctx {
     std::vector<cudaEvent_t> prof_ev;  // 4 events per recorded step
     std::vector<char> prof_kind;       // what each record's events bracket (PROF_*)
     int prof_cap = 0, prof_used = 0;
-    // discrete-adjoint workspace (one device allocation, grown on demand)
+    // discrete-adjoint workspace: base holds the adjoint state (its size depends on the lattice alone),
+    // steps the checkpoints and records of a call, grown on demand
     struct {
-        void *base = nullptr;
-        size_t bytes = 0;
+        void *base = nullptr, *steps = nullptr;
+        size_t bytes = 0;  // of steps
         float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lr_obj = nullptr, *lgb = nullptr, *objph = nullptr,
                *phase2 = nullptr;
         float *ckpt_hist = nullptr, *seg_fm[2] = {}, *seg_hist[2] = {}, *lx = nullptr, *lh[2] = {};
@@ -764,6 +765,7 @@ void lb_destroy(lb_ctx *c) {
         }
     }
     if (c->adj.base) cudaFree(c->adj.base);
+    if (c->adj.steps) cudaFree(c->adj.steps);
     if (c->owns)
         for (int j = 0; j < c->nbufs; ++j)
             if (c->bufs[j]) cudaFree(c->bufs[j]);
@@ -1423,9 +1425,9 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
     const size_t pb = 27 * NN * sizeof(float2), hb = 54 * P * sizeof(float), nb2 = NN * sizeof(float2);
     StepArgs a0 = make_args(c);
     const long long nblk_coll = adj_collide_blocks(a0), nblk_inlet = adj_boundary_blocks(a0);
-    constexpr int kParts = 27;
-    auto layout = [&](long long k, size_t (&parts)[kParts]) {
-        const long long nseg = (T + k - 1) / k;
+    constexpr int kSteps = 13, kParts = 27;  // parts of the steps' block; of both
+    auto layout = [&](long long k, size_t (&parts)[kParts]) {  // bytes of the steps' block
+        const long long nseg = (T - 1) / k + 1;
         const size_t one = nseg > 1 ? 1 : 0, ku = (size_t)k;
         const size_t rec[5] = {ku * 3 * NN * sizeof(float4), ku * NN * sizeof(float4), ku * nb2, ku * hb, (ku + 1) * hb};
         const size_t v[kParts] = {one * nseg * pb, one * nseg * hb, one * 2 * pb,
@@ -1435,46 +1437,77 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
                                   nblk_coll * 3 * sizeof(double), nblk_inlet * 17 * sizeof(double),
                                   nblk_coll * sizeof(double), 32 * sizeof(double), nb2, nb2};
         size_t need = 0;
-        for (int q = 0; q < kParts; ++q) need += align_up(parts[q] = v[q]);
+        for (int q = 0; q < kParts; ++q) {
+            parts[q] = v[q];
+            if (q < kSteps) need += align_up(v[q]);
+        }
         return need;
+    };
+    // whether any device could hold the schedule (its sizes stay far below 2^63)
+    auto possible = [&](long long k) {
+        return k <= (long long)((1ull << 48) / (72 * NN + 2 * hb)) && (T - 1) / k < (long long)((1ull << 48) / (pb + hb));
     };
     size_t parts[kParts];
     auto allocate = [&](size_t need) {
         if (need <= c->adj.bytes) return true;
-        if (c->adj.base) cudaFree(c->adj.base);
-        c->adj.base = nullptr;
+        if (c->adj.steps) cudaFree(c->adj.steps);
+        c->adj.steps = nullptr;
         c->adj.bytes = 0;
-        c->adj.valid = false;
-        if (cudaMalloc(&c->adj.base, need) != cudaSuccess) {
+        if (cudaMalloc(&c->adj.steps, need) != cudaSuccess) {
             cudaGetLastError();
-            c->adj.base = nullptr;
+            c->adj.steps = nullptr;
             return false;
         }
         c->adj.bytes = need;
         return true;
     };
-    // k = 0: every step recorded where that takes no more than a sixth of the free device memory
+    auto no_memory = [](size_t need) {
+        return fail(LB_ENOMEM, "cannot allocate the adjoint workspace (" + std::to_string(need >> 20) + " MiB)");
+    };
+    // k = 0: every step recorded where that takes no more than a quarter of the free device memory
     // (what a previous call left allocated counts as free), else ceil(sqrt(T)).  The recompute that this
     // saves costs as much as the forward pass; run beside the reverse sweep it hid nothing (64x64x256
-    // jet, 50 steps: 20.2 ms with it; 500 steps, 38 GB of records: 116 ms with it, 87 without).
-    long long k = obj_args[2] >= 1 ? std::min<long long>((long long)obj_args[2], T) : 0;
-    bool have = false;
-    if (k == 0) {
+    // jet, 50 steps: 20.2 ms with it, 13.8 without).  What exceeds twice the block of the schedule with
+    // checkpoints is given back when the call ends: a context keeps what it would have kept with them
+    // but for a factor, not what happened to be free.  Allocating and freeing 38 GB (500 steps) takes 20 ms
+    // of that call's 107; with checkpoints it takes 116.
+    const long long k_sqrt = std::max(1ll, std::min<long long>((long long)std::ceil(std::sqrt((double)T)), T));
+    long long k = obj_args[2] < 1 ? 0 : obj_args[2] >= (double)T ? T : (long long)obj_args[2];
+    const bool automatic = k == 0;
+    if (!possible(automatic ? k_sqrt : k)) return no_memory((size_t)1 << 48);
+    if (automatic) {
         size_t free_b = 0, total_b = 0;
         LB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        const size_t all = layout(T, parts);
-        have = all <= (free_b + c->adj.bytes) / 6 && allocate(all);
-        k = have ? T : std::max(1ll, std::min<long long>((long long)std::ceil(std::sqrt((double)T)), T));
+        k = possible(T) && layout(T, parts) <= (free_b + c->adj.bytes) / 4 && allocate(layout(T, parts)) ? T : k_sqrt;
     }
-    const long long nseg = (T + k - 1) / k;
-    if (!have) {
-        const size_t need = layout(k, parts);
-        if (!allocate(need)) return fail(LB_ENOMEM, "cannot allocate the adjoint workspace (" + std::to_string(need >> 20) + " MiB)");
+    const size_t keep = automatic ? 2 * layout(k_sqrt, parts) : ~(size_t)0;
+    struct GiveBack {
+        lb_ctx *c;
+        size_t keep;
+        ~GiveBack() {
+            if (c->adj.bytes <= keep) return;
+            cudaFree(c->adj.steps);
+            c->adj.steps = nullptr;
+            c->adj.bytes = 0;
+        }
+    } give_back{c, keep};
+    const long long nseg = (T - 1) / k + 1;
+    const size_t need = layout(k, parts);
+    if (!allocate(need)) return no_memory(need);
+    if (!c->adj.base) {
+        size_t state = 0;
+        for (int q = kSteps; q < kParts; ++q) state += align_up(parts[q]);
+        if (cudaMalloc(&c->adj.base, state) != cudaSuccess) {
+            cudaGetLastError();
+            c->adj.base = nullptr;
+            return no_memory(state);
+        }
     }
     {
-        char *p = (char *)c->adj.base;
+        char *p = (char *)c->adj.steps;
         void *v[kParts];
         for (int q = 0; q < kParts; ++q) {
+            if (q == kSteps) p = (char *)c->adj.base;
             v[q] = p;
             p += align_up(parts[q]);
         }

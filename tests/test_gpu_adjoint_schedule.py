@@ -38,3 +38,36 @@ def test_an_adjoint_takes_no_profile_records(lb):
     assert {k: n for k, (_, n) in lat.profile_read().items() if n} == {
         "boundary_kernel": 1, "moment_kernel": 1, "advance_kernel": 2, "collide_kernel": 1}
     lat.close()
+
+
+def test_the_automatic_schedule_keeps_no_more_than_twice_the_checkpoints(lb):
+    """200 steps recorded take 14.7 KB a node, with checkpoints every 15 steps 5.7; the context keeps at
+    most twice that, and what is left of the call is the same."""
+    import torch
+    T, k, nseg = 200, 15, 14
+    lat, ref = lattice(lb), lattice(lb)
+    J, g = ref.adjoint(T, checkpoint=T)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    assert lat.adjoint(T)[0] == J
+    kept = before - torch.cuda.mem_get_info()[0]
+    steps = nseg * 216 + 2 * 216 + 2 * k * 72  # bytes a node, the outflow plane's share below
+    assert kept <= 2 * lat.nodes * steps * (1 + 4.0 / GRID[2]) + lat.nodes * 200 + (64 << 20), kept / lat.nodes
+    assert torch.equal(lat.adjoint_state(device=True), ref.adjoint_state(device=True))
+    # a later call that needs less gives back what it does not need
+    lat.adjoint(T, checkpoint=T)
+    lat.adjoint(3)
+    kept = before - torch.cuda.mem_get_info()[0]
+    assert kept <= lat.nodes * (3 * 72 * 4 + 2 * 216 * 4 + 200) + (64 << 20), kept / lat.nodes
+    lat.close()
+    ref.close()
+
+
+def test_a_number_of_steps_beyond_any_memory_is_refused(lb):
+    lat = lattice(lb, (16, 8, 10))
+    for T, k in ((1 << 50, 1 << 50), (1 << 62, 0), (1 << 62, 1)):
+        with pytest.raises(lb.LBError) as e:
+            lat.adjoint(T, checkpoint=k)
+        assert e.value.status == 2  # LB_ENOMEM
+    assert np.isfinite(lat.adjoint(2)[0])
+    lat.close()
