@@ -185,9 +185,7 @@ class Lattice:
             ts = [out[FIELD_NAMES[j]] for j in sel]
             for t in ts:
                 assert t.is_cuda and t.dtype == torch.float32 and t.is_contiguous() and t.numel() == self.nodes
-        elif self.nodes <= 65536:  # one allocation: seven cost more host time than the kernel runs
-            ts = torch.empty((len(sel),) + self.shape, dtype=torch.float32, device=self.device).unbind(0)
-        else:
+        else:  # each its own: views of one allocation cannot be kept, saved or written alone
             ts = [torch.empty(self.shape, dtype=torch.float32, device=self.device) for _ in sel]
         mask, outs, keep = 0, _FieldPointers(), {}
         for j, t in zip(sel, ts):
