@@ -71,3 +71,27 @@ def test_a_number_of_steps_beyond_any_memory_is_refused(lb):
         assert e.value.status == 2  # LB_ENOMEM
     assert np.isfinite(lat.adjoint(2)[0])
     lat.close()
+
+
+def run(lat, T, objective, args, checkpoint):
+    J, g = lat.adjoint(T, objective, args, checkpoint)
+    return J, g, lat.adjoint_state(device=True).clone()
+
+
+@pytest.mark.parametrize("grid,bc", [(GRID, (2, 3)), (GRID, (0, 0)), ((125, 99, 95), (2, 3, 1, 1)), ((70, 66, 400), (1, 1, 1, 1))])
+def test_segments_of_recorded_advances(lb, grid, bc):
+    """Twelve steps in one recorded segment against six of two and four of three, recomputed by
+    advances on the second stream into two alternating sets, and against single steps, which are
+    recorded by the two passes: the same bits."""
+    import torch
+    T = 12
+    want = None
+    for checkpoint in (T, 2, 3, 5, 1):
+        lat = lattice(lb, grid, bc, g=(1e-6, 0.0, 1e-5))
+        got = run(lat, T, "area", (1e-3,), checkpoint)
+        end = lat.populations().clone()
+        if want is None:
+            want, want_end = got, end
+        assert got[0] == want[0] and np.array_equal(got[1], want[1]), checkpoint
+        assert torch.equal(got[2], want[2]) and torch.equal(end, want_end), checkpoint
+        lat.close()
