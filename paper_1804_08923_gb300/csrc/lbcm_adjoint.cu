@@ -128,15 +128,6 @@ __device__ __forceinline__ float2 adj_slot(const StepArgs &a, const AdjArgs &g, 
     return v;
 }
 
-// Asynchronous global -> shared copies (no register holds the value in flight).
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
 __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
 // 1-D transpose of the inverse transform of central moments about u (values v(+-1) = (t +- o)/2,
@@ -536,7 +527,7 @@ __global__ void __launch_bounds__(128, 3) adj_collide_kernel(StepArgs a, AdjArgs
             const int c = t + 128 * k;
             if (c < T::kN) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) cp_async16(dst + q * T::kN + c, g.rec_in.p[q] + (size_t)zs * P + cell0[k]);
+                for (int q = 0; q < 3; ++q) cp_async<16>(dst + q * T::kN + c, g.rec_in.p[q] + (size_t)zs * P + cell0[k]);
             }
         }
     };
@@ -545,9 +536,9 @@ __global__ void __launch_bounds__(128, 3) adj_collide_kernel(StepArgs a, AdjArgs
         if (!live) return;
         const size_t n = (size_t)z * P + (size_t)y * a.nx + x;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) cp_async16(&S.own[q][t], g.mom + q * NN + n);
-        cp_async16(&S.own[3][t], g.grad4 + n);
-        cp_async8(&S.own2[t], g.grad2 + n);
+        for (int q = 0; q < 3; ++q) cp_async<16>(&S.own[q][t], g.mom + q * NN + n);
+        cp_async<16>(&S.own[3][t], g.grad4 + n);
+        cp_async<8>(&S.own2[t], g.grad2 + n);
     };
     const bool gather = g.lr_obj == nullptr;
     if (gather) {

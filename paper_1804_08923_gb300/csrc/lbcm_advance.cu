@@ -17,7 +17,7 @@
 //            still colliding;
 //   gather   each thread of the tile reads the 27 pulls that come from plane k: c_z = -1 completes
 //            the node of plane k - 1, c_z = 0 is joined to plane k, c_z = +1 starts plane k + 1
-//            (z_class, join_classes, finish_moments; 22 registers hold the two open planes).
+//            (z_class, join_classes, finish_moments; 24 registers hold the two open planes).
 // What bounds it: instruction issue and the shared-memory pipe, in turn rather than together (96 x 96 x
 // 384 jet: issue slots 71%, FMA pipe 55%, 1206 instructions a node with its share of the halo; DRAM 104
 // bytes a node, a third of its bandwidth), because the warps of a block go through the same phase at
@@ -51,16 +51,6 @@ struct AdvanceTile {
     static constexpr int kBytes = kBar + 16;
     static_assert(kBytes <= 227 * 1024 && NR <= 2 * NT && kRows % 32 == 0 && kHaloY % 32 == 0, "layout");
 };
-
-template <int B>
-__device__ __forceinline__ void cp_async(unsigned smem, const void *gmem) {
-    if constexpr (B == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(gmem) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // Barrier of the block's warps in two halves: a warp arrives when it has written what it shares, goes
 // on with work of its own and waits when it needs the others'.  The wait is bounded by the number of

@@ -323,15 +323,15 @@ __device__ __forceinline__ void collide_halo_x(const StepArgs &a, Moments mo, fl
     ready();
     const Axis X(q.ux), Y(q.uy);
     float W0[3], W1[3], W2[3];
+    const float cx0 = q.C0 + q.qxx, exy = cx0 + q.qyy, exz = cx0 + q.qzz, exyz = exy + q.qzz;
+    const float uxy = q.ux + q.uy, vxy = q.ux - q.uy, gxy = q.gpx + q.gpy, hxy = q.gpx - q.gpy, Fxy = q.Fx + q.Fy, Hxy = q.Fx - q.Fy;
+    const float qp = q.qxy + q.qxz, qm = q.qxy - q.qxz;
+    q.yline(Y, 1, W0, W1, W2);
     auto xplus = [&](int b) {
         float m_, z_, p_;
         q.xline(X, W0[b], W1[b], W2[b], m_, z_, p_);
         return p_;
     };
-    const float cx0 = q.C0 + q.qxx, exy = cx0 + q.qyy, exz = cx0 + q.qzz, exyz = exy + q.qzz;
-    const float uxy = q.ux + q.uy, vxy = q.ux - q.uy, gxy = q.gpx + q.gpy, hxy = q.gpx - q.gpy, Fxy = q.Fx + q.Fy, Hxy = q.Fx - q.Fy;
-    const float qp = q.qxy + q.qxz, qm = q.qxy - q.qxz;
-    q.yline(Y, 1, W0, W1, W2);
     put(1, q.template one<false>(1, cx0, q.ux, q.Fx, q.gpx, q.sg1, xplus(1)));
     put(7, q.template one<false>(7, exy + q.qxy, uxy, Fxy, gxy, q.sg2, xplus(2)));
     put(9, q.template one<false>(9, exy - q.qxy, vxy, Hxy, hxy, q.sg2, xplus(0)));

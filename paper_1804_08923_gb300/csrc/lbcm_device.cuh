@@ -485,9 +485,27 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// First statement of every kernel of a step: lets the next kernel of the stream be scheduled while
-// this one runs (launch_chained, lbcm_internal.h), and waits until the kernel before it has completed
-// and its writes are visible.  Nothing is read or written before.
+// Asynchronous copies of B (8 or 16) bytes from global to shared memory (no register holds the value in
+// flight), and the waits for them: for all of them, or for the groups committed.
+template <int B>
+__device__ __forceinline__ void cp_async(unsigned smem, const void *gmem) {
+    if constexpr (B == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem), "l"(gmem) : "memory");
+}
+template <int B>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+    cp_async<B>((unsigned)__cvta_generic_to_shared(smem), gmem);
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// First statement of every kernel that launch_chained (lbcm_internal.h) launches, that is, of those of a
+// step but for the general-rates and the fused ones: lets the next kernel of the stream be scheduled
+// while this one runs, and waits until the kernel before it has completed and its writes are visible.
+// Nothing is read or written before.
 __device__ __forceinline__ void chain_begin() {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     asm volatile("griddepcontrol.wait;\n" ::: "memory");

@@ -21,7 +21,8 @@ namespace lbcm {
 // the method's 448 bytes a node from DRAM (450-500 measured, against 522 for the two launches),
 // but its blocks wait and synchronise at every item and it streams at a lower fraction of the
 // bandwidth: on GB300 it is 3% slower than the two launches on the 256x256x1024 jet and about
-// level with them on smaller ones, and the two launches stay the default.
+// level with them on smaller ones, and the two launches, or the advance where a call takes several
+// steps, stay the default.
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
     unsigned long long v;
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");

@@ -98,10 +98,6 @@ __global__ void __launch_bounds__(128) boundary_plane_kernel(StepArgs a) {
             const long long hr = (long long)i * P + pxy, hb = (long long)(27 + i) * P + pxy;
             a.hist_out[hr] = (__ldg(a.hist_in + hr) + lam * fr) * inv;
             a.hist_out[hb] = (__ldg(a.hist_in + hb) + lam * fb) * inv;
-            if (a.fm_out) {
-                a.fm_out[hr] = fr;
-                a.fm_out[hb] = fb;
-            }
         }
     }
 }
@@ -203,10 +199,6 @@ __global__ void __launch_bounds__(128) boundary_column_kernel(StepArgs a) {
             const long long hr = (long long)i * P + pxy, hb = (long long)(27 + i) * P + pxy;
             a.hist_out[hr] = (__ldg(a.hist_in + hr) + lam * fr[i]) * inv;
             a.hist_out[hb] = (__ldg(a.hist_in + hb) + lam * fb[i]) * inv;
-            if (a.fm_out) {
-                a.fm_out[hr] = fr[i];
-                a.fm_out[hb] = fb[i];
-            }
         }
     }
 }

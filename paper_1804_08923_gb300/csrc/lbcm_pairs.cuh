@@ -1,6 +1,6 @@
 // lbcm_pairs.cuh -- per-node pieces in the association over the 13 pairs of opposite directions: the
 // gradient stencil of the general-rates step and of the half-precision storages, the moments and the
-// moment record of the latter, and the inverse 1-D sweep coefficients (also the adjoint's).
+// moment record of the latter, and their inverse 1-D sweep coefficients.
 #pragma once
 #include "lbcm_node.cuh"
 

@@ -254,8 +254,7 @@ __global__ void __launch_bounds__(128) moment_kernel(StepArgs a) {
 // gradients from the 26 neighbours' phase entries and writes the 54 populations.
 // kRec (FP32, adjoint recompute): also writes the node's gradients to a.grad4 / a.grad2 (its
 // moments are already in a.mom).
-// Blocks per SM (register bound): FP32 6, FP16 5, FP16_FIT 4 (its encoding needs the most
-// registers).
+// Blocks per SM (register bound): 6.
 
 // (phi, rho) of the neighbour x + c_j.  Ghosts: z = -1 is phi = 1, rho = rho_r0 inside the inlet
 // disc and the mirror of z = 0 elsewhere; z = N + 1 mirrors z = N (the neighbour offsets are clamped
