@@ -255,19 +255,15 @@ __global__ void init_kernel(InitArgs ia, StepArgs sa) {
         const Nbr nb = node_nbr(sa, n);
         const float usq = ux * ux + uy * uy + uz * uz;
         MassAcc sr, sb;
-        float2 moving[27];
         const bool top = nb.zo[1] == (ia.nz - 1) * (int)sa.plane;
         const long long h = nb.pxy, P = sa.plane;
-#pragma unroll
-        for (int i = 1; i < 27; ++i) {
+        auto put = [&](int i) {  // stores direction i >= 1; what its reader will see
             const float cu = (float)cx(i) * ux + (float)cy(i) * uy + (float)cz(i) * uz;
             const float pw = wgt(i) * eq_poly(cu, usq);
             const float2 f = make_float2(rr * (varphi(i, ia.alpha_r, ia.oma_r) + pw),
                                          rb * (varphi(i, ia.alpha_b, ia.oma_b) + pw));
             const float2 d = store_pop<S>(sa, i, (int)n, f, dest_shift<S>(sa, nb, i));
-            if constexpr (kPaper) {
-                moving[i] = d;
-            } else {
+            if constexpr (!kPaper) {
                 sr.add(i, d.x);
                 sb.add(i, d.y);
             }
@@ -275,9 +271,16 @@ __global__ void init_kernel(InitArgs ia, StepArgs sa) {
                 ia.hist[(long long)i * P + h] = d.x;
                 ia.hist[(long long)(27 + i) * P + h] = d.y;
             }
+            return d;
+        };
+        float2 s;
+        if constexpr (kPaper) {
+            s = moving_mass(put);
+        } else {
+#pragma unroll
+            for (int i = 1; i < 27; ++i) put(i);
+            s = make_float2(sr.s, sb.s);
         }
-        float2 s = make_float2(sr.s, sb.s);
-        if constexpr (kPaper) s = moving_mass([&](int i) { return moving[i]; });
         const float2 f0 = make_float2(rr - s.x, rb - s.y);
         store_pop<S>(sa, 0, (int)n, f0, no_shift());
         if (top) {
