@@ -126,6 +126,17 @@ def kernel_profile(lat, steps, nodes, storage, peak, cfg_name):
     return kernels, roofline
 
 
+def hbm_shares(mlups, kernels, storage, steps, peak):
+    """Shares of the HBM peak of `mlups` node updates (1e6/s) on one GPU: of the bytes that the kernels of a
+    call of `steps` steps move by their design (hbm_pct_of_peak), and, for comparison with methods that
+    read and write their populations every step, of the bytes those take (hbm_pct_of_peak_populations,
+    above 100 where the populations stay on the chip between the steps of a call)."""
+    moved = sum(k["launches"] * k.get("algorithmic_bytes_per_node", 0) for k in kernels.values()) / steps
+    pct = 100.0 * mlups * 1e6 / (peak[0] * 1e9)
+    return {"hbm_pct_of_peak": pct * moved, "bytes_per_node_design": moved,
+            "hbm_pct_of_peak_populations": pct * BYTES[storage][0], "bytes_per_node_algorithmic": BYTES[storage][0]}
+
+
 def storage_leg(lb, torch, cfg, storage, steps, warmup, peak, world, max_over_ranks, barrier):
     """MLUPS, per-kernel times and the dominant kernel's roofline of one storage."""
     nodes = int(np.prod(cfg["grid"]))
@@ -137,12 +148,10 @@ def storage_leg(lb, torch, cfg, storage, steps, warmup, peak, world, max_over_ra
     lat.close()
     del lat
     torch.cuda.empty_cache()
-    bs, _ = BYTES[storage]
     v = job_mlups(nodes, steps, world, ms)
     return {"value": v, "unit": "MLUPS", "ms_per_step": ms / steps, "steps": steps,
-            "storage": STORAGE_TEXT.get(storage, "fp32 populations"), "bytes_per_node_algorithmic": bs,
-            "hbm_pct_of_peak": 100.0 * v * 1e6 * bs / (peak[0] * 1e9) / world,
-            "roofline": roofline, "kernels": kernels}
+            "storage": STORAGE_TEXT.get(storage, "fp32 populations"),
+            **hbm_shares(v / world, kernels, storage, steps, peak), "roofline": roofline, "kernels": kernels}
 
 
 def error_vs_fp32(lb, torch, cfg, checkpoints):
@@ -491,13 +500,13 @@ def run_slabs(args, cfg, lb, torch, dist, rank, world, local, barrier, max_over_
         barrier()
     ms = max_over_ranks(e0.elapsed_time(e1))
     value = nodes * args.steps / (ms * 1e-3) / 1e6
-    bytes_step, _ = BYTES[args.storage]
     line = {"metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "strong",
             "vs_baseline": None, "dtype": "f32" if args.storage == 0 else "f32 arithmetic, f16 population storage",
             "data": "synthetic", "config": dict(config_block(cfg, args.storage),
                                                 parallelism=f"z-slabs over {world} GPUs, halos over NCCL"),
-            "hbm_pct_of_peak": 100.0 * value * 1e6 * bytes_step / (peak[0] * 1e9) / world,
+            **hbm_shares(value / world, {k: {"launches": args.steps, "algorithmic_bytes_per_node": BYTES[args.storage][1][k]}
+                                         for k in ("moment_kernel", "collide_kernel")}, args.storage, args.steps, peak),
             "slab_planes": [list(r) for r in slab.partition(cfg["grid"][2], world)],
             "mass": s.mass().tolist(), "clocks": clk.summary()}
     if rank == 0:
@@ -600,16 +609,12 @@ def main():
     ms_step = ms / args.steps
     value = job_mlups(nodes, args.steps, world, ms)
     clocks = clk.summary()
-    bytes_step, _ = BYTES[st]
     kernels, roofline = kernel_profile(lat, args.steps, nodes, st, peak, cfg["name"])
     line = {"metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32" if st == 0 else "f32 arithmetic, f16 population storage",
             "data": "synthetic", "config": config_block(cfg, st),
-            "hbm_pct_of_peak": 100.0 * value * 1e6 * bytes_step / (peak[0] * 1e9) / world,
-            "bytes_per_node_algorithmic": bytes_step,
-            "bytes_per_node_design": BYTES[st][1]["advance_kernel"] if st == 0 else
-            BYTES[st][1]["collide_kernel"] + BYTES[st][1]["moment_kernel"],
+            **hbm_shares(value / world, kernels, st, args.steps, peak),
             "roofline": roofline, "kernels": kernels, "gpu_launches": launches, "clocks": clocks}
     if args.only_main:
         lat.close()
