@@ -377,7 +377,8 @@ constexpr int kSMs = 152;
 // lattice; the 16-wide ones waste less on extents that are no multiple of 32, and the smallest fills the
 // chip with fewer columns (it replaced 32 x 7, 10 warps for the same 224 nodes, 18.4).  Over lattices of
 // 48 to 192 nodes a side the estimate is 7% (up to 23%) below that of 32 x 16 and 32 x 7 alone; the
-// walled 120 x 120 x 600 jet takes 507 us a step in 16 x 30 and 530 in 32 x 16.
+// walled 120 x 120 x 600 jet takes 507 us a step in 16 x 30 and 530 in 32 x 16 (estimated 404: the
+// estimate knows no side walls, whose blocks take the longer gather).
 struct TileShape {
     int tx, ty, resident;
     float plane_us, alone_us;
