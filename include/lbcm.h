@@ -319,8 +319,9 @@ LB_API lb_status lb_set_params(lb_ctx *ctx, const lb_params *params);
  * obj_args[1] and obj_args[3] unused (0); obj_args[2] = checkpoint interval k (0: k = T, every step
  *   recorded and none recomputed, where the records (72 bytes a node and step) take no more than a
  *   quarter of the free device memory, else ceil(sqrt(T))).  The context keeps the memory for later
- *   calls until it is destroyed; with k = 0 it gives back at the end of the call what exceeds twice the
- *   checkpoints and records of k = ceil(sqrt(T)).
+ *   calls until it is destroyed; with k = 0 it keeps no more than twice the checkpoints and records of
+ *   k = ceil(sqrt(T)), and what a call takes beyond that goes back to a memory pool of the context,
+ *   from which the driver serves other allocations of the process when they need it.
  * grad_out (n_grad >= LB_ADJ_NOUT doubles): [0] J, [1] dJ/du_in, [2] dJ/dsigma, [3] dJ/dnu_r,
  *   [4] dJ/dnu_b, [5 + 2(m-1)] dJ/da_m, [6 + 2(m-1)] dJ/db_m for m = 1..8.
  * On return the context holds S(T) (as after lb_step(T)).  Requires FP32 storage and

@@ -254,8 +254,8 @@ class Lattice:
         """Runs T steps and returns (J, grad): J the objective of the state T steps ahead and
         grad (float64, 20) its gradient w.r.t. GRAD_NAMES.  checkpoint = segment length
         (0: every step recorded if that fits a quarter of the free memory, else ceil(sqrt(T))).  The
-        library keeps its workspace until close(); with checkpoint 0 it gives back what exceeds twice
-        the workspace of checkpoint = ceil(sqrt(T))."""
+        library keeps its workspace until close(); with checkpoint 0 what exceeds twice the workspace
+        of checkpoint = ceil(sqrt(T)) is free for other allocations of the process between calls."""
         a = list(args)[:2] + [0.0] * (2 - len(list(args)[:2]))
         obj_args = (C.c_double * 4)(a[0], a[1], float(checkpoint), 0.0)
         out = (C.c_double * _abi.ADJ_NOUT)()

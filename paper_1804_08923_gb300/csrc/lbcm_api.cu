@@ -162,6 +162,7 @@ struct lb_ctx {
     struct {
         void *base = nullptr, *steps = nullptr;
         size_t bytes = 0;  // of steps
+        cudaMemPool_t pool = nullptr;  // records that a call takes beyond what the context keeps
         float2 *ckpt_pop = nullptr, *seg_pop = nullptr, *lr_obj = nullptr, *lgb = nullptr, *objph = nullptr,
                *phase2 = nullptr;
         float *ckpt_hist = nullptr, *seg_fm[2] = {}, *seg_hist[2] = {}, *lx = nullptr, *lh[2] = {};
@@ -769,6 +770,7 @@ void lb_destroy(lb_ctx *c) {
     }
     if (c->adj.base) cudaFree(c->adj.base);
     if (c->adj.steps) cudaFree(c->adj.steps);
+    if (c->adj.pool) cudaMemPoolDestroy(c->adj.pool);
     if (c->owns)
         for (int j = 0; j < c->nbufs; ++j)
             if (c->bufs[j]) cudaFree(c->bufs[j]);
@@ -1469,35 +1471,65 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         return fail(LB_ENOMEM, "cannot allocate the adjoint workspace (" + std::to_string(need >> 20) + " MiB)");
     };
     // k = 0: every step recorded where that takes no more than a quarter of the free device memory
-    // (what a previous call left allocated counts as free), else ceil(sqrt(T)).  The recompute that this
+    // (what previous calls left allocated counts as free), else ceil(sqrt(T)).  The recompute that this
     // saves costs as much as the forward pass; run beside the reverse sweep it hid nothing (64x64x256
-    // jet, 50 steps: 20.2 ms with it, 13.8 without).  What exceeds twice the block of the schedule with
-    // checkpoints is given back when the call ends: a context keeps what it would have kept with them
-    // but for a factor, not what happened to be free.  Allocating and freeing 38 GB (500 steps) takes 20 ms
-    // of that call's 107; with checkpoints it takes 116.
+    // jet, 50 steps: 20.2 ms with it, 13.8 without).  Records of more than twice the block of the schedule
+    // with checkpoints come from a pool of the context and go back to it when the call ends: the next
+    // call finds them there, and the driver takes them for any other allocation of the process that
+    // needs them (cudaMalloc of all but 18 GB of the device with 38 GB in the pool: no error).  500 steps,
+    // 38 GB: 86.7 ms a call, the first 121; 115 with checkpoints; 107 when the records are allocated and freed by
+    // every call.  What the context itself keeps is at most twice the block with checkpoints.
     const long long k_sqrt = std::max(1ll, std::min<long long>((long long)std::ceil(std::sqrt((double)T)), T));
     long long k = obj_args[2] < 1 ? 0 : obj_args[2] >= (double)T ? T : (long long)obj_args[2];
     const bool automatic = k == 0;
     if (!possible(automatic ? k_sqrt : k)) return no_memory((size_t)1 << 48);
-    if (automatic) {
-        size_t free_b = 0, total_b = 0;
-        LB_CUDA(cudaMemGetInfo(&free_b, &total_b));
-        k = possible(T) && layout(T, parts) <= (free_b + c->adj.bytes) / 4 && allocate(layout(T, parts)) ? T : k_sqrt;
-    }
     const size_t keep = automatic ? 2 * layout(k_sqrt, parts) : ~(size_t)0;
-    struct GiveBack {
+    struct Steps {  // at the end of the call: what is beyond keep goes back
         lb_ctx *c;
         size_t keep;
-        ~GiveBack() {
+        void *pooled = nullptr;
+        ~Steps() {
+            if (pooled) cudaFreeAsync(pooled, c->stream);
             if (c->adj.bytes <= keep) return;
             cudaFree(c->adj.steps);
             c->adj.steps = nullptr;
             c->adj.bytes = 0;
         }
-    } give_back{c, keep};
+    } steps{c, keep};
+    auto from_pool = [&](size_t need) {
+        if (!c->adj.pool) {
+            int dev = 0;
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            unsigned long long all = ~0ull;
+            if (cudaGetDevice(&dev) != cudaSuccess) return false;
+            props.location.id = dev;
+            if (cudaMemPoolCreate(&c->adj.pool, &props) != cudaSuccess ||
+                cudaMemPoolSetAttribute(c->adj.pool, cudaMemPoolAttrReleaseThreshold, &all) != cudaSuccess) {
+                cudaGetLastError();
+                return false;
+            }
+        }
+        if (cudaMallocFromPoolAsync(&steps.pooled, need, c->adj.pool, c->stream) == cudaSuccess) return true;
+        cudaGetLastError();
+        steps.pooled = nullptr;
+        return false;
+    };
+    if (automatic) {
+        size_t free_b = 0, total_b = 0;
+        unsigned long long held = 0;
+        LB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        if (c->adj.pool) LB_CUDA(cudaMemPoolGetAttribute(c->adj.pool, cudaMemPoolAttrReservedMemCurrent, &held));
+        k = k_sqrt;
+        if (possible(T)) {
+            const size_t all = layout(T, parts);
+            if (all <= (free_b + held + c->adj.bytes) / 4 && (all <= keep ? allocate(all) : from_pool(all))) k = T;
+        }
+    }
     const long long nseg = (T - 1) / k + 1;
     const size_t need = layout(k, parts);
-    if (!allocate(need)) return no_memory(need);
+    if (!steps.pooled && !allocate(need)) return no_memory(need);
     if (!c->adj.base) {
         size_t state = 0;
         for (int q = kSteps; q < kParts; ++q) state += align_up(parts[q]);
@@ -1508,7 +1540,7 @@ lb_status lb_adjoint(lb_ctx *c, int32_t objective, int64_t T, const double *obj_
         }
     }
     {
-        char *p = (char *)c->adj.steps;
+        char *p = (char *)(steps.pooled ? steps.pooled : c->adj.steps);
         void *v[kParts];
         for (int q = 0; q < kParts; ++q) {
             if (q == kSteps) p = (char *)c->adj.base;

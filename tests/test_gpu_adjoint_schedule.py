@@ -40,25 +40,35 @@ def test_an_adjoint_takes_no_profile_records(lb):
     lat.close()
 
 
-def test_the_automatic_schedule_keeps_no_more_than_twice_the_checkpoints(lb):
-    """200 steps recorded take 14.7 KB a node, with checkpoints every 15 steps 5.7; the context keeps at
-    most twice that, and what is left of the call is the same."""
+def test_the_automatic_schedule_leaves_the_memory_to_others(lb):
+    """200 steps recorded take 14.7 KB a node, with checkpoints every 15 steps 5.7.  After the call all but
+    twice the latter can be allocated again; the results are those of a schedule that is named, and the
+    next call finds its records."""
     import torch
     T, k, nseg = 200, 15, 14
     lat, ref = lattice(lb), lattice(lb)
-    J, g = ref.adjoint(T, checkpoint=T)
+    start = lat.save()
+    J, _ = ref.adjoint(T, checkpoint=T)
+    state = ref.adjoint_state(device=True).clone()
     torch.cuda.synchronize()
+    torch.cuda.empty_cache()
     before = torch.cuda.mem_get_info()[0]
-    assert lat.adjoint(T)[0] == J
-    kept = before - torch.cuda.mem_get_info()[0]
-    steps = nseg * 216 + 2 * 216 + 2 * k * 72  # bytes a node, the outflow plane's share below
-    assert kept <= 2 * lat.nodes * steps * (1 + 4.0 / GRID[2]) + lat.nodes * 200 + (64 << 20), kept / lat.nodes
-    assert torch.equal(lat.adjoint_state(device=True), ref.adjoint_state(device=True))
+    checkpoints = lat.nodes * (nseg * 216 + 2 * 216 + 2 * k * 72) * (1 + 4.0 / GRID[2])  # and the outflow plane's share
+    kept = 2 * checkpoints + lat.nodes * 200 + (256 << 20)
+    assert lat.nodes * T * 72 > kept + (1 << 30)
+    for _ in range(2):
+        lat.load(start)
+        assert lat.adjoint(T)[0] == J
+        assert torch.equal(lat.adjoint_state(device=True), state)
+        torch.cuda.empty_cache()
+        others = torch.empty(int(before - kept), dtype=torch.uint8, device="cuda")
+        del others
+        torch.cuda.empty_cache()
     # a later call that needs less gives back what it does not need
     lat.adjoint(T, checkpoint=T)
     lat.adjoint(3)
-    kept = before - torch.cuda.mem_get_info()[0]
-    assert kept <= lat.nodes * (3 * 72 * 4 + 2 * 216 * 4 + 200) + (64 << 20), kept / lat.nodes
+    torch.cuda.empty_cache()
+    assert before - torch.cuda.mem_get_info()[0] <= lat.nodes * (3 * 72 * 4 + 2 * 216 * 4 + 200) + (256 << 20)
     lat.close()
     ref.close()
 
