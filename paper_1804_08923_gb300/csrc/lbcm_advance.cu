@@ -19,10 +19,11 @@
 //            the node of plane k - 1, c_z = 0 is joined to plane k, c_z = +1 starts plane k + 1
 //            (z_class, join_classes, finish_moments; 24 registers hold the two open planes).
 // What bounds it: instruction issue and the shared-memory pipe, in turn rather than together (96 x 96 x
-// 384 jet: issue slots 71%, FMA pipe 55%, 1206 instructions a node with its share of the halo; DRAM 104
+// 384 jet: issue slots 74%, FMA pipe 58%, 1238 instructions a node with its share of the halo; DRAM 104
 // bytes a node, a third of its bandwidth), because the warps of a block go through the same phase at
-// the same time.  Tried on
-// 256 x 256 x 512, G nodes/s: 32 x 16 tile, 20 warps, a barrier after each phase 19.2; halo warps of
+// the same time.  96 registers a thread; the outflow epilogue, which one run of a column takes after its
+// march, spills 27 pairs (about 450 bytes).  256 x 256 x 512: 23.4 G nodes/s.  Tried there, before the
+// present order of the sums (22.4): 32 x 16 tile, 20 warps, a barrier after each phase 19.2; halo warps of
 // their own 20.2; gradient moved between arriving at and waiting on the first barrier, the scalar
 // part of the collision before the second 22.4; both barriers split in two halves 21.5.  Two
 // population buffers and one barrier (32 x 11, 14 warps) 16.3 when the first form had 17.2.
@@ -107,7 +108,8 @@ __device__ __forceinline__ int pmod(int a, int n) {
 
 // The run that ends at a convective top computes the outflow after its march, as long as six planes take;
 // it gets that many fewer.  By that number of planes (us a step): 64x64x256 jet 0 72.5, 2 66.3, 4 60.8, 6
-// 56.5, 8 57.2; 96x96x384 jet 180, 177, 171, 167.0, 167.4; runs shorter than 8 planes stay equal.
+// 56.5, 8 57.2; 96x96x384 jet 180, 177, 171, 167.0, 167.4 (52.7 and 159.3 now); runs shorter than 8 planes
+// stay equal.
 constexpr int kTail = 6;
 
 template <bool kForce, bool W, int TX, int TY, int MB>
@@ -377,8 +379,8 @@ constexpr int kSMs = 152;
 // lattice; the 16-wide ones waste less on extents that are no multiple of 32, and the smallest fills the
 // chip with fewer columns (it replaced 32 x 7, 10 warps for the same 224 nodes, 18.4).  Over lattices of
 // 48 to 192 nodes a side the estimate is 7% (up to 23%) below that of 32 x 16 and 32 x 7 alone; the
-// walled 120 x 120 x 600 jet takes 507 us a step in 16 x 30 and 530 in 32 x 16 (estimated 404: the
-// estimate knows no side walls, whose blocks take the longer gather).
+// walled 120 x 120 x 600 jet took 507 us a step in 16 x 30 and 530 in 32 x 16 (487 now; estimated 404:
+// the estimate knows no side walls, whose blocks take the longer gather).
 struct TileShape {
     int tx, ty, resident;
     float plane_us, alone_us;

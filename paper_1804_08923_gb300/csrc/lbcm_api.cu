@@ -1047,7 +1047,7 @@ static cudaEvent_t *profile_record(lb_ctx *c, ProfKind kind) {
 // of through the populations: the paper's rates, FP32 storage and the default step kernel, where an
 // advance is estimated faster than the two passes it replaces.  Those run at 12.7 G nodes/s on large
 // lattices and take 6 us on the smallest (two dependent launches), 3 us more where boundary planes are
-// computed first.  32^3: 8.5 us for the passes, 12 measured for an advance, whose blocks collide three
+// computed first.  32^3: 8.6 us for the passes, 12 measured for an advance, whose blocks collide three
 // planes for each that they own, and 19.6 estimated: plan_advance allows 12 us for filling and draining,
 // what lattices of a few waves take, and the line lies on the side of the passes below 72^3.
 static bool use_advance(const lb_ctx *c, const StepArgs &a, AdvancePlan *plan) {
